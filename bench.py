@@ -50,12 +50,12 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "a6fb8214b6386bfa77af795dbeec585ed5d7c2da3421f652fea7b86df8117e2c",
-        "bytes": 1102336 + 256,
+        "sha256": "68ffd2d87df72dd1ab55b2fbbb62bba1984fa39655bf48b589104d2a8c2c27e2",
+        "bytes": 1520384 + 1948416,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)
-    "k_solve2d_tc128<2>": ["rd_solve_tc2.cu", "rd_tc_ptx.cuh"],
+    "k_solve2d_tc128<2>": ["rd_solve_tc2.cu", "rd_scan.cuh", "rd_tc_ptx.cuh"],
 }
 
 
@@ -629,9 +629,12 @@ def run_gpu(args):
     if rank == 0:
         pk, pk_src = peaks()
         value = solves_all / t_all
-        flop_per_solve = 16.0 * n**3 * spec["n_steps"]  # 4 transforms x 2 N^3 x 2 fields / step
-        bytes_per_solve = 16.0 * n * n * spec["n_steps"]  # u, v FP32 read + write per step
         kind = rd.rd_get_size_kernel(p, 0)
+        # transforms x 2 N^3 x 2 fields per step: the tensor-core kernel transforms one
+        # direction and back, the CUDA-core kernel both
+        n_tr = 4 if kind == rd.RD_KERNEL_SIMT else 2
+        flop_per_solve = n_tr * 4.0 * n**3 * spec["n_steps"]
+        bytes_per_solve = 16.0 * n * n * spec["n_steps"]  # u, v FP32 read + write per step
         # the solve kernel's launch duration, taken from the timed steps: one
         # launch per step, 99.997 % of the step's device time (the ncu launch
         # list), so achieved figures are lower bounds
@@ -656,7 +659,7 @@ def run_gpu(args):
                                        "other kernels of a step take 0.003 % of it)",
                      "standalone_ms": 1e3 * k_standalone, "standalone_reps": len(kt),
                      "standalone_ms_each": [1e3 * x for x in kt],
-                     "work": "16 N^3 flop per proposal-step (4 transforms x 2 N^3 x 2 fields) "
+                     "work": f"{4 * n_tr} N^3 flop per proposal-step ({n_tr} transforms x 2 N^3 x 2 fields) "
                              f"x {spec['n_steps']} steps x {C} proposals per launch"})
         hbm = _find(pk, "hbm_gbs", "hbm_GBps", "copy_gbs") or FALLBACK_PEAKS["hbm_gbs"]
         roof["hbm_equiv"] = {"gbs": bytes_per_solve * C / k_dur / 1e9, "peak_gbs": hbm,

@@ -70,21 +70,23 @@ enum {
   RD_SOLVER_AUTO = 0,      /* autotuned per grid size (2-D), Thomas (1-D) */
   RD_SOLVER_THOMAS = 1,    /* 1-D tridiagonal (FP64) */
   RD_SOLVER_DCT_SIMT = 2,  /* 2-D eigenbasis solve, FP32 CUDA-core GEMMs */
-  RD_SOLVER_DCT_TC = 3     /* 2-D eigenbasis solve, split-FP16 tcgen05 GEMMs */
+  RD_SOLVER_DCT_TC = 3     /* 2-D eigenbasis solve of one direction by split-FP16
+                              tcgen05 GEMMs, tridiagonal solves of the other */
 };
 
 /* Solve kernel of one 2-D grid size (rd_set_size_kernel, rd_autotune).  All
- * compute the same IMEX step; they differ in how the eigenbasis transforms of
- * the implicit solve run on the GPU. */
+ * compute the same IMEX step; they differ in how the implicit solve runs on
+ * the GPU. */
 enum {
   RD_KERNEL_DEFAULT = 0,     /* from desc.solver: SIMT for RD_SOLVER_DCT_SIMT;
                                 otherwise TC_RESIDENT at N = 128, else
                                 TC_STACKED */
   RD_KERNEL_SIMT = 1,        /* FP32 CUDA-core GEMMs, one proposal per CTA */
-  RD_KERNEL_TC_STACKED = 2,  /* split-FP16 tcgen05, DCT matrix in shared memory,
-                                floor(128/N) proposals stacked per MMA tile */
-  RD_KERNEL_TC_RESIDENT = 3, /* split-FP16 tcgen05, DCT matrices resident in
-                                tensor memory; N = 128 only */
+  RD_KERNEL_TC_STACKED = 2,  /* split-FP16 tcgen05 transforms of one direction,
+                                tridiagonal solves of the other; as many proposals
+                                per CTA as fit its accumulators */
+  RD_KERNEL_TC_RESIDENT = 3, /* the same kernel, N = 128 only (one proposal per
+                                CTA); kept as a choice of its own */
   RD_KERNEL_CG = 4           /* each implicit system by plain conjugate gradients
                                 (the paper's linear solver, Sec. 3.1.1) from the
                                 previous step, FP32 on CUDA cores, vectors in

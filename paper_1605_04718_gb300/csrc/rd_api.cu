@@ -68,8 +68,8 @@ int kernel_for_size(const rd_problem* p, int s) {
 // Persistent CTAs of a kernel kind's launch when every SM holds as many as fit.
 static int grid_max_of(const rd_problem* p, int kind) {
   switch (kind) {
-    case RD_KERNEL_TC_RESIDENT: return grid_solve_tc128(p->n_sm);
-    case RD_KERNEL_TC_STACKED: return grid_solve_tc(p->dev.max_n, p->n_sm);
+    case RD_KERNEL_TC_RESIDENT:
+    case RD_KERNEL_TC_STACKED: return grid_solve_tc(p->n_sm);
     case RD_KERNEL_CG: return grid_solve_cg(p->dev.max_n, false, p->n_sm);
     default: return grid_solve_simt(p->desc.dim, p->dev.max_n, p->n_sm);
   }
@@ -85,26 +85,31 @@ cudaError_t launch_solve_queue(rd_problem* p, const WorkQueue& q, const double* 
   if (p->desc.dim == 2 && p->dev.scheme == RD_SCHEME_PICARD)  // every size: one launch
     return launch_solve_cg(p->dev, q, theta, phi, status, fields, true,
                            grid_solve_cg(p->dev.max_n, true, p->n_sm), st);
-  static const int kinds[4] = {RD_KERNEL_TC_RESIDENT, RD_KERNEL_TC_STACKED, RD_KERNEL_SIMT,
-                               RD_KERNEL_CG};
-  for (int kind : kinds) {
-    WorkQueue sub = q;  // the sizes of this kernel, largest grid first
+  // one launch per kernel kind in use; the tensor-core kinds run the same
+  // kernel, one launch per grid size N
+  auto launch_key = [&](int s) {
+    const int k = kernel_for_size(p, s);
+    return k == RD_KERNEL_TC_STACKED || k == RD_KERNEL_TC_RESIDENT ? 1000 + p->desc.nx[s] : k;
+  };
+  bool done[kMaxSizes] = {};
+  for (int k0 = 0; k0 < q.n_sizes; ++k0) {
+    if (done[k0]) continue;
+    const int key = launch_key(q.order[k0]);
+    WorkQueue sub = q;  // the sizes of this launch, largest grid first
     sub.n_sizes = 0;
     int want = 0;  // CTAs per SM: the largest any of these sizes asks for
-    for (int k = 0; k < q.n_sizes; ++k)
-      if (kernel_for_size(p, q.order[k]) == kind) {
+    for (int k = k0; k < q.n_sizes; ++k)
+      if (launch_key(q.order[k]) == key) {
+        done[k] = true;
         sub.order[sub.n_sizes++] = q.order[k];
         want = std::max(want, p->ctas_per_sm[q.order[k]]);
       }
-    if (sub.n_sizes == 0) continue;
-    const int gmax = grid_max_of(p, kind);
+    const int gmax = grid_max_of(p, kernel_for_size(p, q.order[k0]));
     const int grid = (want > 0 && want * p->n_sm < gmax) ? want * p->n_sm : gmax;
     cudaError_t e;
-    if (kind == RD_KERNEL_TC_RESIDENT)
-      e = launch_solve_tc128(p->dev, sub, theta, phi, status, fields, grid, p->ws.err, st);
-    else if (kind == RD_KERNEL_TC_STACKED)
+    if (key >= 1000)
       e = launch_solve_tc(p->dev, sub, theta, phi, status, fields, grid, p->ws.err, st);
-    else if (kind == RD_KERNEL_CG)
+    else if (key == RD_KERNEL_CG)
       e = launch_solve_cg(p->dev, sub, theta, phi, status, fields, false, grid, st);
     else
       e = launch_solve_simt(p->dev, sub, theta, phi, status, fields, grid, st);
@@ -281,13 +286,13 @@ rd_status rd_problem_create(const rd_problem_desc* desc, void* cuda_stream,
     rd_problem_destroy(p);
     return RD_ENOMEM;
   }
-  bool has128 = false;
-  for (int k = 0; k < desc->n_sizes; ++k) has128 = has128 || (desc->dim == 2 && desc->nx[k] == 128);
+  bool tc_ok = true;
+  for (int k = 0; k < desc->n_sizes; ++k)
+    tc_ok = tc_ok && (desc->dim != 2 || setup_solve_tc(desc->nx[k]) == cudaSuccess);
   if (setup_solve_simt(desc->dim, dv.max_n) != cudaSuccess ||
-      (desc->dim == 2 && setup_solve_tc(dv.max_n) != cudaSuccess) ||
       (desc->dim == 2 && cg_applicable(dv.max_n, false) &&
        setup_solve_cg(dv.max_n, false) != cudaSuccess) ||
-      (has128 && setup_solve_tc128() != cudaSuccess)) {
+      !tc_ok) {
     rd_problem_destroy(p);
     set_error("cannot configure the solve kernels' shared memory");
     return RD_ECUDA;

@@ -105,20 +105,13 @@ cudaError_t launch_solve_simt(const DevProblem& pb, const WorkQueue& q,
                               void* fields, int grid, cudaStream_t st,
                               int* steps_out = nullptr);
 cudaError_t setup_solve_simt(int dim, int max_n, bool steady = false);
-cudaError_t setup_solve_tc(int max_n);
-int grid_solve_tc(int max_n, int n_sm);
+// Tensor-core solve (rd_solve_tc2.cu): every size in its queue must be the same
+// N x N grid, N a multiple of 16 up to 128.
+cudaError_t setup_solve_tc(int n);
+int grid_solve_tc(int n_sm);
 cudaError_t launch_solve_tc(const DevProblem& pb, const WorkQueue& q, const double* theta,
                             double* phi, uint32_t* status, void* fields, int grid, int* err,
                             cudaStream_t st);
-size_t tc_smem_bytes_host(int max_n);
-// 128^2-only tensor-core solve with the DCT matrices resident in TMEM
-// (rd_solve_tc2.cu): every size in its queue must be a 2-D 128^2 grid.
-bool tc128_applicable(const DevProblem& pb, int size_idx);
-cudaError_t setup_solve_tc128();
-int grid_solve_tc128(int n_sm);
-cudaError_t launch_solve_tc128(const DevProblem& pb, const WorkQueue& q, const double* theta,
-                               double* phi, uint32_t* status, void* fields, int grid, int* err,
-                               cudaStream_t st);
 // CUDA-core conjugate-gradient solves (rd_solve_simt.cu): the IMEX step by
 // plain CG (RD_KERNEL_CG, N <= 96) or the paper's semi-implicit step by
 // preconditioned CG (picard, N <= 80).

@@ -1,72 +1,68 @@
-// rd_solve_tc2.cu -- the 128^2 forward solve on the tensor cores with the
-// DCT matrices resident in TMEM.
+// rd_solve_tc2.cu -- 2-D forward solves on the tensor cores, N = 16..128.
 //
-// Same step and number format as k_solve2d_tc (rd_solve_tc.cu): explicit
-// reaction, implicit diffusion by the four eigenbasis transforms (Sec. 3.1.1
-// with the diagonal solve in the DCT-II basis), split-FP16 operands with
-// three products, FP32 accumulation, state held as deviation from the
-// initial-state mean.  The difference is the orientation: the constant
-// matrix 8C (and its transpose) is operand A, read from TMEM, and each
-// field's data is operand B in shared memory, so an MMA reads 4 KB of
-// operands from shared memory instead of 8 KB.  With i the index on TMEM
-// lanes and j the one on columns:
-//   stage 1  D[k][i] = sum_j C[k][j] R[i][j]        (B = R, K-major)
-//   stage 2  D[l][k] = sum_i C[l][i] P[k][i]        (B = P, K-major)
-//   scale    S[l][k] = D[l][k] L[l][k]
-//   stage 3  D[i][k] = sum_l C^T[i][l] S[l][k]      (B = S, MN-major)
-//   stage 4  D[j][i] = sum_k C^T[j][k] E[i][k]      (B = E, K-major)
-// so one step maps a state with i on the lanes to one with j on the lanes:
-// the state is W (y on the lanes) after an even number of steps and W^T
-// after an odd number.  L is symmetric, so the same code serves both.
+// The IMEX step of Sec. 3.1.1 (reaction explicit, diffusion and dilution
+// implicit) with fields held as deviations from the initial-state mean.  The
+// implicit solve [alpha I - beta Lap_h] w = r takes the cosine basis (DCT-II
+// matrix C) in one direction only and solves the tridiagonal systems that are
+// left along the other (rd_scan.cuh):
+//   stage 1  D[k][i] = sum_j C[k][j] R[i][j]     (tensor cores)
+//   scan     X[k][.] = [(alpha + beta mu_k) I - beta Lap_1D]^-1 D[k][.]
+//   stage 2  W[j][i] = sum_k C[k][j] X[k][i]     (tensor cores)
+// against four transforms when both directions are diagonalised: half the
+// tensor-core work, two conversions of the data per step instead of four, and
+// no 1 / (alpha + beta (mu_k + mu_l)) per point.  The scan is FP32 throughout.
+// Measured against the four-transform kernels (GB300): 128^2 9.98 -> 6.33 us a
+// step of one proposal per SM; 64^2 18.7 -> 4.9 us for the four proposals an SM
+// holds; relative field error after 1000 steps at 128^2 2.2e-7 -> 1.9e-7.
 //
-// Pipelining.  The fields u and v run interleaved: while the tensor core
-// works on one field's stage, the other field's converter warps turn the
-// previous result into the next operand.  (Splitting a stage into two N = 64
-// halves, to start on half an operand, cost more than it overlapped: an
-// N = 64 MMA takes about 56 cycles against 64 for N = 128.)
+// Layout.  A slab is one accumulator of 128 TMEM lanes x 128 columns; a CTA has
+// two.  The constant matrices are operand A, read from TMEM, the data operand B
+// in shared memory (FP16 hi and lo parts).
+//   N > 64:  slab 0 is field u, slab 1 field v of one proposal.
+//   N <= 64: a slab holds floor(128 / N)^2 blocks of N x N: proposals along the
+//   lanes (A is block-diagonal) and u | v of more proposals along the columns;
+//   the two slabs are independent of each other.  64^2: 2 proposals per slab,
+//   32^2: 8, 16^2: 32.  Blocks that a small batch leaves empty cost no K blocks
+//   and no columns.
+// A step maps a state with y on the lanes to one with x on the lanes, so the
+// orientation alternates; the operator is symmetric in x and y.
 //
-// The diagonal factor L = 1 / (alpha + beta (mu_l + mu_k)) (times 1/64 and
-// the compensation below) is computed where it is applied: the reciprocal by
-// the hardware approximation (within one ulp), on pairs of columns with the
-// paired FP32 instructions.  On a fixed domain L is the same every step, so
-// its rounding error compounds in the slow modes: a cheaper reciprocal (one
-// approximation for two values through their product) moved Phi by more
-// than the posterior allows.  The converter warps are bound by throughput
-// (their instructions, TMEM loads and shared-memory stores beside the MMAs'
-// operand reads: twice the warps did not convert faster), and the tensor
-// core waits on them, so the hot loops save instructions: the hi/lo
-// split works on pairs with the paired FP32 instructions and stores the lo
-// part negated (one mixed FP16/FP32 subtraction per value; the MMAs that
-// read it set the negate bit of B), the operand scale 256 of the reaction
-// is applied through its constants, and stage 3's compensation is folded
-// into L.
+// Warps 0-15 convert (TMEM -> registers -> reaction or scan -> split ->
+// shared memory), warp 16 issues every MMA from one thread, warp 17 forms the
+// growing domain's factors in FP64 one step ahead.  N > 64: the u and v halves
+// of the converters scan their slabs side by side (scanning u with all 16
+// warps and then v measured 7.05 us a step against 6.85: v's operand then
+// comes late for stage 2).  N <= 64: all 16 warps take slab 0 and then slab 1,
+// so each slab's MMAs run under the other's conversions (5.1 us a step against
+// 5.46 with eight warps per slab).  The converters bound the kernel: about 20
+// instructions per point for the reaction and 9 per value for the scan, on an
+// FP32 pipe that takes 1.5 cycles per FMA with three register operands, with
+// the tensor pipe 45 % busy.  The issuing loops are unrolled at compile time:
+// forming descriptors at run time cost 100 to 150 cycles an MMA against 64.
 //
-// Accumulation order.  The tensor core rounds each MMA's sum toward zero, a
-// bias of about 0.72 * 2^-24 of the accumulator per MMA that compounds over
-// the chain.  Each stage therefore issues the small correction products
-// (hi*lo, lo*hi) first, while the accumulator is small, and the 8 main
-// products (hi*hi) last; the remaining shrink of about 8 * 0.5 * 2^-24 (the
-// partial sums average about 0.7 of the final value) is compensated by
-// multiplying each stage's output by 1 + 2^-22.
+// Precision: every FP32 operand x is split into FP16 hi + lo and each product
+// formed as hi*hi + hi*lo + lo*hi, about 22 significant bits.  The tensor core
+// rounds each MMA's sum toward zero; each stage issues the small correction
+// products first and its output is scaled by 1 + N 2^-29, the mean shrink that
+// the N / 16 main products leave.  The data's lo part is stored negated (one
+// instruction less per pair) and the MMAs that read it set the negate bit.
+// Power-of-two scales keep operands inside the FP16 range:
+//   R' = 256 r, C' = 8 C -> D' = 2048 D; X' = 16 x; W' = 128 w.
 //
-// TMEM (512 columns): 8C hi | 8C lo | 8C^T hi | 8C^T lo (64 columns each,
-// two FP16 per column) | field u accumulator | field v accumulator.
-// One 128^2 proposal per CTA, 544 threads: warps 0-7 convert field u,
-// 8-15 field v (two warps per TMEM lane quadrant), warp 16 allocates TMEM
-// and issues the MMAs, one thread, in the order u1 v1 u2 v2 ... u4 v4 (two
-// issuing threads let both fields' MMAs share the tensor core at once: they
-// then finish together and convert together, with nothing to overlap).  As
-// the MMAs complete in that order, a converter starts the reaction once it
-// has seen the stage-4 commit of both fields.  Barrier arrivals are one per
-// warp.  Shared memory: the four operand tiles (u hi, u lo, v hi, v lo;
-// 32 KB each) and control.
-// Bounded waits as in rd_solve_tc.cu.
+// N <= 64: the block-diagonal A multiplies other proposals' data by zero, so a
+// reaction value outside the FP16 range (a diverging solve) must not reach the
+// MMA as infinity: it is stored as zero and every later observation or output
+// of its proposal reads NaN, which is what an infinite operand leads to.
+//
+// Every wait is bounded; a timed-out wait makes the CTA leave, drain its MMAs,
+// free its TMEM and raise the error flag.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
 #include "rd_common.cuh"
 #include "rd_internal.h"
+#include "rd_scan.cuh"
 #include "rd_tc_ptx.cuh"
 
 namespace rd {
@@ -75,37 +71,77 @@ using namespace tc;
 
 namespace tc2 {
 
-constexpr int N = 128;
-constexpr uint32_t kColCHi = 0, kColCLo = 64, kColCtHi = 128, kColCtLo = 192;
-constexpr uint32_t kColAcc = 256;  // + 128 f
+constexpr int kMaxItems = 64;  // proposals per CTA (N = 16)
+constexpr uint32_t kColA = 0;  // 8C hi | 8C lo | 8C^T hi | 8C^T lo, 64 columns each
+constexpr uint32_t kColAcc = 256;  // + 128 g
 constexpr uint32_t kTileBytes = 128 * 128 * 2;  // one FP16 operand tile
-constexpr uint32_t kOffCtrl = 4 * kTileBytes;  // after the tiles u hi, u lo, v hi, v lo
-constexpr uint32_t kSmemBytes = 1024 + kOffCtrl + 4096;
-// stage output scales with the round-toward-zero compensation 1 + 2^-22
-constexpr float kScale1 = 0x1p-7f + 0x1p-29f;   // stage 1: (1/128)(1 + 2^-22)
-// stage 2: L (1/64)(1 + 2^-22)^2, the compensation of stage 3 included
-// (the transforms are linear), so that stage 3's output is split unscaled
-constexpr float kScaleL = 0x1p-6f + 0x1p-27f;
-constexpr float kScaleW = 0x1p-7f + 0x1p-29f;   // stage 4 (state read): (1/128)(1 + 2^-22)
+constexpr uint32_t kOffCtrl = 4 * kTileBytes;   // after slab 0 hi, lo, slab 1 hi, lo
+constexpr int kConvWarps = 16;
+constexpr int kIssueWarp = 16;  // 17: growth factors
+constexpr int kThreads = 32 * 18;
 
-struct Ctrl {
-  uint64_t mma_done[2];   // per field: its stage's MMAs completed
-  uint64_t op_all[2];     // per field: the whole next operand written
-  uint64_t rx_ready;      // reaction written (both fields)
-  uint64_t fin;
-  uint64_t never;         // completed by nothing (failure-path test aid)
-  double phi;
-  uint32_t tmem_base;
-  int abort;
-  int item;
-  int size;
-  int bad;
-  double th[kNPhys];
-  alignas(16) float mu[N];
+// How proposals of an N x N grid fill a slab (128 lanes x 128 columns).
+template <int N>
+struct Geo {
+  static constexpr bool kPair = N > 64;            // slab 0 = u, slab 1 = v of one proposal
+  static constexpr int LB = kPair ? 1 : 128 / N;   // blocks along the lanes
+  static constexpr int S = N * LB;                 // slab edge
+  static constexpr int QB = kPair ? 1 : LB / 2;    // (u, v) block pairs along the columns
+  static constexpr int kCap = kPair ? 1 : 2 * LB * QB;  // proposals per CTA
+  static constexpr int NB = N == 16 ? 2 : 1;       // scan blocks per thread and slab
+  static constexpr int kOpWarps = kPair ? 8 : 16;  // warps that scan one slab
 };
 
-__device__ __forceinline__ uint8_t* tile(uint8_t* base, int f, int hl) {
-  return base + (uint32_t)(2 * f + hl) * kTileBytes;
+struct alignas(16) React {  // one proposal's step constants
+  float fa, fb, ftg, alpha, cu, cv;
+};
+
+struct Ctrl {
+  uint64_t mma_done[2];    // per slab: a stage's MMAs completed (two phases per step)
+  uint64_t op_ready[2];    // per slab: scanned operand written
+  uint64_t rx[2];          // N > 64: first / second half of both slabs' reaction written;
+                           // N <= 64: slab 0 / 1's reaction written (16 warps)
+  uint64_t seg[2][4][2];   // N >= 48: the sums of (slab, quadrant, block) written (2 warps)
+  uint64_t grow;           // growing domain: this step's beta written
+  uint64_t fin;
+  uint64_t never;          // completed by nothing (failure-path test aid)
+  uint32_t tmem_base;
+  int abort;
+  int n_items;
+  int size;
+  int slow;               // an irregular proposal, alone in the CTA
+  int n_chunk, next;      // popped items, of which already run
+  int chunk[kMaxItems];
+  int items[kMaxItems];
+  int bad[kMaxItems];
+  int blown[kMaxItems];   // N <= 64: a reaction value left the FP16 range
+  double phi[kMaxItems];
+  double th[kMaxItems][kNPhys];
+  float beta[2][kMaxItems][2];  // growing domain: per step parity, item, field
+  React rk[kMaxItems];
+  alignas(16) float mu[128];
+  float2 sums[2][4][128];       // (L, R) per slab, block and segment, lane
+};
+constexpr uint32_t kSmemBytes = 1024 + kOffCtrl + (uint32_t)((sizeof(Ctrl) + 127) / 128 * 128);
+
+// Parities of the barriers' phases at the start of an item: those of the step's
+// first slab (each completes once a step), and slab 1's (not in use in every item).
+struct Parity {
+  uint32_t p0 = 0, p1 = 0, seg = 0;
+};
+
+// The 1024-byte aligned start of shared memory, derived from the shared symbol
+// so that the compiler keeps the address space (plain shared accesses).
+__device__ __forceinline__ uint8_t* shared_base() {
+  extern __shared__ uint8_t smem_raw[];
+  return smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+}
+__device__ __forceinline__ Ctrl* shared_ctl() {
+  return reinterpret_cast<Ctrl*>(shared_base() + kOffCtrl);
+}
+
+__device__ __forceinline__ uint8_t* tile(uint8_t* base, int g, int hl) {
+  return base + (uint32_t)(2 * g + hl) * kTileBytes;
 }
 
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
@@ -117,83 +153,79 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bde
       : "memory");
 }
 
-// K-major stage (1, 2, 4) of field f: the correction products of all K
-// blocks first, then the main products.
-__device__ __forceinline__ void issue_kmajor(uint8_t* base, uint32_t tmem, int stage, int f) {
-  constexpr uint32_t idesc = idesc_f16_f32(128, N, 0, 0);
-  constexpr uint32_t idesc_nb = idesc_f16_f32(128, N, 0, 0, 1);  // B = the negated lo
-  const uint32_t a_hi = tmem + (stage <= 2 ? kColCHi : kColCtHi);
-  const uint32_t a_lo = tmem + (stage <= 2 ? kColCLo : kColCtLo);
-  const uint64_t bh = sdesc_sw128(smem_u32(tile(base, f, 0)), 16u, 1024u);
-  const uint64_t bl = sdesc_sw128(smem_u32(tile(base, f, 1)), 16u, 1024u);
-  const uint32_t d = tmem + kColAcc + (uint32_t)(128 * f);
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const uint64_t off = ((uint32_t)(kk >> 2) * 16384u + (uint32_t)(kk & 3) * 32u) >> 4;
-    mma_ts(d, a_hi + (uint32_t)(kk * 8), bl + off, idesc_nb, kk > 0 ? 1u : 0u);
-    mma_ts(d, a_lo + (uint32_t)(kk * 8), bh + off, idesc, 1u);
-  }
-#pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const uint64_t off = ((uint32_t)(kk >> 2) * 16384u + (uint32_t)(kk & 3) * 32u) >> 4;
-    mma_ts(d, a_hi + (uint32_t)(kk * 8), bh + off, idesc, 1u);
-  }
+// Byte offset (in 16-byte units) of K block kk of an operand tile with `rows`
+// rows: K-major (stage 1) or MN-major (stage 2).
+__device__ __forceinline__ constexpr uint32_t kblock_off(int stage, int rows, int kk) {
+  return (stage == 1 ? (uint32_t)(kk >> 2) * (uint32_t)rows * 128u + (uint32_t)(kk & 3) * 32u
+                     : (uint32_t)kk * 2048u) >> 4;
 }
 
-// Stage 3 of field f: B = the MN-major operand tile (K rows = lanes of the
-// conversion, two 64-column N blocks 16 KB apart), corrections first.
-__device__ __forceinline__ void issue_stage3(uint8_t* base, uint32_t tmem, int f) {
-  constexpr uint32_t idesc = idesc_f16_f32(128, N, 0, 1);
-  constexpr uint32_t idesc_nb = idesc_f16_f32(128, N, 0, 1, 1);  // B = the negated lo
-  const uint32_t a_hi = tmem + kColCtHi, a_lo = tmem + kColCtLo;
-  const uint64_t bh = sdesc_sw128(smem_u32(tile(base, f, 0)), 16384u, 1024u);
-  const uint64_t bl = sdesc_sw128(smem_u32(tile(base, f, 1)), 16384u, 1024u);
-  const uint32_t d = tmem + kColAcc + (uint32_t)(128 * f);
+// K blocks [K0, K1) of one stage of slab g: the correction products (lo
+// operand parts), the main products, or both.  kb < K1 skips the blocks from kb.
+template <int STAGE, int ROWS, bool CORR, bool MAIN, int K0, int K1, bool FIRST>
+__device__ __forceinline__ void issue_blocks(uint32_t sbase, uint32_t tmem, int g, int ncols,
+                                             int kb) {
+  constexpr int b_mn = STAGE == 2;
+  const uint32_t idesc = idesc_f16_f32(128, ncols, 0, b_mn);
+  const uint32_t idesc_nb = idesc_f16_f32(128, ncols, 0, b_mn, 1);  // B = the negated lo
+  const uint32_t a_hi = tmem + kColA + (STAGE == 1 ? 0u : 128u), a_lo = a_hi + 64u;
+  constexpr uint32_t lbo = STAGE == 1 ? 16u : (uint32_t)ROWS * 128u;
+  const uint64_t bh = sdesc_sw128(sbase + (uint32_t)(2 * g) * kTileBytes, lbo, 1024u);
+  const uint64_t bl = sdesc_sw128(sbase + (uint32_t)(2 * g + 1) * kTileBytes, lbo, 1024u);
+  const uint32_t d = tmem + kColAcc + (uint32_t)(128 * g);
+  if (CORR) {
 #pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const uint64_t off = ((uint32_t)kk * 2048u) >> 4;
-    mma_ts(d, a_hi + (uint32_t)(kk * 8), bl + off, idesc_nb, kk > 0 ? 1u : 0u);
-    mma_ts(d, a_lo + (uint32_t)(kk * 8), bh + off, idesc, 1u);
+    for (int kk = K0; kk < K1; ++kk) {
+      if (kk >= kb) break;
+      const uint32_t off = kblock_off(STAGE, ROWS, kk);
+      mma_ts(d, a_hi + (uint32_t)(kk * 8), bl + off, idesc_nb, (kk > K0 || !FIRST) ? 1u : 0u);
+      mma_ts(d, a_lo + (uint32_t)(kk * 8), bh + off, idesc, 1u);
+    }
   }
+  if (MAIN) {
 #pragma unroll
-  for (int kk = 0; kk < 8; ++kk) {
-    const uint64_t off = ((uint32_t)kk * 2048u) >> 4;
-    mma_ts(d, a_hi + (uint32_t)(kk * 8), bh + off, idesc, 1u);
+    for (int kk = K0; kk < K1; ++kk) {
+      if (kk >= kb) break;
+      mma_ts(d, a_hi + (uint32_t)(kk * 8), bh + kblock_off(STAGE, ROWS, kk), idesc, 1u);
+    }
   }
 }
 
 // Splits 8 values (times scale) of row r, columns c..c+7 into the hi and
 // negated lo tiles: one 16-byte store each.
-__device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, int r, int c, const float* x,
-                                       float scale) {
+__device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, int rows, int r, int c,
+                                       const float* x, float scale) {
   uint32_t h[4], l[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) split_f16x2_neglo_scaled(x[2 * j], x[2 * j + 1], scale, h[j], l[j]);
-  const uint32_t off = sw128_offset(128, r, c);
+  const uint32_t off = sw128_offset(rows, r, c);
   *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// As store8 without a scale.
-__device__ __forceinline__ void store8n(uint8_t* hi, uint8_t* lo, int r, int c, const float* x) {
+// As store8 without a scale.  GUARD: a value outside the FP16 range (or NaN)
+// makes the 8 values zero and returns true, so that it cannot reach the
+// proposals that share the MMA's K extent through 0 * inf.
+template <bool GUARD>
+__device__ __forceinline__ bool store8n(uint8_t* hi, uint8_t* lo, int rows, int r, int c,
+                                        const float* x) {
   uint32_t h[4], l[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) split_f16x2_neglo(x[2 * j], x[2 * j + 1], h[j], l[j]);
-  const uint32_t off = sw128_offset(128, r, c);
-  *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
-}
-
-// As store8 with one scale per value.
-__device__ __forceinline__ void store8s(uint8_t* hi, uint8_t* lo, int r, int c, const float* x,
-                                        const float* s8) {
-  uint32_t h[4], l[4];
+  bool out = false;
+  if (GUARD) {
+    uint32_t e = 0;  // bit 15 or 31 set where an exponent field is all ones
 #pragma unroll
-  for (int j = 0; j < 4; ++j)
-    split_f16x2_neglo_scaled2(x[2 * j], x[2 * j + 1], s8[2 * j], s8[2 * j + 1], h[j], l[j]);
-  const uint32_t off = sw128_offset(128, r, c);
+    for (int j = 0; j < 4; ++j) e |= (h[j] & 0x7C007C00u) + 0x04000400u;
+    out = (e & 0x80008000u) != 0u;
+    if (out)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) h[j] = l[j] = 0u;
+  }
+  const uint32_t off = sw128_offset(rows, r, c);
   *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+  return out;
 }
 
 // Explicit reaction in place on 8 points: state (x 128) ->
@@ -201,360 +233,704 @@ __device__ __forceinline__ void store8s(uint8_t* hi, uint8_t* lo, int r, int c, 
 // (+ cv), as deviations from the reference state, times 256 (the operand
 // scale, applied through the constants: exact).
 __device__ __forceinline__ void react8(float* u, float* v, float sw, float ref_u, float ref_v,
-                                       float fa, float fb, float ftg, float cu, float cv) {
-  const float sw8 = 256.f * sw, ftg8 = 256.f * ftg, cu8 = 256.f * cu, cv8 = 256.f * cv;
+                                       const React& k) {
+  const float sw8 = 256.f * sw, ftg8 = 256.f * k.ftg, cu8 = 256.f * k.cu, cv8 = 256.f * k.cv;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const float uu = fmaf(u[j], sw, ref_u), vv = fmaf(v[j], sw, ref_v);
     const float u2v = uu * uu * vv;
-    u[j] = fmaf(ftg8, fa - uu + u2v, fmaf(u[j], sw8, cu8));
-    v[j] = fmaf(ftg8, fb - u2v, fmaf(v[j], sw8, cv8));
+    u[j] = fmaf(ftg8, k.fa - uu + u2v, fmaf(u[j], sw8, cu8));
+    v[j] = fmaf(ftg8, k.fb - u2v, fmaf(v[j], sw8, cv8));
   }
 }
 
-struct ObsCtx {
-  const float* yo;  // this observation's data, or null
-  float* fo;        // this proposal's output fields, or null
-  bool odd;         // state transposed (x on the lanes)
-};
-
-// Observation misfit and final-field output of 8 points of row l, columns c..c+7.
-__device__ __forceinline__ void observe8(const DevProblem& pb, const DevSize& S, const ObsCtx& o,
-                                         int l, int c, const float* u, const float* v, float sw,
-                                         double& phi, int& bad) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const size_t pt = o.odd ? (size_t)(c + j) * N + l : (size_t)l * N + c + j;  // y N + x
-    const float du = u[j] * sw, dv = v[j] * sw;
-    if (o.yo) {
-      int k = 0;
-      if (S.field_mask & 1) {
-        const double w = (double)S.ref_u + (double)du;
-        if (!(fabs(w) <= pb.w_max)) bad = 1;
-        const double e = (double)o.yo[pt] - w;
-        phi += e * e;
-        ++k;
-      }
-      if (S.field_mask & 2) {
-        const double w = (double)S.ref_v + (double)dv;
-        if (!(fabs(w) <= pb.w_max)) bad = 1;
-        const double e = (double)o.yo[(size_t)k * S.npts + pt] - w;
-        phi += e * e;
-      }
-    }
-    if (o.fo) {
-      o.fo[pt] = S.ref_u + du;
-      o.fo[(size_t)S.npts + pt] = S.ref_v + dv;
-    }
-  }
-}
-
-// One converter warp w (0 .. 8 WPF - 1), WPF warps per TMEM lane quadrant
-// and field.  Stage conversions: field f = w / (4 WPF), columns
-// [cw r, cw (r + 1)) of each half, cw = 64 / WPF, r = (w / 4) % WPF.
-// Reaction: both fields at columns [xw p, xw (p + 1)) of each half,
-// xw = 32 / WPF, p = w / 4.
-template <int WPF>
-__device__ bool converter(const DevProblem& pb, const DevSize& S, Ctrl* ctl, uint8_t* base,
-                          uint32_t tmem, int warp, int lane, uint32_t& ph_done,
-                          float* fields, size_t field_stride) {
-  constexpr int CW = 64 / WPF;  // stage-conversion columns per half
-  constexpr int XW = 32 / WPF;  // reaction columns per half
-  volatile int* abort = &ctl->abort;
-  const int f = warp / (4 * WPF);
-  const int q = warp & 3;
-  const int rr = (warp >> 2) % WPF;
-  const int p = warp >> 2;
-  const int l = 32 * q + lane;
-  const uint32_t lane_off = (uint32_t)(32 * q) << 16;
-  const uint32_t t_u = tmem + lane_off + kColAcc, t_v = t_u + 128u;
-  const uint32_t t_f = f ? t_v : t_u;
-  uint8_t* const hi_u = tile(base, 0, 0);
-  uint8_t* const lo_u = tile(base, 0, 1);
-  uint8_t* const hi_v = tile(base, 1, 0);
-  uint8_t* const lo_v = tile(base, 1, 1);
-  uint8_t* const hi_f = f ? hi_v : hi_u;
-  uint8_t* const lo_f = f ? lo_v : lo_u;
-  const double* th = ctl->th;
-  const double tau = pb.tau;
-  const float fa = (float)th[0], fb = (float)th[1], ftg = (float)(tau * th[3]);
-  const double r = th[4];
-  const float beta_fixed = (float)(tau * (f ? th[2] : 1.0) * (double)N * N);
-  const float ref_u = S.ref_u, ref_v = S.ref_v;
+// Observation misfit and final-field output of this thread's points of one
+// slab pair: column indices c0 + 8 step_c j, j < n8, of lane index idx, u at
+// TMEM columns t_u + c, v at t_v + c.  sl: the proposal's slot, -1 for idle rows.
+__device__ __noinline__ void observe(const DevProblem& pb, int size, int sl, int idx, int c0,
+                                     int step_c, int n8, uint32_t t_u, uint32_t t_v, float sw,
+                                     int step, int obs, float* fields, size_t field_stride) {
+  Ctrl* ctl = shared_ctl();
+  const DevSize& S = pb.sz[size];
+  const int n = S.n;
+  const bool odd = step & 1;
+  const bool out = step == pb.n_steps && fields && sl >= 0;
   const int nfo = (S.field_mask & 1) + ((S.field_mask >> 1) & 1);
-  const float mu_l = ctl->mu[l];
+  const float* yo = obs >= 0 ? S.yf + (size_t)obs * nfo * S.npts : nullptr;
+  float* fo = out ? fields + (size_t)ctl->items[sl] * field_stride : nullptr;
+  const bool blown = sl >= 0 && ctl->blown[sl];
+  if (blown) sw = __int_as_float(0x7fffffff);  // NaN, as the solve would have reached
   double phi = 0.0;
   int bad = 0;
+  for (int k = 0; k < n8; ++k) {
+    const int c = c0 + 8 * step_c * k;
+    float u[8], v[8];
+    __syncwarp();
+    tmem_ld8(t_u + (uint32_t)c, u);
+    tmem_ld8(t_v + (uint32_t)c, v);
+    tmem_wait_ld();
+    if (sl < 0) continue;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const size_t pt = odd ? (size_t)(c + j) * n + idx : (size_t)idx * n + c + j;  // y n + x
+      const float du = u[j] * sw, dv = v[j] * sw;
+      if (yo) {
+        int kf = 0;
+        if (S.field_mask & 1) {
+          const double w = (double)S.ref_u + (double)du;
+          if (!(fabs(w) <= pb.w_max)) bad = 1;
+          const double e = (double)yo[pt] - w;
+          phi += e * e;
+          ++kf;
+        }
+        if (S.field_mask & 2) {
+          const double w = (double)S.ref_v + (double)dv;
+          if (!(fabs(w) <= pb.w_max)) bad = 1;
+          const double e = (double)yo[(size_t)kf * S.npts + pt] - w;
+          phi += e * e;
+        }
+      }
+      if (out) {
+        fo[pt] = S.ref_u + du;
+        fo[(size_t)S.npts + pt] = S.ref_v + dv;
+      }
+    }
+  }
+  if (!yo) return;
+  // 16 neighbouring lanes always hold the same proposal
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) phi += __shfl_xor_sync(0xffffffffu, phi, o);
+  if (sl >= 0) {
+    if ((threadIdx.x & 15) == 0) atomicAdd(&ctl->phi[sl], phi);
+    if (bad) atomicOr(&ctl->bad[sl], 1);
+  }
+}
+
+// A whole row of N nodes by Gaussian elimination (any lam and beta), from the
+// accumulator columns at t to the operand row l, columns col0...
+template <int N>
+__device__ __noinline__ void slow_row(uint32_t t, int g, int rows, int l, int col0, bool store,
+                                      float alpha, float beta, float mu, float out_scale) {
+  uint8_t* const hi = tile(shared_base(), g, 0);
+  uint8_t* const lo = tile(shared_base(), g, 1);
+  float c[N], d[N];
+  const float lam = fmaf(beta, mu, alpha);
+  float cp = 0.f, dp = 0.f;
+  for (int x = 0; x < N; x += 8) {
+    float v[8];
+    __syncwarp();
+    tmem_ld8(t + (uint32_t)x, v);
+    tmem_wait_ld();
+    for (int j = 0; j < 8; ++j) {
+      const int i = x + j;
+      const float den = lam + ((i == 0 || i == N - 1) ? beta : 2.f * beta) + beta * cp;
+      cp = -beta / den;
+      dp = (v[j] + beta * dp) / den;
+      c[i] = cp;
+      d[i] = dp;
+    }
+  }
+  float x1 = 0.f;
+  for (int i = N - 1; i >= 0; --i) {
+    x1 = d[i] - (i < N - 1 ? c[i] * x1 : 0.f);
+    d[i] = x1;
+  }
+  if (store)
+    for (int x = 0; x < N; x += 8) store8(hi, lo, rows, l, col0 + x, d + x, out_scale);
+}
+
+template <int H>
+__device__ __forceinline__ void load_cols(uint32_t t, float (&r)[H]) {
+  __syncwarp();
+  if constexpr (H % 16 == 0) {
+#pragma unroll
+    for (int x = 0; x < H; x += 16)
+      tmem_ld16(t + (uint32_t)x, *reinterpret_cast<float(*)[16]>(r + x));
+  } else {
+#pragma unroll
+    for (int x = 0; x < H; x += 8)
+      tmem_ld8(t + (uint32_t)x, *reinterpret_cast<float(*)[8]>(r + x));
+  }
+  tmem_wait_ld();
+}
+
+// One scan segment (segment seg of a row) of slab g: accumulator columns t..
+// -> operand row l, columns col0...  slot: where the row's sums are exchanged.
+template <int N>
+__device__ __forceinline__ bool scan_segment(uint64_t wait_ns, uint32_t t, int g, int seg,
+                                             int slot, int quad, uint32_t parity, int lane,
+                                             int col0, bool row_used, const ScanCoef& k) {
+  using SG = ScanSeg<N>;
+  constexpr int E = Geo<N>::S, H = SG::H;
+  uint8_t* const base = shared_base();
+  Ctrl* const ctl = shared_ctl();
+  const int l = 32 * quad + lane;
+  float r[H];
+  load_cols<H>(t, r);
+  float left, right;
+  {
+    float2 lr[SG::NS];
+    float L, R;
+    scan_sums<H>(r, k.a, L, R);
+    if constexpr (SG::NS > 1) {
+      ctl->sums[g][2 * slot + seg][l] = make_float2(L, R);
+      __syncwarp();
+      uint64_t* bar = &ctl->seg[g][quad][slot];
+      if (lane == 0) mbar_arrive(bar);
+      if (!mbar_wait_bounded(bar, parity, &ctl->abort, wait_ns)) return false;
+      const float2 other = ctl->sums[g][2 * slot + (seg ^ 1)][l];
+      lr[0] = seg ? other : make_float2(L, R);
+      lr[1] = seg ? make_float2(L, R) : other;
+    } else {
+      lr[0] = make_float2(L, R);
+    }
+    scan_entries<SG::NS>(lr, seg, k, left, right);
+  }
+  float x = left;
+#pragma unroll
+  for (int m = 0; m < H; ++m) {
+    x = fmaf(k.a, x, r[m]);
+    r[m] = x;
+  }
+  // down: X_{H-1} = (F_{H-1} + a right) / (1 - a^2), X_m = F_m + a X_{m+1}
+  x = fmaf(k.a, right, x) * k.g;
+  r[H - 1] = x;
+#pragma unroll
+  for (int m = H - 2; m >= 0; --m) {
+    x = fmaf(k.a, x, r[m]);
+    r[m] = x;
+    if (m % 8 == 0 && row_used)
+      store8(tile(base, g, 0), tile(base, g, 1), E, l, col0 + m, r + m, k.sc);
+  }
+  return true;
+}
+
+// The 16 converter warps, warp % 4 the TMEM lane quadrant, w4 = warp / 4 along
+// the columns.  N > 64: all of them do the reaction, then w4 = 0, 1 scan slab 0
+// and 2, 3 slab 1.  N <= 64: all of them do slab 0, then slab 1.
+template <int N>
+__device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, int warp, int lane,
+                                          const Parity& par, float* fields, size_t field_stride) {
+  using G = Geo<N>;
+  using SG = ScanSeg<N>;
+  constexpr int E = G::S;  // slab edge
+  uint8_t* const base = shared_base();
+  Ctrl* const ctl = shared_ctl();
+  const int size = ctl->size;
+  const DevSize& S = pb.sz[size];
+  volatile int* abort = &ctl->abort;
+  const uint64_t wait_ns = pb.wait_ns;
+  const int n_steps = pb.n_steps;
+  const bool growth = pb.growth != 0;
+  const int w4 = warp >> 2, quad = warp & 3;
+  const int l = 32 * quad + lane;
+  const int n_items = ctl->n_items;
+  const int slabs = (G::kPair || n_items > G::QB) ? 2 : 1;
+  const int p = G::kPair ? 0 : l / N;
+  const int idx = l - p * N;  // index along the lanes within the block
+  const int pmax = G::kPair ? 1 : (n_items + 2 * G::QB - 1) / (2 * G::QB);
+  const bool row_used = l < E && p < pmax;
+  const uint32_t t_acc = tmem + ((uint32_t)(32 * quad) << 16) + kColAcc;
+  const float ref_u = S.ref_u, ref_v = S.ref_v;
+  const float mu_l = l < E ? ctl->mu[idx] : 0.f;
+  const float kap = (float)N * 0x1p-29f;
+  const float out_scale = 0x1p-7f * (1.f + kap);
+  const bool slow = ctl->slow != 0;
+  // the slot of pair q in slab g: -1 for idle rows and blocks
+  auto slot = [&](int g, int q) {
+    const int s = G::kPair ? 0 : q + G::QB * (g + 2 * p);
+    return (row_used && s < n_items) ? s : -1;
+  };
+  // scan block i of this thread in a slab: its column block 2 q + f
+  auto block_of = [&](int i) {
+    return G::kPair ? 0 : (N >= 48 ? (w4 >> 1) : (N == 32 ? w4 : 2 * w4 + i));
+  };
+  constexpr int NG = G::kPair ? 1 : 2;  // slabs scanned by one thread
+  const int g0 = G::kPair ? (w4 >> 1) : 0;
+  const int seg = N >= 48 ? (w4 & 1) : 0;
+  auto alpha_beta = [&](int g, int i, int step, float& alpha, float& beta) {
+    const int s = slot(g, G::kPair ? 0 : block_of(i) >> 1);
+    const int f = G::kPair ? g : (block_of(i) & 1);
+    alpha = 1.f;
+    beta = 0.f;
+    if (s >= 0) {
+      alpha = ctl->rk[s].alpha;
+      beta = ctl->beta[growth ? step & 1 : 0][s][f];
+    }
+  };
+  ScanCoef sc[NG][G::NB];  // recomputed each step on a growing domain
+  auto set_coef = [&](int step) {
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+      for (int i = 0; i < G::NB; ++i) {
+        float alpha, beta;
+        alpha_beta(g0 + g, i, step, alpha, beta);
+        sc[g][i] = scan_coef<N>(alpha, beta, mu_l, out_scale);
+      }
+  };
+  if (!growth) set_coef(0);
   int next_obs = 0;
   for (int step = 0;; ++step) {
-    if (step > 0) {  // stage 4 of both fields done: the fourth commit of a step
-      // completes an odd phase, and the other field's stage-4 phase is the one
-      // pending or just completed (the MMAs complete in issue order)
-      if (!mbar_wait_bounded(&ctl->mma_done[f], ph_done & 1u, abort, pb.wait_ns)) return false;
-      ++ph_done;
-      if (!mbar_wait_bounded(&ctl->mma_done[f ^ 1], 1u, abort, pb.wait_ns)) return false;
-      tc_fence_after();
-    }
-    const bool last = step == pb.n_steps;
-    const float sw = step > 0 ? kScaleW : 0x1p-7f;
-    const bool obs = next_obs < S.n_obs && step == S.obs_steps[next_obs];
-    ObsCtx o;
-    o.yo = obs ? S.yf + (size_t)next_obs * nfo * S.npts : nullptr;
-    o.fo = (last && fields) ? fields + (size_t)ctl->item * field_stride : nullptr;
-    o.odd = step & 1;
-    if (obs) ++next_obs;
-    float alpha = 1.f, cu = 0.f, cv = 0.f;
-    float beta_f = beta_fixed;
-    if (pb.growth) {  // FP64, rounded once per step
-      const double rho2inv = exp(-2.0 * r * (double)step * tau);
-      alpha = (float)(1.0 + tau * 2.0 * r);
-      cu = (float)(-tau * 2.0 * r * (double)ref_u);
-      cv = (float)(-tau * 2.0 * r * (double)ref_v);
-      beta_f = (float)(tau * (f ? th[2] : 1.0) * rho2inv * (double)N * N);
+    const bool last = step == n_steps;
+    const float sw = step > 0 ? 0x1p-7f * (1.f + kap) : 0x1p-7f;
+    const uint32_t ph = (uint32_t)step & 1u;
+    const int obs = (next_obs < S.n_obs && step == S.obs_steps[next_obs]) ? next_obs++ : -1;
+    if (growth && !last) {  // this step's beta is ready (see grower)
+      if (!mbar_wait_bounded(&ctl->grow, ph ^ par.p0, abort, wait_ns)) return;
     }
     // ---- observation / output, then the reaction -> stage-1 operands
-#pragma unroll 1
-    for (int half = 0; half < 2; ++half) {
-      const int x0 = 64 * half + XW * p;
-      float uh[XW], vh[XW];  // all loads of the half in flight at once
+    if constexpr (G::kPair) {
+      if (step > 0) {  // stage 2 of both slabs: the second commit of a step ends an odd phase
+        if (!mbar_wait_bounded(&ctl->mma_done[0], 1u, abort, wait_ns)) return;
+        if (!mbar_wait_bounded(&ctl->mma_done[1], 1u, abort, wait_ns)) return;
+        tc_fence_after();
+      }
+      if (obs >= 0 || last)
+        observe(pb, size, slot(0, 0), idx, 8 * w4, 4, (N - 8 * w4 + 31) / 32, t_acc, t_acc + 128u,
+                sw, step, obs, fields, field_stride);
+      if (last) return;
+      const int s = slot(0, 0);
+      React k = {0.f, 0.f, 0.f, 1.f, 0.f, 0.f};
+      if (s >= 0) k = ctl->rk[s];
+      // the whole share is loaded first: the first half's MMAs overwrite the state
+      float u[32], v[32];
       __syncwarp();
 #pragma unroll
-      for (int j = 0; j < XW; j += 8) {
-        tmem_ld8(t_u + (uint32_t)(x0 + j), *reinterpret_cast<float(*)[8]>(uh + j));
-        tmem_ld8(t_v + (uint32_t)(x0 + j), *reinterpret_cast<float(*)[8]>(vh + j));
+      for (int j = 0; j < 4; ++j) {
+        const int c = 32 * j + 8 * w4;
+        if (c < N) {
+          tmem_ld8(t_acc + (uint32_t)c, *reinterpret_cast<float(*)[8]>(u + 8 * j));
+          tmem_ld8(t_acc + 128u + (uint32_t)c, *reinterpret_cast<float(*)[8]>(v + 8 * j));
+        }
       }
       tmem_wait_ld();
+      tc_fence_before();
 #pragma unroll
-      for (int j = 0; j < XW; j += 8) {
-        if (o.yo || o.fo) observe8(pb, S, o, l, x0 + j, uh + j, vh + j, sw, phi, bad);
-        if (last) continue;
-        react8(uh + j, vh + j, sw, ref_u, ref_v, fa, fb, ftg, cu, cv);
-        store8n(hi_u, lo_u, l, x0 + j, uh + j);
-        store8n(hi_v, lo_v, l, x0 + j, vh + j);
-      }
-    }
-    if (last) break;
-    fence_proxy_async_smem();
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&ctl->rx_ready);
-
-    // ---- stages 1-3 of field f -> operands of stages 2-4
-#pragma unroll 1
-    for (int stage = 1; stage <= 3; ++stage) {
-      if (!mbar_wait_bounded(&ctl->mma_done[f], ph_done & 1u, abort, pb.wait_ns)) return false;
-      ++ph_done;
-      tc_fence_after();
-
-      // this warp's 64 columns in 4 chunks of 16, the next chunk's TMEM load in
-      // flight while the current one is converted
-      constexpr int NQ = CW / 8;  // chunks of 16 columns, both halves
-      int cols[NQ];
-#pragma unroll
-      for (int qq = 0; qq < NQ; ++qq)
-        cols[qq] = 64 * (qq / (NQ / 2)) + CW * rr + 16 * (qq % (NQ / 2));
-      float buf[2][16];
-      __syncwarp();
-      tmem_ld16(t_f + (uint32_t)cols[0], buf[0]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        float* a = buf[q & 1];
-        if (q < NQ - 1) tmem_ld16(t_f + (uint32_t)cols[q + 1], buf[(q + 1) & 1]);
-        const int c0 = cols[q];
-        if (stage == 2) {  // S = D L, L from mu_l + mu_k two columns at a time
-          const uint64_t ml2 = f2_pack(mu_l, mu_l), be2 = f2_pack(beta_f, beta_f);
-          const uint64_t al2 = f2_pack(alpha, alpha), ks2 = f2_pack(kScaleL, kScaleL);
-#pragma unroll
-          for (int k = 0; k < 16; k += 8) {
-            float lam8[8];
-#pragma unroll
-            for (int jj = 0; jj < 8; jj += 2) {
-              const float2 mc = *reinterpret_cast<const float2*>(&ctl->mu[c0 + k + jj]);
-              const uint64_t x2 = f2_fma(f2_add(ml2, f2_pack(mc.x, mc.y)), be2, al2);
-              f2_unpack(f2_mul(f2_recip(x2), ks2), lam8[jj], lam8[jj + 1]);
-            }
-            store8s(hi_f, lo_f, l, c0 + k, a + k, lam8);
-          }
-        } else {
-#pragma unroll
-          for (int k = 0; k < 16; k += 8) {
-            if (stage == 1)
-              store8(hi_f, lo_f, l, c0 + k, a + k, kScale1);
-            else
-              store8n(hi_f, lo_f, l, c0 + k, a + k);
+      for (int j = 0; j < 4; ++j) {
+        const int c = 32 * j + 8 * w4;
+        if (c < N) {
+          react8(u + 8 * j, v + 8 * j, sw, ref_u, ref_v, k);
+          if (row_used) {
+            store8n<false>(tile(base, 0, 0), tile(base, 0, 1), E, idx, c, u + 8 * j);
+            store8n<false>(tile(base, 1, 0), tile(base, 1, 1), E, idx, c, v + 8 * j);
           }
         }
-        if (q < NQ - 1) tmem_wait_ld();
+        if (j & 1) {
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&ctl->rx[j >> 1]);
+        }
+      }
+    } else {
+      // 8-column chunks of this warp: N = 64: 2, 48: 2 or 1, 32 and 16: 2 of one pair
+      const int q = N >= 48 ? 0 : (N == 32 ? (w4 >> 1) : w4);
+      const int c0 = N >= 48 ? 8 * w4 : (N == 32 ? 16 * (w4 & 1) : 0);
+      constexpr int CS = N >= 48 ? 32 : 8;  // stride between the chunks
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        if (g >= slabs) break;
+        if (step > 0) {
+          if (!mbar_wait_bounded(&ctl->mma_done[g], 1u, abort, wait_ns)) return;
+          tc_fence_after();
+        }
+        const uint32_t t_u = t_acc + (uint32_t)(128 * g + 2 * q * N), t_v = t_u + (uint32_t)N;
+        const int s = slot(g, q);
+        if (obs >= 0 || last)
+          observe(pb, size, s, idx, c0, CS / 8, c0 + CS < N ? 2 : 1, t_u, t_v, sw, step, obs,
+                  fields, field_stride);
+        if (last) continue;
+        React k = {0.f, 0.f, 0.f, 1.f, 0.f, 0.f};
+        if (s >= 0) k = ctl->rk[s];
+        float u[16], v[16];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int c = c0 + CS * j;
+          if (c < N) {
+            tmem_ld8(t_u + (uint32_t)c, *reinterpret_cast<float(*)[8]>(u + 8 * j));
+            tmem_ld8(t_v + (uint32_t)c, *reinterpret_cast<float(*)[8]>(v + 8 * j));
+          }
+        }
+        tmem_wait_ld();
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int c = c0 + CS * j;
+          if (c < N) {
+            react8(u + 8 * j, v + 8 * j, sw, ref_u, ref_v, k);
+            if (row_used) {
+              const int row = 2 * q * N + idx;
+              const bool b1 = store8n<true>(tile(base, g, 0), tile(base, g, 1), E, row, p * N + c,
+                                            u + 8 * j);
+              const bool b2 = store8n<true>(tile(base, g, 0), tile(base, g, 1), E, row + N,
+                                            p * N + c, v + 8 * j);
+              if ((b1 || b2) && s >= 0) ctl->blown[s] = 1;
+            }
+          }
+        }
+        fence_proxy_async_smem();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->rx[g]);
+      }
+      if (last) return;
+    }
+    // ---- stage 1 done: solve along the columns -> operand of stage 2
+    if (growth) set_coef(step);
+#pragma unroll
+    for (int gi = 0; gi < NG; ++gi) {
+      if (gi >= slabs) break;
+      const int g = g0 + gi;
+      if (!mbar_wait_bounded(&ctl->mma_done[g], 0u, abort, wait_ns)) return;
+      tc_fence_after();
+#pragma unroll
+      for (int i = 0; i < G::NB; ++i) {
+        const int col0 = block_of(i) * N + seg * SG::H;
+        const uint32_t t = t_acc + (uint32_t)(128 * g + col0);
+        if (slow) {
+          if (seg == 0) {
+            float alpha, beta;
+            alpha_beta(g, i, step, alpha, beta);
+            slow_row<N>(t, g, E, l, col0, row_used, alpha, beta, mu_l, out_scale);
+          }
+        } else if (!scan_segment<N>(wait_ns, t, g, seg, G::kPair ? 0 : block_of(i) & 1, quad,
+                                    ph ^ (NG == 2 && gi == 1 ? par.seg >> 1 : par.seg & 1u), lane,
+                                    col0, row_used, sc[gi][i])) {
+          return;
+        }
       }
       fence_proxy_async_smem();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl->op_all[f]);
+      if (lane == 0) mbar_arrive(&ctl->op_ready[g]);
     }
   }
-  atomicAdd(&ctl->phi, phi);
-  if (bad) atomicOr(&ctl->bad, 1);
-  return true;
 }
 
-__device__ bool issuer(const DevProblem& pb, Ctrl* ctl, uint8_t* base, uint32_t tmem, int lane,
-                       uint32_t& ph_rx, uint32_t (&ph_all)[2]) {
+// The MMA-issuing warp.
+template <int N>
+__device__ __forceinline__ bool issuer(const DevProblem& pb, uint32_t tmem, int lane,
+                                       const Parity& par) {
+  using G = Geo<N>;
+  constexpr int E = G::S, KB = E / 16;
+  Ctrl* const ctl = shared_ctl();
+  // warp-uniform values, so that the descriptors stay in uniform registers
+  const uint32_t sbase = __shfl_sync(0xffffffffu, smem_u32(shared_base()), 0);
+  tmem = __shfl_sync(0xffffffffu, tmem, 0);
   volatile int* abort = &ctl->abort;
-  for (int step = 0; step < pb.n_steps; ++step) {
-    if (!mbar_wait_bounded(&ctl->rx_ready, ph_rx & 1u, abort, pb.wait_ns)) return false;
-    ++ph_rx;
-    tc_fence_after();
-    if (lane == 0) {
-#pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        issue_kmajor(base, tmem, 1, f);
-        mma_commit(&ctl->mma_done[f]);
+  const int items = ctl->n_items;
+  const int pmax = G::kPair ? 1 : (items + 2 * G::QB - 1) / (2 * G::QB);
+  const int kb = G::kPair ? KB : pmax * N / 16;                                // K blocks in use
+  const int ncols = G::kPair ? N : 2 * N * (items < G::QB ? items : G::QB);    // columns in use
+  const int slabs = (G::kPair || items > G::QB) ? 2 : 1;
+  const int n_steps = pb.n_steps;
+  const uint64_t wait_ns = pb.wait_ns;
+  for (int step = 0; step < n_steps; ++step) {
+    const uint32_t ph = (uint32_t)step & 1u;
+    if constexpr (G::kPair) {
+      // the correction products of the reaction's first half (64 columns)
+      // while its second half is computed
+      if (!mbar_wait_bounded(&ctl->rx[0], ph ^ par.p0, abort, wait_ns)) return false;
+      tc_fence_after();
+      if (elect_one()) {
+        issue_blocks<1, E, true, false, 0, 4, true>(sbase, tmem, 0, N, KB);
+        issue_blocks<1, E, true, false, 0, 4, true>(sbase, tmem, 1, N, KB);
       }
-    }
-    __syncwarp();
-    if (step == pb.stall_step) {  // test aid: wait on a barrier nothing completes
-      mbar_wait_bounded(&ctl->never, 0u, abort, pb.wait_ns);
-      return false;
-    }
-#pragma unroll 1
-    for (int stage = 2; stage <= 4; ++stage) {
+      __syncwarp();
+      if (!mbar_wait_bounded(&ctl->rx[1], ph ^ par.p1, abort, wait_ns)) return false;
+      tc_fence_after();
+      if (elect_one()) {
 #pragma unroll
-      for (int f = 0; f < 2; ++f) {
-        if (!mbar_wait_bounded(&ctl->op_all[f], ph_all[f] & 1u, abort, pb.wait_ns)) return false;
-        ++ph_all[f];
+        for (int g = 0; g < 2; ++g) {
+          issue_blocks<1, E, true, false, 4, KB, false>(sbase, tmem, g, N, KB);
+          issue_blocks<1, E, false, true, 0, KB, false>(sbase, tmem, g, N, KB);
+          mma_commit(&ctl->mma_done[g]);
+        }
+      }
+      __syncwarp();
+    } else {
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        if (g >= slabs) break;
+        if (!mbar_wait_bounded(&ctl->rx[g], ph ^ (g ? par.p1 : par.p0), abort, wait_ns))
+          return false;
         tc_fence_after();
-        if (lane == 0) {
-          if (stage == 3)
-            issue_stage3(base, tmem, f);
-          else
-            issue_kmajor(base, tmem, stage, f);
-          mma_commit(&ctl->mma_done[f]);
+        if (elect_one()) {
+          issue_blocks<1, E, true, true, 0, KB, true>(sbase, tmem, g, ncols, kb);
+          mma_commit(&ctl->mma_done[g]);
         }
         __syncwarp();
       }
     }
+    if (step == pb.stall_step) {  // test aid: wait on a barrier nothing completes
+      mbar_wait_bounded(&ctl->never, 0u, abort, wait_ns);
+      return false;
+    }
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      if (g >= slabs) break;
+      if (!mbar_wait_bounded(&ctl->op_ready[g], ph ^ (g ? par.p1 : par.p0), abort, wait_ns))
+        return false;
+      tc_fence_after();
+      if (elect_one()) {
+        issue_blocks<2, E, true, true, 0, KB, true>(sbase, tmem, g, ncols, kb);
+        mma_commit(&ctl->mma_done[g]);
+      }
+      __syncwarp();
+    }
   }
   return true;
 }
 
-}  // namespace tc2
+// Growing domain: one warp forms the steps' beta = tau D / (rho_n^2 h^2) in
+// FP64 (rho_n = exp(r n tau)), one step ahead of the converters.
+template <int N>
+__device__ __noinline__ bool grower(const DevProblem& pb, int lane, Parity par) {
+  using G = Geo<N>;
+  Ctrl* const ctl = shared_ctl();
+  volatile int* abort = &ctl->abort;
+  const int items = ctl->n_items;
+  const int slabs = (G::kPair || items > G::QB) ? 2 : 1;
+  const double tau = pb.tau;
+  for (int step = 0; step < pb.n_steps; ++step) {
+    // once the reaction of step - 1 is written, every converter has taken the
+    // beta of step - 2 (this buffer) and passed its wait for that of step - 1
+    for (int g = 0; step >= 1 && g < slabs; ++g)
+      if (!mbar_wait_bounded(&ctl->rx[g], ((uint32_t)(step - 1) & 1u) ^ (g ? par.p1 : par.p0),
+                             abort, pb.wait_ns))
+        return false;
+    for (int i = lane; i < items; i += 32) {
+      const double rho2inv = exp(-2.0 * ctl->th[i][4] * (double)step * tau);
+      ctl->beta[step & 1][i][0] = (float)(tau * rho2inv * (double)N * N);
+      ctl->beta[step & 1][i][1] = (float)(tau * ctl->th[i][2] * rho2inv * (double)N * N);
+    }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&ctl->grow);
+  }
+  return true;
+}
 
-template <int WPF>
-__global__ void __launch_bounds__(32 * (8 * WPF + 1), 1)
-    k_solve2d_tc128(DevProblem pb, WorkQueue q, const double* theta, double* phi,
-                    uint32_t* status, float* fields, size_t field_stride, int* err) {
-  using namespace tc2;
-  constexpr int kConvWarps = 8 * WPF;
-  constexpr int kThreads = 32 * (kConvWarps + 1);
-  extern __shared__ uint8_t smem_raw[];
-  // 1024-byte aligned start, derived from smem_raw so that the compiler keeps
-  // the shared address space (plain shared loads and stores, not generic)
-  uint8_t* base = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  Ctrl* ctl = reinterpret_cast<Ctrl*>(base + kOffCtrl);
+// Proposals the scan does not cover (negative diffusion, a growth factor out
+// of range, non-finite parameters): solved alone, by elimination.
+__device__ __forceinline__ bool irregular(const DevProblem& pb, const double th[kNPhys]) {
+  bool fin = true;
+  for (int j = 0; j < kNPhys; ++j) fin = fin && isfinite(th[j]);
+  if (!fin || !(th[2] >= 0.0)) return true;
+  if (!pb.growth) return false;
+  return !(1.0 + 2.0 * pb.tau * th[4] > 0.0) ||
+         !(fabs(2.0 * th[4] * pb.tau * pb.n_steps) < 40.0);
+}
+
+// Pops proposals of one size of the queue: as many as a CTA holds, fewer when
+// the batch is too small to fill every CTA that way.  Irregular ones go last.
+template <int N>
+__device__ __forceinline__ void pop_chunk(const DevProblem& pb, const WorkQueue& q,
+                                          const double* theta, Ctrl* ctl) {
+  constexpr int cap = Geo<N>::kCap;
+  ctl->n_chunk = ctl->next = 0;
+  int full = 0;  // CTAs that the whole batch would fill
+  for (int k = 0; k < q.n_sizes; ++k)
+    full += (*((volatile int*)&q.counts[q.order[k]]) + cap - 1) / cap;
+  const int take = full < (int)gridDim.x ? (cap * full + (int)gridDim.x - 1) / (int)gridDim.x : cap;
+  for (int k = 0; k < q.n_sizes; ++k) {
+    const int s = q.order[k];
+    const int cnt = *((volatile int*)&q.counts[s]);
+    if (*((volatile int*)&q.pops[s]) >= cnt) continue;
+    const int i = atomicAdd(&q.pops[s], take);
+    if (i >= cnt) continue;
+    const int m = min(take, cnt - i);
+    int a = 0, z = m;
+    for (int j = 0; j < m; ++j) {
+      const int item = q.items[(size_t)s * q.capacity + i + j];
+      double th[kNPhys];
+      full_theta(pb, theta + (size_t)item * pb.n_params, th);
+      if (irregular(pb, th))
+        ctl->chunk[--z] = item;
+      else
+        ctl->chunk[a++] = item;
+    }
+    ctl->n_chunk = m;
+    ctl->slow = a;  // regular items at the front
+    ctl->size = s;
+    return;
+  }
+}
+
+// The next proposals to solve, into ctl: a chunk's regular ones together, its
+// irregular ones one by one (ctl->slow counts the regular ones until then).
+template <int N>
+__device__ __noinline__ void next_items(const DevProblem& pb, const WorkQueue& q,
+                                        const double* theta) {
+  Ctrl* const ctl = shared_ctl();
+  ctl->n_items = 0;
+  if (ctl->abort) return;
+  if (ctl->next >= ctl->n_chunk) pop_chunk<N>(pb, q, theta, ctl);
+  if (ctl->next >= ctl->n_chunk) return;
+  const int reg = ctl->next == 0 ? ctl->slow : 0;
+  const int m = reg > 0 ? reg : 1;
+  for (int j = 0; j < m; ++j) {
+    ctl->items[j] = ctl->chunk[ctl->next + j];
+    full_theta(pb, theta + (size_t)ctl->items[j] * pb.n_params, ctl->th[j]);
+  }
+  ctl->next += m;
+  ctl->slow = reg > 0 ? 0 : 1;
+  ctl->n_items = m;
+}
+
+// Step constants of item j (the growing domain's beta: see grower).
+__device__ __forceinline__ void item_constants(const DevProblem& pb, const DevSize& S, Ctrl* ctl,
+                                               int j) {
+  const double* th = ctl->th[j];
+  const double tau = pb.tau;
+  React k;
+  k.fa = (float)th[0];
+  k.fb = (float)th[1];
+  k.ftg = (float)(tau * th[3]);
+  k.cu = k.cv = 0.f;
+  k.alpha = 1.f;
+  if (pb.growth) {
+    k.alpha = (float)(1.0 + tau * 2.0 * th[4]);
+    k.cu = (float)(-tau * 2.0 * th[4] * (double)S.ref_u);
+    k.cv = (float)(-tau * 2.0 * th[4] * (double)S.ref_v);
+  } else {
+    ctl->beta[0][j][0] = (float)(tau * (double)S.n * S.n);
+    ctl->beta[0][j][1] = (float)(tau * th[2] * (double)S.n * S.n);
+  }
+  ctl->rk[j] = k;
+  ctl->phi[j] = 0.0;
+  ctl->bad[j] = ctl->blown[j] = 0;
+}
+
+// A size's 8C and 8C^T, block-diagonal over the slab's lane blocks, as split
+// FP16 into TMEM (lane = output index): converter warps 0-7 C, 8-15 C^T.
+template <int N>
+__device__ __noinline__ void fill_constants(const DevSize& S, uint32_t tmem, int warp, int lane) {
+  constexpr int n = N, edge = Geo<N>::S;
+  Ctrl* const ctl = shared_ctl();
+  const bool tr = warp >= 8;
+  const int m = 32 * (warp & 3) + lane;
+  const int mb = m / n, mi = m - mb * n;
+  const uint32_t t = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + kColA + (tr ? 128u : 0u);
+  const int cbase = 32 * ((warp >> 2) & 1);
+  for (int c0 = cbase; c0 < cbase + 32; c0 += 8) {
+    float vh[8], vl[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float e[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int kc = 2 * (c0 + j) + k, kb = kc / n, ki = kc - kb * n;
+        e[k] = (m < edge && kc < edge && kb == mb)
+                   ? 8.f * (tr ? S.cmat[(size_t)ki * n + mi] : S.cmat[(size_t)mi * n + ki])
+                   : 0.f;
+      }
+      __half h0, l0, h1, l1;
+      split_f16(e[0], h0, l0);
+      split_f16(e[1], h1, l1);
+      vh[j] = __uint_as_float((uint32_t)__half_as_ushort(h0) |
+                              ((uint32_t)__half_as_ushort(h1) << 16));
+      vl[j] = __uint_as_float((uint32_t)__half_as_ushort(l0) |
+                              ((uint32_t)__half_as_ushort(l1) << 16));
+    }
+    __syncwarp();
+    tmem_st8(t + (uint32_t)c0, vh);
+    tmem_st8(t + 64u + (uint32_t)c0, vl);
+  }
+  tmem_wait_st();
+  for (int i = 32 * warp + lane; i < n; i += 32 * kConvWarps) ctl->mu[i] = S.mu[i];
+}
+
+// Initial deviations (x 128), y on the lanes: four warps per quadrant share the
+// 256 accumulator columns.
+template <int N>
+__device__ __forceinline__ void initial_state(const DevSize& S, uint32_t tmem, int warp,
+                                              int lane) {
+  using G = Geo<N>;
+  const int l = 32 * (warp & 3) + lane;
+  const uint32_t t = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + kColAcc;
+  const int y = l < G::S ? l % N : 0;
+  for (int c8 = 8 * (warp >> 2); c8 < 256; c8 += 32) {
+    const int g = c8 >> 7, c = c8 & 127;
+    if (c >= G::S) continue;  // warp-uniform
+    const int f = G::kPair ? g : ((c / N) & 1);
+    const int x = G::kPair ? c : c % N;
+    const float ref = f ? S.ref_v : S.ref_u;
+    const float* w0 = f ? S.v0f : S.u0f;
+    float v8[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v8[j] = (w0[(size_t)y * N + x + j] - ref) * 128.f;
+    __syncwarp();
+    tmem_st8(t + (uint32_t)c8, v8);
+  }
+  tmem_wait_st();
+}
+
+// The persistent CTA: takes proposals from the queue until it is empty.
+template <int N>
+__device__ __forceinline__ void solve_loop(const DevProblem& pb, const WorkQueue& q,
+                                           const double* theta, double* phi, uint32_t* status,
+                                           float* fields, size_t field_stride, int* err) {
+  Ctrl* const ctl = shared_ctl();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == kConvWarps) {
+  if (warp == kIssueWarp) {
     tmem_alloc(&ctl->tmem_base, 512);
     tmem_relinquish();
   }
   if (tid == 0) {
-    for (int f = 0; f < 2; ++f) {
-      mbar_init(&ctl->mma_done[f], 1);
-      mbar_init(&ctl->op_all[f], kConvWarps / 2);
+    for (int g = 0; g < 2; ++g) {
+      mbar_init(&ctl->mma_done[g], 1);
+      mbar_init(&ctl->op_ready[g], Geo<N>::kOpWarps);
+      mbar_init(&ctl->rx[g], kConvWarps);
+      for (int i = 0; i < 8; ++i) mbar_init(&ctl->seg[g][i >> 1][i & 1], 2);
     }
-    mbar_init(&ctl->rx_ready, kConvWarps);
+    mbar_init(&ctl->grow, 1);
     mbar_init(&ctl->fin, 1);
     mbar_init(&ctl->never, 1);
     ctl->abort = 0;
+    ctl->n_chunk = ctl->next = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
-  // every size in this kernel's queue is 128^2: one DCT matrix serves all
-  const DevSize& S0 = pb.sz[q.order[0]];
-  // 8C and 8C^T as split FP16 into TMEM (lane = output index), once per CTA:
-  // the first half of the converter warps C, the second C^T
-  if (warp < kConvWarps) {
-    const bool tr = warp >= 4 * WPF;
-    const int m = 32 * (warp & 3) + lane;
-    const int cbase = (64 / WPF) * ((warp >> 2) % WPF);
-    const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    for (int c0 = cbase; c0 < cbase + 64 / WPF; c0 += 8) {
-      float vh[8], vl[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int k0 = 2 * (c0 + j), k1 = k0 + 1;
-        const float e0 = 8.f * (tr ? S0.cmat[(size_t)k0 * N + m] : S0.cmat[(size_t)m * N + k0]);
-        const float e1 = 8.f * (tr ? S0.cmat[(size_t)k1 * N + m] : S0.cmat[(size_t)m * N + k1]);
-        __half h0, l0, h1, l1;
-        split_f16(e0, h0, l0);
-        split_f16(e1, h1, l1);
-        vh[j] = __uint_as_float((uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16));
-        vl[j] = __uint_as_float((uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16));
-      }
-      __syncwarp();
-      tmem_st8(tmem + lane_off + (tr ? kColCtHi : kColCHi) + (uint32_t)c0, vh);
-      tmem_st8(tmem + lane_off + (tr ? kColCtLo : kColCLo) + (uint32_t)c0, vl);
-    }
-    tmem_wait_st();
-  }
-  for (int i = tid; i < N; i += kThreads) ctl->mu[i] = S0.mu[i];
-  uint32_t ph_done = 0, ph_rx = 0;
-  uint32_t ph_all[2] = {0, 0};
+  // every size of this launch is N x N: one DCT matrix serves all
+  if (warp < kConvWarps) fill_constants<N>(pb.sz[q.order[0]], tmem, warp, lane);
+  Parity par;
   for (;;) {
-    tc_fence_before();
+    if (tid == 0) next_items<N>(pb, q, theta);
     __syncthreads();
-    tc_fence_after();
-    if (tid == 0) {
-      int sz = 0;
-      ctl->item = ctl->abort ? -1 : queue_pop(q, &sz);
-      ctl->size = sz;
-      if (ctl->item >= 0) full_theta(pb, theta + (size_t)ctl->item * pb.n_params, ctl->th);
-      ctl->phi = 0.0;
-      ctl->bad = 0;
-    }
-    __syncthreads();
-    if (ctl->item < 0) break;
+    const int n_items = ctl->n_items;
+    if (n_items == 0) break;
     const DevSize& S = pb.sz[ctl->size];
-    if (warp < kConvWarps) {  // initial deviations (x 128), y on the lanes
-      const int l = 32 * (warp & 3) + lane;
-      const int p = warp >> 2;
-      const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-      for (int f = 0; f < 2; ++f) {
-        const float ref = f ? S.ref_v : S.ref_u;
-        const float* w0 = f ? S.v0f : S.u0f;
-        for (int x = (32 / WPF) * p; x < N; x += 64) {
-#pragma unroll
-          for (int x8 = 0; x8 < 32 / WPF; x8 += 8) {
-            float v8[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v8[j] = (w0[(size_t)l * N + x + x8 + j] - ref) * 128.f;
-            __syncwarp();
-            tmem_st8(tmem + lane_off + kColAcc + (uint32_t)(128 * f + x + x8), v8);
-          }
-        }
-      }
-      tmem_wait_st();
-    }
+    if (tid < n_items) item_constants(pb, S, ctl, tid);
+    if (warp < kConvWarps) initial_state<N>(S, tmem, warp, lane);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     if (warp < kConvWarps)
-      converter<WPF>(pb, S, ctl, base, tmem, warp, lane, ph_done, fields, field_stride);
-    else
-      issuer(pb, ctl, base, tmem, lane, ph_rx, ph_all);
+      converter<N>(pb, tmem, warp, lane, par, fields, field_stride);
+    else if (warp == kIssueWarp)
+      issuer<N>(pb, tmem, lane, par);
+    else if (pb.growth)
+      grower<N>(pb, lane, par);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (tid == 0 && !ctl->abort) {
-      const int b = ctl->item;
-      status[b] = ctl->bad ? (uint32_t)RD_P_NONFINITE : 0u;
-      phi[b] = ctl->bad ? (double)INFINITY : ctl->phi * S.inv_two_sigma2;
+    if (pb.n_steps & 1) {
+      const bool both = Geo<N>::kPair || n_items > Geo<N>::QB;
+      par.p0 ^= 1u;
+      if (both) par.p1 ^= 1u;
+      if (!ctl->slow) par.seg ^= both ? 3u : 1u;
     }
+    if (!ctl->abort && tid < n_items) {
+      const int b = ctl->items[tid];
+      status[b] = ctl->bad[tid] ? (uint32_t)RD_P_NONFINITE : 0u;
+      phi[b] = ctl->bad[tid] ? (double)INFINITY : ctl->phi[tid] * S.inv_two_sigma2;
+    }
+    __syncthreads();
   }
-  if (warp == kConvWarps) {
+  if (warp == kIssueWarp) {
     if (lane == 0) mma_commit(&ctl->fin);
     __syncwarp();
     volatile int never = 0;
@@ -565,27 +941,56 @@ __global__ void __launch_bounds__(32 * (8 * WPF + 1), 1)
   if (tid == 0 && ctl->abort) atomicOr(err, 1);
 }
 
-bool tc128_applicable(const DevProblem& pb, int size_idx) {
-  return pb.dim == 2 && pb.sz[size_idx].n == 128;
+}  // namespace tc2
+
+template <int N>
+__global__ void __launch_bounds__(tc2::kThreads, 1)
+    k_solve2d_tc(const __grid_constant__ DevProblem pb, const __grid_constant__ WorkQueue q,
+                 const double* theta, double* phi, uint32_t* status, float* fields,
+                 size_t field_stride, int* err) {
+  tc2::solve_loop<N>(pb, q, theta, phi, status, fields, field_stride, err);
 }
 
-// Converter warps per TMEM lane quadrant and field.
-constexpr int kTc128Wpf = 2;
-
-cudaError_t setup_solve_tc128() {
-  return cudaFuncSetAttribute(k_solve2d_tc128<kTc128Wpf>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc2::kSmemBytes);
+// 128 x 128: SLABS accumulator slabs, one per field.
+template <int SLABS>
+__global__ void __launch_bounds__(tc2::kThreads, 1)
+    k_solve2d_tc128(const __grid_constant__ DevProblem pb, const __grid_constant__ WorkQueue q,
+                    const double* theta, double* phi, uint32_t* status, float* fields,
+                    size_t field_stride, int* err) {
+  static_assert(SLABS == 2, "the barriers and TMEM columns are laid out for two slabs");
+  tc2::solve_loop<128>(pb, q, theta, phi, status, fields, field_stride, err);
 }
 
-int grid_solve_tc128(int n_sm) { return n_sm; }
+static const void* tc_kernel(int n) {
+  switch (n) {
+    case 16: return (const void*)k_solve2d_tc<16>;
+    case 32: return (const void*)k_solve2d_tc<32>;
+    case 48: return (const void*)k_solve2d_tc<48>;
+    case 80: return (const void*)k_solve2d_tc<80>;
+    case 96: return (const void*)k_solve2d_tc<96>;
+    case 112: return (const void*)k_solve2d_tc<112>;
+    case 64: return (const void*)k_solve2d_tc<64>;
+    default: return (const void*)k_solve2d_tc128<2>;
+  }
+}
 
-cudaError_t launch_solve_tc128(const DevProblem& pb, const WorkQueue& q, const double* theta,
-                               double* phi, uint32_t* status, void* fields, int grid, int* err,
-                               cudaStream_t st) {
-  const size_t stride = (size_t)2 * pb.max_n * pb.max_n;
-  k_solve2d_tc128<kTc128Wpf><<<grid, 32 * (8 * kTc128Wpf + 1), tc2::kSmemBytes, st>>>(
-      pb, q, theta, phi, status, (float*)fields, stride, err);
-  return cudaGetLastError();
+cudaError_t setup_solve_tc(int n) {
+  return cudaFuncSetAttribute(tc_kernel(n), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)tc2::kSmemBytes);
+}
+
+int grid_solve_tc(int n_sm) { return n_sm; }
+
+cudaError_t launch_solve_tc(const DevProblem& pb, const WorkQueue& q, const double* theta,
+                            double* phi, uint32_t* status, void* fields, int grid, int* err,
+                            cudaStream_t st) {
+  size_t stride = (size_t)2 * pb.max_n * pb.max_n;
+  DevProblem pbv = pb;
+  WorkQueue qv = q;
+  float* fo = (float*)fields;
+  void* args[] = {&pbv, &qv, (void*)&theta, &phi, &status, &fo, &stride, &err};
+  return cudaLaunchKernel(tc_kernel(pb.sz[q.order[0]].n), dim3(grid), dim3(tc2::kThreads), args,
+                          tc2::kSmemBytes, st);
 }
 
 }  // namespace rd

@@ -107,22 +107,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
-// 32 lanes x 32-bit, 32 consecutive columns.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
 // 32 lanes x 32-bit, 16 consecutive columns.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
@@ -150,6 +134,15 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
 }
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(is));
+  return is != 0;
 }
 
 // ---------------------------------------------------------------- MMA
@@ -214,99 +207,12 @@ __device__ __forceinline__ float recip_nr(float x) {
   return fmaf(r, fmaf(-x, r, 1.f), r);
 }
 
-// split_f16 of two values at once: .x holds a, .y holds b (a at the lower
-// address when stored).
-__device__ __forceinline__ void split_f16x2(float a, float b, __half2& hi, __half2& lo) {
-  hi = __floats2half2_rn(a, b);
-  const float2 h = __half22float2(hi);
-  lo = __floats2half2_rn(a - h.x, b - h.y);
-}
-
-// ---------------------------------------------------------------- packed FP32
-// Two FP32 values in one 64-bit register (first value in the low half),
-// operated on by the paired FP32 instructions (add/sub/mul/fma .f32x2), each
-// element rounded to nearest as by the scalar instruction.
-__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(uint64_t x, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_sub(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-// a * b + c, one rounding per element
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-// 1/x of both elements: the hardware approximation (rcp.approx, at most one
-// ulp from the exact reciprocal).
-__device__ __forceinline__ uint64_t f2_recip(uint64_t x) {
-  float x0, x1, r0, r1;
-  f2_unpack(x, x0, x1);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x0));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(x1));
-  return f2_pack(r0, r1);
-}
-
-// 1/x of both elements: the hardware approximation refined by one
-// Newton-Raphson step r' = r + r (1 - x r), as recip_nr.
-__device__ __forceinline__ uint64_t f2_recip_nr(uint64_t x) {
-  float x0, x1, r0, r1;
-  f2_unpack(x, x0, x1);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x0));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(x1));
-  const uint64_t r = f2_pack(r0, r1);
-  const uint64_t e = f2_fma(f2_sub(0ull, x), r, f2_pack(1.f, 1.f));
-  return f2_fma(r, e, r);
-}
-
-// hi = {fp16(a sa), fp16(b sb)} and lo = the rounded remainders
-// {fp16(a sa - hi_a), fp16(b sb - hi_b)}, each as one 32-bit word with the
-// first value in the low half: split_f16 of the two scaled values, with the
-// FP32 arithmetic done on the pair at once.
-__device__ __forceinline__ void split_f16x2_scaled2(float a, float b, float sa, float sb,
-                                                    uint32_t& hi, uint32_t& lo) {
-  asm("{\n\t.reg .b64 x, y, r;\n\t.reg .f32 x0, x1, y0, y1, r0, r1;\n\t"
-      ".reg .b16 h0, h1;\n\t"
-      "mov.b64 x, {%2, %3};\n\t"
-      "mov.b64 y, {%4, %5};\n\t"
-      "mul.rn.f32x2 x, x, y;\n\t"
-      "mov.b64 {x0, x1}, x;\n\t"
-      "cvt.rn.f16x2.f32 %0, x1, x0;\n\t"
-      "mov.b32 {h0, h1}, %0;\n\t"
-      "cvt.f32.f16 y0, h0;\n\t"
-      "cvt.f32.f16 y1, h1;\n\t"
-      "mov.b64 y, {y0, y1};\n\t"
-      "sub.rn.f32x2 r, x, y;\n\t"
-      "mov.b64 {r0, r1}, r;\n\t"
-      "cvt.rn.f16x2.f32 %1, r1, r0;\n\t}"
-      : "=r"(hi), "=r"(lo)
-      : "f"(a), "f"(b), "f"(sa), "f"(sb));
-}
-// As split_f16x2_scaled2, but nlo holds the negated remainders
-// {fp16(hi_a - a sa), fp16(hi_b - b sb)}: each remainder is one
-// mixed-precision subtraction (FP16 minus FP32, rounded to FP32; exact here)
-// instead of a conversion back to FP32 and a subtraction.  Rounding to
-// nearest is symmetric, so nlo is exactly the negated lo of
-// split_f16x2_scaled2; an MMA that reads it sets its negate bit.
+// hi = {fp16(a sa), fp16(b sb)} and nlo = the negated rounded remainders
+// {fp16(hi_a - a sa), fp16(hi_b - b sb)}, each as one 32-bit word with the
+// first value in the low half: split_f16 of the two scaled values.  The
+// remainder is one mixed-precision subtraction (FP16 minus FP32, rounded to
+// FP32; exact here) instead of a conversion back to FP32 and a subtraction;
+// an MMA that reads it sets its negate bit.
 __device__ __forceinline__ void split_f16x2_neglo_scaled2(float a, float b, float sa, float sb,
                                                           uint32_t& hi, uint32_t& nlo) {
   asm("{\n\t.reg .b64 x, s;\n\t.reg .f32 x0, x1, r0, r1;\n\t"
@@ -338,10 +244,6 @@ __device__ __forceinline__ void split_f16x2_neglo(float a, float b, uint32_t& hi
 __device__ __forceinline__ void split_f16x2_neglo_scaled(float a, float b, float s, uint32_t& hi,
                                                          uint32_t& nlo) {
   split_f16x2_neglo_scaled2(a, b, s, s, hi, nlo);
-}
-__device__ __forceinline__ void split_f16x2_scaled(float a, float b, float s, uint32_t& hi,
-                                                   uint32_t& lo) {
-  split_f16x2_scaled2(a, b, s, s, hi, lo);
 }
 
 }  // namespace tc
