@@ -105,6 +105,12 @@ cudaError_t launch_solve_simt(const DevProblem& pb, const WorkQueue& q,
                               void* fields, int grid, cudaStream_t st,
                               int* steps_out = nullptr);
 cudaError_t setup_solve_simt(int dim, int max_n, bool steady = false);
+// FP64 solves on the interval (rd_solve_1d.cu), reached through the above.
+cudaError_t setup_solve_1d(int max_n);
+int grid_solve_1d(int max_n, int n_sm);
+cudaError_t launch_solve_1d(const DevProblem& pb, const WorkQueue& q, const double* theta,
+                            double* phi, uint32_t* status, void* fields, int grid,
+                            cudaStream_t st, int* steps_out);
 // Tensor-core solve (rd_solve_tc2.cu): every size in its queue must be the same
 // N x N grid, N a multiple of 16 up to 128.
 cudaError_t setup_solve_tc(int n);
