@@ -6,12 +6,19 @@
 // master weights, Adam with decoupled weight decay, and the output mapped to
 // a log-likelihood by Phi~ = floor + exp(shift + scale * net(x)).
 //
-// GEMM kernel: D[M][N] = sum_k A[m][k] B[n][k] for one 128-row tile of M and
-// all N <= 256 columns per CTA; K is staged 64 at a time into 128B-swizzled
-// shared memory (K-major or MN-major per operand, matching how the operand is
-// stored in global memory), one thread issues the M=128 kind::f16 MMAs (BF16
-// inputs, FP32 accumulator in TMEM) and four warps run the fused epilogue
-// (bias + SiLU, SiLU', or a plain FP32 store) from TMEM.
+// Forward and backward are row-local, so one kernel (k_mlp) takes a tile of 128
+// rows through all layers: weights stream into shared memory (128B-swizzled,
+// cp.async), each layer is M = 128, N = 256 kind::f16 MMAs (BF16 inputs, FP32
+// accumulator in TMEM) issued by one thread, and 16 warps run the bias + SiLU
+// (or SiLU') epilogue from TMEM straight into the next layer's operand tile.
+// Only the weight gradients sum over rows: k_mlp_wgrad forms them per layer,
+// half of the outputs and a share of the row tiles, k_mlp_reduce adds the
+// shares in a fixed order.  Measured (GB300): Phi~ of 4096 rows 375 ->
+// 36 us (a kernel per layer, one thread writing a row of
+// pre-activations nobody read); loss and gradients of 1024 rows 1020 ->
+// 118 us (column sums ran over the rows in one thread per column).
+// What is left is latency: one tile per SM, its weights' way from L2, and the
+// epilogues' 16 instructions per value.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -31,10 +38,9 @@ namespace mlp {
 using namespace tc;
 
 constexpr int kIn = 16;        // padded input features
-constexpr int kGemmThreads = 128;
-constexpr int kKChunk = 64;    // K elements staged per round (one 128-byte swizzle atom)
-
-enum Epi { EPI_FWD_SILU = 0, EPI_BWD_SILU = 1, EPI_F32 = 2 };
+constexpr int kW = RD_SURROGATE_WIDTH;  // 256
+constexpr int kMlpThreads = 512;
+constexpr int kMaxSplits = 16;  // row shares of the weight gradients
 
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 D.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int a_mn, int b_mn) {
@@ -48,127 +54,463 @@ __device__ __forceinline__ float silu_grad(float z) {
   return s * (1.f + z * (1.f - s));
 }
 
-struct GemmArgs {
-  int M, N, K;
-  const __nv_bfloat16* A;  // K-major: A[m * lda + k]; MN-major: A[k * lda + m]
-  int lda;
-  const __nv_bfloat16* B;  // K-major: B[n * ldb + k]; MN-major: B[k * ldb + n]
-  int ldb;
-  const float* bias;       // EPI_FWD_SILU: [N]
-  const float* zprev;      // EPI_BWD_SILU: [M][N] pre-activations
-  float* out_f32;          // EPI_FWD_SILU: Z [M][N]; EPI_F32: D [M][N]
-  __nv_bfloat16* out_bf16; // EPI_FWD_SILU: SiLU(Z); EPI_BWD_SILU: dZ
+struct Norm {
+  double in_mu[RD_NPARAM], in_sd[RD_NPARAM];
+  double floor, shift, scale;
+};
+
+// FP32 parameter layout: W1 [W][16], b1 [W], W2 [W][W], b2, W3 [W][W], b3, W4 [W], b4 [1].
+struct Layout {
+  int W;
+  size_t oW1, ob1, oW2, ob2, oW3, ob3, oW4, ob4, total;
+  __host__ __device__ constexpr explicit Layout(int w)
+      : W(w),
+        oW1(0),
+        ob1((size_t)w * kIn),
+        oW2(ob1 + w),
+        ob2(oW2 + (size_t)w * w),
+        oW3(ob2 + w),
+        ob3(oW3 + (size_t)w * w),
+        oW4(ob3 + w),
+        ob4(oW4 + w),
+        total(ob4 + 1) {}
+  __host__ __device__ constexpr size_t stride() const { return (total + 3) / 4 * 4; }
+};
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Copies rows x cols of a row-major BF16 matrix (16-byte aligned rows) into a
+// 128B-swizzled tile, asynchronously; rows from rows_valid on become zero.
+template <int COLS>
+__device__ __forceinline__ void load_tile(uint8_t* tile, const __nv_bfloat16* g, int ld, int rows,
+                                          int rows_valid) {
+  constexpr int PER = COLS / 8;
+  const uint32_t base = smem_u32(tile);
+  for (int i = threadIdx.x; i < rows * PER; i += kMlpThreads) {
+    const int r = i / PER, c = (i % PER) * 8;
+    const uint32_t off = sw128_offset(rows, r, c);
+    if (r < rows_valid)
+      cp_async16(base + off, g + (size_t)r * ld + c);
+    else
+      *reinterpret_cast<uint4*>(tile + off) = make_uint4(0, 0, 0, 0);
+  }
+}
+
+struct MlpArgs {
+  int B;
+  const __nv_bfloat16* X;   // [B][16]
+  const __nv_bfloat16* Wb;  // BF16 weights in the parameter layout
+  const float* params;
+  Norm nm;
+  double* phit;             // MLP_PREDICT: [B]
+  const float* target;      // else: [B]
+  float* out;               // else: [B]
+  double* sq_err;           // else: summed
+  // MLP_GRAD
+  __nv_bfloat16 *H1, *H2, *dZ1, *dZ2, *dZ3;  // [B][W]
+  float* Z1;                                 // [B][W]
+  float* part4;             // [tile][W + 1]: shares of dW4, db4
   int* err;
 };
 
-// Stages rows [0, rows) x K columns [k0, k0 + kc) of a K-major matrix into a
-// 128B-swizzled tile with `rows` rows (columns beyond kc are zero).
-__device__ __forceinline__ void stage_kmajor(uint8_t* tile, const __nv_bfloat16* g, int ld,
-                                             int rows, int row0, int rows_valid, int k0, int kc) {
-  for (int i = threadIdx.x; i < rows * 8; i += kGemmThreads) {
-    const int r = i >> 3, c8 = (i & 7) * 8;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (r < rows_valid && c8 < kc)
-      v = *reinterpret_cast<const uint4*>(g + (size_t)(row0 + r) * ld + k0 + c8);
-    *reinterpret_cast<uint4*>(tile + sw128_offset(rows, r, c8)) = v;
+enum { MLP_PREDICT = 0, MLP_LOSS = 1, MLP_GRAD = 2 };
+
+struct MlpCtrl {
+  uint64_t bar;
+  uint32_t tmem_base;
+  int abort;
+  float bias[3][kW];
+  float w4[kW];
+  float out[128];
+  float dout[128];
+  float acc4[2][kW];
+};
+constexpr uint32_t kMlpTileA = 128 * kW * 2;  // 64 KB: activations, one 128-row tile
+constexpr uint32_t kMlpTileW = kW * kW * 2;   // 128 KB: one layer's weights
+constexpr uint32_t kMlpSmem = 1024 + kMlpTileA + kMlpTileW + sizeof(MlpCtrl);
+
+// K = 16 kk MMAs of D[128][256] (+)= A B^T; a_mn / b_mn: operand stored with K
+// along the rows; a_rows / b_rows: rows of the operand's tile.
+template <int KK, int A_MN, int B_MN>
+__device__ __forceinline__ void issue_layer(uint32_t d, uint32_t ta, int a_rows, uint32_t tb,
+                                            int b_rows, int n) {
+  const uint32_t idesc = idesc_bf16(128, n, A_MN, B_MN);
+  const uint64_t ad = sdesc_sw128(ta, A_MN ? (uint32_t)a_rows * 128u : 16u, 1024u);
+  const uint64_t bd = sdesc_sw128(tb, B_MN ? (uint32_t)b_rows * 128u : 16u, 1024u);
+#pragma unroll
+  for (int kk = 0; kk < KK; ++kk) {
+    const uint32_t oa = A_MN ? kk * 2048u : (uint32_t)(kk >> 2) * a_rows * 128u + (kk & 3) * 32u;
+    const uint32_t ob = B_MN ? kk * 2048u : (uint32_t)(kk >> 2) * b_rows * 128u + (kk & 3) * 32u;
+    mma_f16(d, ad + (oa >> 4), bd + (ob >> 4), idesc, kk > 0 ? 1u : 0u);
   }
 }
 
-// Stages K rows [k0, k0 + kc) x MN columns [mn0, mn0 + cols) of an MN-major
-// matrix (g[k * ld + mn]) into a swizzled tile of 64 K rows (rows beyond kc
-// are zero).
-__device__ __forceinline__ void stage_mnmajor(uint8_t* tile, const __nv_bfloat16* g, int ld,
-                                              int cols, int mn0, int k0, int kc) {
-  const int per_row = cols / 8;
-  for (int i = threadIdx.x; i < kKChunk * per_row; i += kGemmThreads) {
-    const int r = i / per_row, c8 = (i - r * per_row) * 8;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (r < kc) v = *reinterpret_cast<const uint4*>(g + (size_t)(k0 + r) * ld + mn0 + c8);
-    *reinterpret_cast<uint4*>(tile + sw128_offset(kKChunk, r, c8)) = v;
+__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
+  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// f(column, 16 accumulator values, 16 results): this thread's 64 columns of one
+// row, results as BF16 into the operand tile and, if g is not null, global row g.
+template <class F>
+__device__ __forceinline__ void epilogue(uint32_t t, uint8_t* tile, int row, int c0,
+                                         __nv_bfloat16* g, F&& f) {
+#pragma unroll 1
+  for (int c = c0; c < c0 + 64; c += 16) {
+    float v[16];
+    __nv_bfloat16 h[16];
+    __syncwarp();
+    tmem_ld16(t + (uint32_t)c, v);
+    tmem_wait_ld();
+    f(c, v, h);
+#pragma unroll
+    for (int k = 0; k < 16; k += 8) {
+      const uint4 q = make_uint4(pack_bf16(h[k], h[k + 1]), pack_bf16(h[k + 2], h[k + 3]),
+                                 pack_bf16(h[k + 4], h[k + 5]), pack_bf16(h[k + 6], h[k + 7]));
+      *reinterpret_cast<uint4*>(tile + sw128_offset(128, row, c + k)) = q;
+      if (g) *reinterpret_cast<uint4*>(g + c + k) = q;
+    }
   }
 }
 
-template <int EPI, int A_MN, int B_MN>
-__global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(GemmArgs g) {
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* ta = base;                 // A tile: 128 x 64 (16 KB)
-  uint8_t* tb = base + 16384;         // B tile: up to 256 x 64 (32 KB)
+template <int MODE>
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ MlpArgs a) {
+  extern __shared__ uint8_t mlp_smem[];
+  uint8_t* const base = mlp_smem + ((1024u - (smem_u32(mlp_smem) & 1023u)) & 1023u);
+  uint8_t* const ta = base;
+  uint8_t* const tw = base + kMlpTileA;
+  MlpCtrl* const ctl = reinterpret_cast<MlpCtrl*>(base + kMlpTileA + kMlpTileW);
+  constexpr Layout L(kW);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int row0 = blockIdx.x * 128, valid = min(128, a.B - row0);
+  const int row = 32 * (warp & 3) + lane, c0 = 64 * (warp >> 2);
+  const bool mine = row < valid;
+  // layer 1's operands, then layer 2's weights behind its bytes
+  uint8_t* const tw1 = tw + kMlpTileW - 32768;  // the last 64-column block of the weights
+  load_tile<kIn>(ta, a.X + (size_t)row0 * kIn, kIn, 128, valid);
+  load_tile<kIn>(tw1, a.Wb + L.oW1, kIn, kW, kW);
+  cp_async_commit();
+  // columns 0..191 of W2 now, the last 64 once layer 1 has read its weights there
+  auto load_w_cols = [&](const __nv_bfloat16* w, int b0, int b1) {
+    const uint32_t tb = smem_u32(tw);
+    const int per = 8 * (b1 - b0);
+    for (int i = tid; i < kW * per; i += kMlpThreads) {
+      const int r = i / per, c = (i - r * per + 8 * b0) * 8;
+      cp_async16(tb + sw128_offset(kW, r, c), w + (size_t)r * kW + c);
+    }
+    cp_async_commit();
+  };
+  load_w_cols(a.Wb + L.oW2, 0, 3);
+  for (int i = tid; i < kW; i += kMlpThreads) {
+    ctl->bias[0][i] = a.params[L.ob1 + i];
+    ctl->bias[1][i] = a.params[L.ob2 + i];
+    ctl->bias[2][i] = a.params[L.ob3 + i];
+    ctl->w4[i] = a.params[L.oW4 + i];
+  }
+  if (warp == 0) {
+    tmem_alloc(&ctl->tmem_base, 512);
+    tmem_relinquish();
+  }
+  if (tid == 0) {
+    mbar_init(&ctl->bar, 1);
+    ctl->abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  cp_async_wait<1>();
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = ctl->tmem_base;
+  const uint32_t d0 = tmem, d1 = tmem + 256u;  // accumulators
+  const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+  const uint32_t sa = smem_u32(ta), sw = smem_u32(tw);
+  uint32_t phase = 0;
+  // waits for the MMAs issued since the last wait (a wait that gives up leaves
+  // wrong values and raises the error flag at the end)
+  auto done = [&]() {
+    mbar_wait_bounded(&ctl->bar, phase & 1u, &ctl->abort);
+    ++phase;
+    tc_fence_after();
+  };
+  auto operands_ready = [&]() {
+    fence_proxy_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  };
+  // ---- layer 1 -> d0
+  if (tid == 0) {
+    issue_layer<1, 0, 0>(d0, sa, 128, smem_u32(tw1), kW, kW);
+    mma_commit(&ctl->bar);
+  }
+  __syncwarp();
+  done();
+  load_w_cols(a.Wb + L.oW2, 3, 4);
+  auto silu_epilogue = [&](uint32_t d, int layer, __nv_bfloat16* h_out, float* z_out) {
+    epilogue(d + lane_off, ta, row, c0, (h_out && mine) ? h_out + (size_t)(row0 + row) * kW : nullptr,
+             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+#pragma unroll
+               for (int j = 0; j < 16; ++j) {
+                 v[j] += ctl->bias[layer][c + j];
+                 h[j] = __float2bfloat16_rn(silu(v[j]));
+               }
+               if (z_out && mine) {
+                 float4* z = reinterpret_cast<float4*>(z_out + (size_t)(row0 + row) * kW + c);
+#pragma unroll
+                 for (int j = 0; j < 4; ++j)
+                   z[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+               }
+             });
+  };
+  silu_epilogue(d0, 0, MODE == MLP_GRAD ? a.H1 : nullptr, MODE == MLP_GRAD ? a.Z1 : nullptr);
+  cp_async_wait<0>();
+  operands_ready();
+  // ---- layer 2 -> d1
+  if (tid == 0) {
+    issue_layer<16, 0, 0>(d1, sa, 128, sw, kW, kW);
+    mma_commit(&ctl->bar);
+  }
+  __syncwarp();
+  done();
+  load_w_cols(a.Wb + L.oW3, 0, 4);
+  silu_epilogue(d1, 1, MODE == MLP_GRAD ? a.H2 : nullptr, nullptr);
+  cp_async_wait<0>();
+  operands_ready();
+  // ---- layer 3 -> d0
+  if (tid == 0) {
+    issue_layer<16, 0, 0>(d0, sa, 128, sw, kW, kW);
+    mma_commit(&ctl->bar);
+  }
+  __syncwarp();
+  done();
+  silu_epilogue(d0, 2, nullptr, nullptr);
+  __syncthreads();
+  // ---- head: out[b] = sum_j H3[b][j] W4[j] + b4, one warp per row
+#pragma unroll 1
+  for (int r = warp; r < valid; r += kMlpThreads / 32) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < kW / 32; ++i) {
+      const int j = lane + 32 * i;
+      const __nv_bfloat16 h =
+          *reinterpret_cast<const __nv_bfloat16*>(ta + sw128_offset(128, r, j));
+      s += __bfloat162float(h) * ctl->w4[j];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) ctl->out[r] = s + a.params[L.ob4];
+  }
+  __syncthreads();
+  if (MODE == MLP_PREDICT) {
+    if (tid < valid)
+      a.phit[row0 + tid] = a.nm.floor + exp(a.nm.shift + a.nm.scale * (double)ctl->out[tid]);
+  } else {
+    if (tid < 128) {
+      double e2 = 0.0;
+      if (tid < valid) {
+        const float y = ctl->out[tid];
+        const float e = y - a.target[row0 + tid];
+        a.out[row0 + tid] = y;
+        ctl->dout[tid] = 2.f * e / (float)a.B;
+        e2 = (double)e * (double)e;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+      if (lane == 0) atomicAdd(a.sq_err, e2);
+    }
+    __syncthreads();
+  }
+  if (MODE == MLP_GRAD) {
+    // shares of dW4 and db4 over the tile's rows (valid = 128)
+    {
+      const int j = tid & (kW - 1), hlf = tid / kW;
+      float s = 0.f;
+      for (int r = 64 * hlf; r < 64 * hlf + 64; ++r)
+        s += ctl->dout[r] *
+             __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(ta + sw128_offset(128, r, j)));
+      ctl->acc4[hlf][j] = s;
+      __syncthreads();
+      float* p4 = a.part4 + (size_t)blockIdx.x * (kW + 1);
+      if (tid < kW) p4[tid] = ctl->acc4[0][tid] + ctl->acc4[1][tid];
+      if (tid == 0) {
+        float t = 0.f;
+        for (int r = 0; r < 128; ++r) t += ctl->dout[r];
+        p4[kW] = t;
+      }
+    }
+    // ---- dZ3 = dout W4 o SiLU'(Z3), Z3 still in d0
+    const float dout = ctl->dout[row];
+    epilogue(d0 + lane_off, ta, row, c0, a.dZ3 + (size_t)(row0 + row) * kW,
+             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+#pragma unroll
+               for (int j = 0; j < 16; ++j)
+                 h[j] = __float2bfloat16_rn(dout * ctl->w4[c + j] *
+                                            silu_grad(v[j] + ctl->bias[2][c + j]));
+             });
+    operands_ready();
+    // ---- dH2 = dZ3 W3 -> d0; dZ2 = dH2 o SiLU'(Z2), Z2 in d1
+    if (tid == 0) {
+      issue_layer<16, 0, 1>(d0, sa, 128, sw, kW, kW);
+      mma_commit(&ctl->bar);
+    }
+    __syncwarp();
+    done();
+    load_w_cols(a.Wb + L.oW2, 0, 4);
+    epilogue(d0 + lane_off, ta, row, c0, a.dZ2 + (size_t)(row0 + row) * kW,
+             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+               float z[16];
+               tmem_ld16(d1 + lane_off + (uint32_t)c, z);
+               tmem_wait_ld();
+#pragma unroll
+               for (int j = 0; j < 16; ++j)
+                 h[j] = __float2bfloat16_rn(v[j] * silu_grad(z[j] + ctl->bias[1][c + j]));
+             });
+    cp_async_wait<0>();
+    operands_ready();
+    // ---- dH1 = dZ2 W2 -> d0; dZ1 = dH1 o SiLU'(Z1)
+    if (tid == 0) {
+      issue_layer<16, 0, 1>(d0, sa, 128, sw, kW, kW);
+      mma_commit(&ctl->bar);
+    }
+    __syncwarp();
+    done();
+    epilogue(d0 + lane_off, ta, row, c0, a.dZ1 + (size_t)(row0 + row) * kW,
+             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+               const float4* z4 =
+                   reinterpret_cast<const float4*>(a.Z1 + (size_t)(row0 + row) * kW + c);
+#pragma unroll
+               for (int j = 0; j < 4; ++j) {
+                 const float4 z = z4[j];
+                 h[4 * j] = __float2bfloat16_rn(v[4 * j] * silu_grad(z.x));
+                 h[4 * j + 1] = __float2bfloat16_rn(v[4 * j + 1] * silu_grad(z.y));
+                 h[4 * j + 2] = __float2bfloat16_rn(v[4 * j + 2] * silu_grad(z.z));
+                 h[4 * j + 3] = __float2bfloat16_rn(v[4 * j + 3] * silu_grad(z.w));
+               }
+             });
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+  if (tid == 0 && ctl->abort) atomicOr(a.err, 1);
+}
+
+// Weight and bias gradients dW_l = dZ_l^T H_{l-1}, db_l = column sums of dZ_l:
+// block (x = outputs 128 x .. 128 x + 127, y = layer, z = share of the row
+// tiles), into that share's copy of the parameter layout.
+struct WgradArgs {
+  int tiles, splits;
+  const __nv_bfloat16* dZ[3];
+  const __nv_bfloat16* H[3];
+  float* part;  // [splits][stride()]
+  int* err;
+};
+constexpr uint32_t kWgTileA = 128 * 128 * 2, kWgTileB = 128 * kW * 2;
+constexpr uint32_t kWgSmem = 1024 + 2 * (kWgTileA + kWgTileB) + 4 * 128 * 4;
+
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_constant__ WgradArgs a) {
+  extern __shared__ uint8_t wg_smem[];
+  uint8_t* const base = wg_smem + ((1024u - (smem_u32(wg_smem) & 1023u)) & 1023u);
+  float* const sums = reinterpret_cast<float*>(base + 2 * (kWgTileA + kWgTileB));  // [4][128]
   __shared__ uint64_t bar;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * 128;
-  const int N = g.N;
+  constexpr Layout L(kW);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int layer = blockIdx.y, m0 = 128 * blockIdx.x, share = blockIdx.z;
+  const int n = layer == 0 ? kIn : kW;
+  const __nv_bfloat16* dz = a.dZ[layer] + m0;
+  const __nv_bfloat16* hh = a.H[layer];
+  const int t0 = (int)((long long)a.tiles * share / a.splits);
+  const int t1 = (int)((long long)a.tiles * (share + 1) / a.splits);
   if (warp == 0) {
     tmem_alloc(&tmem_base, 256);
     tmem_relinquish();
   }
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     mbar_init(&bar, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  auto load = [&](int t) {
+    uint8_t* s = base + (uint32_t)(t & 1) * (kWgTileA + kWgTileB);
+    load_tile<128>(s, dz + (size_t)t * 128 * kW, kW, 128, 128);
+    if (layer == 0)
+      load_tile<kIn>(s + kWgTileA, hh + (size_t)t * 128 * kIn, kIn, 128, 128);
+    else
+      load_tile<kW>(s + kWgTileA, hh + (size_t)t * 128 * kW, kW, 128, 128);
+    cp_async_commit();
+  };
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base;
-  const uint32_t idesc = idesc_bf16(128, N, A_MN, B_MN);
+  const uint32_t idesc = idesc_bf16(128, n, 1, 1);
+  const int col = tid & 127, quarter = tid >> 7;
+  float colsum = 0.f;
   uint32_t phase = 0;
   bool ok = true;
-  for (int k0 = 0; k0 < g.K && ok; k0 += kKChunk) {
-    const int kc = min(kKChunk, g.K - k0);
-    if (A_MN)
-      stage_mnmajor(ta, g.A, g.lda, 128, m0, k0, kc);
-    else
-      stage_kmajor(ta, g.A, g.lda, 128, m0, g.M - m0, k0, kc);
-    if (B_MN)
-      stage_mnmajor(tb, g.B, g.ldb, N, 0, k0, kc);
-    else
-      stage_kmajor(tb, g.B, g.ldb, N, 0, N, k0, kc);
+  load(t0);
+  for (int t = t0; t < t1; ++t) {
+    uint8_t* s = base + (uint32_t)(t & 1) * (kWgTileA + kWgTileB);
+    if (t > t0) {  // the other buffer's MMAs are done: it may be refilled
+      ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag) && ok;
+      ++phase;
+      tc_fence_after();
+    }
+    cp_async_wait<0>();
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {
-      tc_fence_after();
-      const uint64_t ad = sdesc_sw128(smem_u32(ta), A_MN ? 128u * 64u : 16u, 1024u);
-      const uint64_t bd = sdesc_sw128(smem_u32(tb), B_MN ? 128u * 64u : 16u, 1024u);
-      for (int kk = 0; kk < kc / 16; ++kk) {
-        const uint64_t off = (uint64_t)(A_MN ? kk * 2048 : kk * 32) >> 4;
-        const uint64_t offb = (uint64_t)(B_MN ? kk * 2048 : kk * 32) >> 4;
-        mma_f16(tmem, ad + off, bd + offb, idesc, (k0 > 0 || kk > 0) ? 1u : 0u);
-      }
+    tc_fence_after();
+    if (tid == 0) {
+      const uint64_t ad = sdesc_sw128(smem_u32(s), 128u * 128u, 1024u);
+      const uint64_t bd = sdesc_sw128(smem_u32(s + kWgTileA), 128u * 128u, 1024u);
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk)
+        mma_f16(tmem, ad + (kk * 2048u >> 4), bd + (kk * 2048u >> 4), idesc,
+                (t > t0 || kk > 0) ? 1u : 0u);
       mma_commit(&bar);
     }
-    // the tiles are overwritten next round: wait for the MMAs to finish
-    ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag);
-    ++phase;
-    tc_fence_after();
-    __syncthreads();
+    __syncwarp();
+    if (t + 1 < t1) load(t + 1);
+#pragma unroll 8
+    for (int r = 32 * quarter; r < 32 * quarter + 32; ++r)
+      colsum += __bfloat162float(
+          *reinterpret_cast<const __nv_bfloat16*>(s + sw128_offset(128, r, col)));
   }
+  ok = ok && mbar_wait_bounded(&bar, phase & 1u, &abort_flag);
+  tc_fence_after();
+  sums[tid] = colsum;
+  __syncthreads();
+  const size_t oW[3] = {L.oW1, L.oW2, L.oW3}, ob[3] = {L.ob1, L.ob2, L.ob3};
+  float* part = a.part + (size_t)share * L.stride();
+  if (tid < 128)
+    part[ob[layer] + m0 + tid] =
+        (sums[tid] + sums[128 + tid]) + (sums[256 + tid] + sums[384 + tid]);
   if (ok) {
-    const int m = m0 + 32 * warp + lane;  // TMEM lane = row of the tile
-    const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
-    for (int n0 = 0; n0 < N; n0 += 8) {
-      float v[8];
+    const int m = m0 + 32 * (warp & 3) + lane;  // TMEM lane = output
+    const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    float* dst = part + oW[layer] + (size_t)m * n;
+    for (int c = 16 * (warp >> 2); c < n; c += 64) {
+      float v[16];
       __syncwarp();
-      tmem_ld8(trow + (uint32_t)n0, v);
+      tmem_ld16(trow + (uint32_t)c, v);
       tmem_wait_ld();
-      if (m >= g.M) continue;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const size_t o = (size_t)m * N + n0 + j;
-        if (EPI == EPI_FWD_SILU) {
-          const float z = v[j] + g.bias[n0 + j];
-          g.out_f32[o] = z;
-          g.out_bf16[o] = __float2bfloat16_rn(silu(z));
-        } else if (EPI == EPI_BWD_SILU) {
-          g.out_bf16[o] = __float2bfloat16_rn(v[j] * silu_grad(g.zprev[o]));
-        } else {
-          g.out_f32[o] = v[j];
-        }
-      }
+      for (int j = 0; j < 16; j += 4)
+        *reinterpret_cast<float4*>(dst + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
     }
   }
   tc_fence_before();
@@ -177,103 +519,43 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_gemm_bf16(GemmArgs g) {
     tc_fence_after();
     tmem_dealloc(tmem, 256);
   }
-  if (threadIdx.x == 0 && abort_flag) atomicOr(g.err, 1);
+  if (tid == 0 && abort_flag) atomicOr(a.err, 1);
 }
 
-// The tiles need 49 KB; asking for 100 KB keeps at most two CTAs (two
-// 256-column TMEM allocations) on an SM, so an allocation never waits.
-constexpr size_t kGemmSmem = 100 * 1024;
-
-template <int EPI, int A_MN, int B_MN>
-static cudaError_t gemm(const GemmArgs& a, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_bf16<EPI, A_MN, B_MN>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kGemmSmem);
-    if (e != cudaSuccess) return e;
-    configured = true;
+// grads = the shares' sum, in share (row tile) order.
+__global__ void k_mlp_reduce(int splits, int tiles, const float* part, const float* part4,
+                             float* grads) {
+  constexpr Layout L(kW);
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= L.total) return;
+  float s = 0.f;
+  if (i < L.oW4) {
+#pragma unroll 4
+    for (int k = 0; k < splits; ++k) s += part[(size_t)k * L.stride() + i];
+  } else {
+#pragma unroll 4
+    for (int k = 0; k < tiles; ++k) s += part4[(size_t)k * (kW + 1) + (i - L.oW4)];
   }
-  k_gemm_bf16<EPI, A_MN, B_MN><<<(a.M + 127) / 128, kGemmThreads, kGemmSmem, st>>>(a);
-  return cudaGetLastError();
+  grads[i] = s;
 }
 
 // ---------------------------------------------------------------------------
 // Small CUDA-core kernels
 // ---------------------------------------------------------------------------
-struct Norm {
-  double in_mu[RD_NPARAM], in_sd[RD_NPARAM];
-  double floor, shift, scale;
-};
-
-// Features x_i = (log theta_i - mu_i) / s_i as BF16, zero-padded to 16.
-__global__ void k_features(int B, int P, const double* theta, Norm nm, __nv_bfloat16* X) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  for (int j = 0; j < kIn; ++j) {
-    float v = 0.f;
-    if (j < P) {
-      const double t = theta[(size_t)b * P + j];
-      v = (float)((log(t > 0.0 ? t : 1e-300) - nm.in_mu[j]) / nm.in_sd[j]);
-    }
-    X[(size_t)b * kIn + j] = __float2bfloat16_rn(v);
-  }
-}
-
-// Last layer out[b] = sum_j H3[b][j] W4[j] + b4 (FP32), one warp per row; with
-// a target, also dOut[b] = 2 (out - z) / B and the squared error.
-__global__ void k_head_fwd(int B, int W, const __nv_bfloat16* H3, const float* W4,
-                           const float* b4, float* out, const float* target, float* dout,
+// Features x_i = (log theta_i - mu_i) / s_i as BF16, zero-padded to 16, one
+// thread per inferred parameter: the FP64 logarithms are what this costs, so no
+// lane of a warp is spent on padding.  Also clears the squared error's sum.
+__global__ void k_features(int B, int P, const double* theta, Norm nm, __nv_bfloat16* X,
                            double* sq_err) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= B) return;
-  float s = 0.f;
-  for (int j = lane; j < W; j += 32) s += __bfloat162float(H3[(size_t)warp * W + j]) * W4[j];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) {
-    const float y = s + b4[0];
-    out[warp] = y;
-    if (target) {
-      const float e = y - target[warp];
-      dout[warp] = 2.f * e / (float)B;
-      atomicAdd(sq_err, (double)e * (double)e);
-    }
-  }
-}
-
-// dZ3[b][j] = dOut[b] W4[j] SiLU'(Z3[b][j]) (BF16)
-__global__ void k_head_bwd(int B, int W, const float* dout, const float* W4, const float* Z3,
-                           __nv_bfloat16* dZ3) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)B * W) return;
-  const int b = (int)(i / W), j = (int)(i - (size_t)b * W);
-  dZ3[i] = __float2bfloat16_rn(dout[b] * W4[j] * silu_grad(Z3[i]));
-}
-
-// Column sums: g[j] = sum_b D[b][j] for a BF16 (dZ) or FP32 matrix, and for
-// the head dW4[j] = sum_b dOut[b] H3[b][j], db4 = sum_b dOut[b].
-__global__ void k_colsum_bf16(int B, int W, const __nv_bfloat16* D, float* g) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= W) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += __bfloat162float(D[(size_t)b * W + j]);
-  g[j] = s;
-}
-
-__global__ void k_head_wgrad(int B, int W, const float* dout, const __nv_bfloat16* H3, float* gW4,
-                             float* gb4) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < W) {
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += dout[b] * __bfloat162float(H3[(size_t)b * W + j]);
-    gW4[j] = s;
-  }
-  if (j == 0) {
-    float s = 0.f;
-    for (int b = 0; b < B; ++b) s += dout[b];
-    gb4[0] = s;
-  }
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && sq_err) *sq_err = 0.0;
+  if (i >= B * P) return;
+  const int b = i / P, j = i - b * P;
+  const double t = theta[i];
+  const float v = (float)((log(t > 0.0 ? t : 1e-300) - nm.in_mu[j]) / nm.in_sd[j]);
+  __nv_bfloat16* x = X + (size_t)b * kIn;
+  x[j] = __float2bfloat16_rn(v);
+  for (int k = P + j; k < kIn; k += P) x[k] = __float2bfloat16_rn(0.f);
 }
 
 // Adam with bias correction and decoupled weight decay on the weights (mask
@@ -304,41 +586,12 @@ __global__ void k_to_bf16(int n, const float* src, __nv_bfloat16* dst) {
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
 }
 
-// Phi~ = floor + exp(shift + scale * out) in FP64.
-__global__ void k_output(int B, const float* out, Norm nm, double* phit) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) phit[b] = nm.floor + exp(nm.shift + nm.scale * (double)out[b]);
-}
-
 }  // namespace mlp
 }  // namespace rd
 
 // ---------------------------------------------------------------------------
 // Host side: the surrogate object, forward/backward, training, prediction
 // ---------------------------------------------------------------------------
-namespace rd {
-namespace mlp {
-
-// FP32 parameter layout: W1 [W][16], b1 [W], W2 [W][W], b2, W3 [W][W], b3, W4 [W], b4 [1].
-struct Layout {
-  int W;
-  size_t oW1, ob1, oW2, ob2, oW3, ob3, oW4, ob4, total;
-  explicit Layout(int w) : W(w) {
-    oW1 = 0;
-    ob1 = oW1 + (size_t)W * kIn;
-    oW2 = ob1 + W;
-    ob2 = oW2 + (size_t)W * W;
-    oW3 = ob2 + W;
-    ob3 = oW3 + (size_t)W * W;
-    oW4 = ob3 + W;
-    ob4 = oW4 + W;
-    total = ob4 + 1;
-  }
-};
-
-}  // namespace mlp
-}  // namespace rd
-
 struct rd_surrogate {
   rd_problem* pb = nullptr;
   int P = 0;
@@ -353,54 +606,74 @@ struct rd_surrogate {
   int adam_t = 0;
   // activations for up to `cap` rows
   int cap = 0;
-  __nv_bfloat16 *X = nullptr, *H1 = nullptr, *H2 = nullptr, *H3 = nullptr;
-  __nv_bfloat16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr, *out = nullptr, *dout = nullptr,
-        *target = nullptr;
+  __nv_bfloat16* X = nullptr;
+  float *out = nullptr, *target = nullptr;
   double* sqerr = nullptr;
+  // the backward pass's, for up to `grad_cap` rows
+  int grad_cap = 0;
+  __nv_bfloat16 *H1 = nullptr, *H2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
+  float *Z1 = nullptr, *part = nullptr, *part4 = nullptr;
 };
 
 namespace rd {
 namespace mlp {
 
 static void free_acts(rd_surrogate* s) {
-  void* ptrs[] = {s->X, s->H1, s->H2, s->H3, s->dZ1, s->dZ2, s->dZ3, s->Z1,
-                  s->Z2, s->Z3, s->out, s->dout, s->target, s->sqerr};
+  void* ptrs[] = {s->X, s->out, s->target, s->sqerr};
   for (void* p : ptrs) cudaFree(p);
-  s->X = s->H1 = s->H2 = s->H3 = s->dZ1 = s->dZ2 = s->dZ3 = nullptr;
-  s->Z1 = s->Z2 = s->Z3 = s->out = s->dout = s->target = nullptr;
+  s->X = nullptr;
+  s->out = s->target = nullptr;
   s->sqerr = nullptr;
   s->cap = 0;
 }
 
+static void free_grad(rd_surrogate* s) {
+  void* ptrs[] = {s->H1, s->H2, s->dZ1, s->dZ2, s->dZ3, s->Z1, s->part, s->part4};
+  for (void* p : ptrs) cudaFree(p);
+  s->H1 = s->H2 = s->dZ1 = s->dZ2 = s->dZ3 = nullptr;
+  s->Z1 = s->part = s->part4 = nullptr;
+  s->grad_cap = 0;
+}
+
+#define RD_ALLOC(ptr, bytes) \
+  if ((e = cudaMalloc(&(ptr), (bytes))) != cudaSuccess) return e;
+
+// Buffers of a forward pass over `rows` rows.
 cudaError_t ensure_rows(rd_surrogate* s, int rows) {
   if (rows <= s->cap) return cudaSuccess;
   cudaStreamSynchronize(s->pb->stream);
   free_acts(s);
-  const int cap = ((rows + 127) / 128) * 128;
-  const size_t W = (size_t)s->W;
+  const size_t cap = (size_t)((rows + 127) / 128) * 128;
   cudaError_t e;
-#define RD_ALLOC(ptr, bytes) \
-  if ((e = cudaMalloc(&(ptr), (bytes))) != cudaSuccess) return e;
   RD_ALLOC(s->X, sizeof(__nv_bfloat16) * cap * kIn);
+  RD_ALLOC(s->out, sizeof(float) * cap);
+  RD_ALLOC(s->target, sizeof(float) * cap);
+  RD_ALLOC(s->sqerr, sizeof(double));
+  s->cap = (int)cap;
+  s->pb->generation++;  // captured graphs may hold the old buffers
+  return cudaSuccess;
+}
+
+// And of a backward pass (rows a multiple of 128).
+static cudaError_t ensure_grad_rows(rd_surrogate* s, int rows) {
+  cudaError_t e = ensure_rows(s, rows);
+  if (e != cudaSuccess || rows <= s->grad_cap) return e;
+  cudaStreamSynchronize(s->pb->stream);
+  free_grad(s);
+  const size_t cap = (size_t)rows, W = (size_t)s->W;
+  const Layout L(s->W);
   RD_ALLOC(s->H1, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->H2, sizeof(__nv_bfloat16) * cap * W);
-  RD_ALLOC(s->H3, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->dZ1, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->dZ2, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->dZ3, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->Z1, sizeof(float) * cap * W);
-  RD_ALLOC(s->Z2, sizeof(float) * cap * W);
-  RD_ALLOC(s->Z3, sizeof(float) * cap * W);
-  RD_ALLOC(s->out, sizeof(float) * cap);
-  RD_ALLOC(s->dout, sizeof(float) * cap);
-  RD_ALLOC(s->target, sizeof(float) * cap);
-  RD_ALLOC(s->sqerr, sizeof(double));
-#undef RD_ALLOC
-  s->cap = cap;
-  s->pb->generation++;  // captured graphs may hold the old buffers
+  RD_ALLOC(s->part, sizeof(float) * kMaxSplits * L.stride());
+  RD_ALLOC(s->part4, sizeof(float) * (cap / 128) * (W + 1));
+  s->grad_cap = rows;
   return cudaSuccess;
 }
+#undef RD_ALLOC
 
 static cudaError_t refresh_bf16(rd_surrogate* s, cudaStream_t st) {
   const Layout L(s->W);
@@ -409,98 +682,72 @@ static cudaError_t refresh_bf16(rd_surrogate* s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-// Forward pass for B rows of theta (device [B][P]) into s->out; with a
-// target (device [B], normalised), also dOut and the summed squared error.
-cudaError_t forward(rd_surrogate* s, int B, const double* theta, bool with_target,
-                    cudaStream_t st) {
-  const Layout L(s->W);
-  const int W = s->W;
-  int* err = s->pb->ws.err;
-  k_features<<<(B + 127) / 128, 128, 0, st>>>(B, s->P, theta, s->norm, s->X);
-  GemmArgs g{};
-  g.err = err;
-  g.M = B;
-  g.N = W;
-  g.K = kIn;
-  g.A = s->X;
-  g.lda = kIn;
-  g.B = s->Wb + L.oW1;
-  g.ldb = kIn;
-  g.bias = s->params + L.ob1;
-  g.out_f32 = s->Z1;
-  g.out_bf16 = s->H1;
-  cudaError_t e = gemm<EPI_FWD_SILU, 0, 0>(g, st);
+template <int MODE>
+static cudaError_t launch_mlp(const MlpArgs& a, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_mlp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)kMlpSmem);
   if (e != cudaSuccess) return e;
-  g.K = W;
-  g.A = s->H1;
-  g.lda = W;
-  g.B = s->Wb + L.oW2;
-  g.ldb = W;
-  g.bias = s->params + L.ob2;
-  g.out_f32 = s->Z2;
-  g.out_bf16 = s->H2;
-  if ((e = gemm<EPI_FWD_SILU, 0, 0>(g, st)) != cudaSuccess) return e;
-  g.A = s->H2;
-  g.B = s->Wb + L.oW3;
-  g.bias = s->params + L.ob3;
-  g.out_f32 = s->Z3;
-  g.out_bf16 = s->H3;
-  if ((e = gemm<EPI_FWD_SILU, 0, 0>(g, st)) != cudaSuccess) return e;
-  if (with_target) {
-    if ((e = cudaMemsetAsync(s->sqerr, 0, sizeof(double), st)) != cudaSuccess) return e;
-  }
-  k_head_fwd<<<(B * 32 + 255) / 256, 256, 0, st>>>(
-      B, W, s->H3, s->params + L.oW4, s->params + L.ob4, s->out,
-      with_target ? s->target : nullptr, s->dout, s->sqerr);
+  k_mlp<MODE><<<(a.B + 127) / 128, kMlpThreads, kMlpSmem, st>>>(a);
   return cudaGetLastError();
 }
 
-// Backward pass of the mean-squared error after forward(with_target): all
-// parameter gradients into s->grads.
-cudaError_t backward(rd_surrogate* s, int B, cudaStream_t st) {
+// One pass over B rows of theta (device [B][P]): MLP_PREDICT writes Phi~ to
+// phit; MLP_LOSS writes s->out and the summed squared error against s->target;
+// MLP_GRAD also leaves what the weight gradients need.
+static cudaError_t pass(rd_surrogate* s, int mode, int B, const double* theta, double* phit,
+                        cudaStream_t st) {
+  k_features<<<(B * s->P + 127) / 128, 128, 0, st>>>(B, s->P, theta, s->norm, s->X,
+                                                     mode == MLP_PREDICT ? nullptr : s->sqerr);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  MlpArgs a{};
+  a.B = B;
+  a.X = s->X;
+  a.Wb = s->Wb;
+  a.params = s->params;
+  a.nm = s->norm;
+  a.phit = phit;
+  a.target = s->target;
+  a.out = s->out;
+  a.sq_err = s->sqerr;
+  a.H1 = s->H1;
+  a.H2 = s->H2;
+  a.dZ1 = s->dZ1;
+  a.dZ2 = s->dZ2;
+  a.dZ3 = s->dZ3;
+  a.Z1 = s->Z1;
+  a.part4 = s->part4;
+  a.err = s->pb->ws.err;
+  if (mode == MLP_PREDICT) return launch_mlp<MLP_PREDICT>(a, st);
+  if (mode == MLP_LOSS) return launch_mlp<MLP_LOSS>(a, st);
+  return launch_mlp<MLP_GRAD>(a, st);
+}
+
+// Loss and gradient of the mean-squared error against s->target for B rows (a
+// multiple of 128): the summed squared error into s->sqerr, all parameter
+// gradients into s->grads.
+static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, cudaStream_t st) {
+  cudaError_t e = pass(s, MLP_GRAD, B, theta, nullptr, st);
+  if (e != cudaSuccess) return e;
   const Layout L(s->W);
-  const int W = s->W;
-  int* err = s->pb->ws.err;
-  const size_t nW = (size_t)B * W;
-  k_head_bwd<<<(unsigned)((nW + 255) / 256), 256, 0, st>>>(B, W, s->dout, s->params + L.oW4,
-                                                           s->Z3, s->dZ3);
-  k_head_wgrad<<<(W + 127) / 128, 128, 0, st>>>(B, W, s->dout, s->H3, s->grads + L.oW4,
-                                                s->grads + L.ob4);
-  const __nv_bfloat16* Hs[3] = {s->X, s->H1, s->H2};  // inputs of layers 1..3
-  __nv_bfloat16* dZs[3] = {s->dZ1, s->dZ2, s->dZ3};
-  const float* Zs[3] = {s->Z1, s->Z2, s->Z3};
-  const size_t oW[3] = {L.oW1, L.oW2, L.oW3}, ob[3] = {L.ob1, L.ob2, L.ob3};
-  const int in[3] = {kIn, W, W};
-  cudaError_t e;
-  for (int l = 2; l >= 0; --l) {
-    // dW_l = dZ_l^T H_{l-1}: M = W (outputs), N = in_l, K = B
-    GemmArgs g{};
-    g.err = err;
-    g.M = W;
-    g.N = in[l];
-    g.K = B;
-    g.A = dZs[l];
-    g.lda = W;
-    g.B = Hs[l];
-    g.ldb = in[l];
-    g.out_f32 = s->grads + oW[l];
-    if ((e = gemm<EPI_F32, 1, 1>(g, st)) != cudaSuccess) return e;
-    k_colsum_bf16<<<(W + 127) / 128, 128, 0, st>>>(B, W, dZs[l], s->grads + ob[l]);
-    if (l == 0) break;
-    // dZ_{l-1} = (dZ_l W_l) o SiLU'(Z_{l-1}): M = B, N = W, K = W
-    GemmArgs h{};
-    h.err = err;
-    h.M = B;
-    h.N = W;
-    h.K = W;
-    h.A = dZs[l];
-    h.lda = W;
-    h.B = s->Wb + oW[l];
-    h.ldb = W;
-    h.zprev = Zs[l - 1];
-    h.out_bf16 = dZs[l - 1];
-    if ((e = gemm<EPI_BWD_SILU, 0, 1>(h, st)) != cudaSuccess) return e;
-  }
+  WgradArgs g{};
+  g.tiles = B / 128;
+  g.splits = std::min(g.tiles, kMaxSplits);
+  g.dZ[0] = s->dZ1;
+  g.dZ[1] = s->dZ2;
+  g.dZ[2] = s->dZ3;
+  g.H[0] = s->X;
+  g.H[1] = s->H1;
+  g.H[2] = s->H2;
+  g.part = s->part;
+  g.err = s->pb->ws.err;
+  if ((e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kWgSmem)) != cudaSuccess)
+    return e;
+  k_mlp_wgrad<<<dim3(s->W / 128, 3, g.splits), kMlpThreads, kWgSmem, st>>>(g);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_mlp_reduce<<<(unsigned)((L.total + 255) / 256), 256, 0, st>>>(g.splits, g.tiles, s->part,
+                                                                   s->part4, s->grads);
   return cudaGetLastError();
 }
 
@@ -529,10 +776,7 @@ cudaError_t adam_step(rd_surrogate* s, double lr, double b1, double b2, double e
 }
 
 cudaError_t predict(rd_surrogate* s, int B, const double* theta, double* phit, cudaStream_t st) {
-  cudaError_t e = forward(s, B, theta, false, st);
-  if (e != cudaSuccess) return e;
-  k_output<<<(B + 127) / 128, 128, 0, st>>>(B, s->out, s->norm, phit);
-  return cudaGetLastError();
+  return pass(s, MLP_PREDICT, B, theta, phit, st);
 }
 
 }  // namespace mlp
@@ -562,6 +806,7 @@ rd_status rd_surrogate_destroy(rd_surrogate* s) {
   if (!s) return RD_OK;
   if (s->pb) cudaStreamSynchronize(s->pb->stream);
   rd::mlp::free_acts(s);
+  rd::mlp::free_grad(s);
   cudaFree(s->params);
   cudaFree(s->grads);
   cudaFree(s->adam_m);
@@ -684,10 +929,9 @@ rd_status rd_surrogate_loss_grad(rd_surrogate* s, int B, const double* theta,
   RD_SCHECK(s && theta && target && loss, RD_EINVAL, "NULL argument");
   RD_SCHECK(B >= 128 && B % 128 == 0, RD_EINVAL, "B must be a positive multiple of 128");
   cudaStream_t st = s->pb->stream;
-  RD_SCUDA(mlp::ensure_rows(s, B));
+  RD_SCUDA(mlp::ensure_grad_rows(s, B));
   RD_SCUDA(cudaMemcpyAsync(s->target, target, sizeof(float) * B, cudaMemcpyDeviceToDevice, st));
-  RD_SCUDA(mlp::forward(s, B, theta, true, st));
-  RD_SCUDA(mlp::backward(s, B, st));
+  RD_SCUDA(mlp::loss_grad(s, B, theta, st));
   double se = 0.0;
   RD_SCUDA(cudaMemcpyAsync(&se, s->sqerr, sizeof(double), cudaMemcpyDeviceToHost, st));
   const mlp::Layout L(s->W);
@@ -786,7 +1030,7 @@ rd_status rd_surrogate_train(rd_surrogate* s, int n, const double* theta, const 
   RD_SCUDA(cudaMalloc(&d_z, sizeof(float) * z_s.size()));
   RD_SCUDA(cudaMemcpy(d_th, th_s.data(), sizeof(double) * th_s.size(), cudaMemcpyHostToDevice));
   RD_SCUDA(cudaMemcpy(d_z, z_s.data(), sizeof(float) * z_s.size(), cudaMemcpyHostToDevice));
-  RD_SCUDA(mlp::ensure_rows(s, td->batch));
+  RD_SCUDA(mlp::ensure_grad_rows(s, td->batch));
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -804,8 +1048,7 @@ rd_status rd_surrogate_train(rd_surrogate* s, int n, const double* theta, const 
       const int b = order[k];
       RD_SCUDA(cudaMemcpyAsync(s->target, d_z + (size_t)b * td->batch, sizeof(float) * td->batch,
                                cudaMemcpyDeviceToDevice, st));
-      RD_SCUDA(mlp::forward(s, td->batch, d_th + (size_t)b * td->batch * P, true, st));
-      RD_SCUDA(mlp::backward(s, td->batch, st));
+      RD_SCUDA(mlp::loss_grad(s, td->batch, d_th + (size_t)b * td->batch * P, st));
       RD_SCUDA(mlp::adam_step(s, td->lr, td->beta1, td->beta2, 1e-8, td->weight_decay, st));
       if (ep == td->epochs - 1) {
         double v = 0.0;
@@ -822,7 +1065,7 @@ rd_status rd_surrogate_train(rd_surrogate* s, int n, const double* theta, const 
   for (int off = n_train; off + td->batch <= n_train + n_hold; off += td->batch) {
     RD_SCUDA(cudaMemcpyAsync(s->target, d_z + off, sizeof(float) * td->batch,
                              cudaMemcpyDeviceToDevice, st));
-    RD_SCUDA(mlp::forward(s, td->batch, d_th + (size_t)off * P, true, st));
+    RD_SCUDA(mlp::pass(s, mlp::MLP_LOSS, td->batch, d_th + (size_t)off * P, nullptr, st));
     double v = 0.0;
     RD_SCUDA(cudaMemcpyAsync(&v, s->sqerr, sizeof(double), cudaMemcpyDeviceToHost, st));
     RD_SCUDA(cudaMemcpyAsync(outv.data(), s->out, sizeof(float) * td->batch, cudaMemcpyDeviceToHost, st));
