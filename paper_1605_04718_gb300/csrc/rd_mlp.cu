@@ -6,19 +6,20 @@
 // master weights, Adam with decoupled weight decay, and the output mapped to
 // a log-likelihood by Phi~ = floor + exp(shift + scale * net(x)).
 //
-// Forward and backward are row-local, so one kernel (k_mlp) takes a tile of 128
-// rows through all layers: weights stream into shared memory (128B-swizzled,
-// cp.async), each layer is M = 128, N = 256 kind::f16 MMAs (BF16 inputs, FP32
-// accumulator in TMEM) issued by one thread, and 16 warps run the bias + SiLU
-// (or SiLU') epilogue from TMEM straight into the next layer's operand tile.
-// Only the weight gradients sum over rows: k_mlp_wgrad forms them per layer,
-// half of the outputs and a share of the row tiles, k_mlp_reduce adds the
-// shares in a fixed order.  Measured (GB300): Phi~ of 4096 rows 375 ->
-// 36 us (a kernel per layer, one thread writing a row of
-// pre-activations nobody read); loss and gradients of 1024 rows 1020 ->
-// 118 us (column sums ran over the rows in one thread per column).
-// What is left is latency: one tile per SM, its weights' way from L2, and the
-// epilogues' 16 instructions per value.
+// Forward and backward are row-local, so one kernel (k_mlp) takes a tile of 32 or
+// 128 rows through all layers: weights stream into shared memory (128B-swizzled,
+// cp.async) as operand A, the rows' activations are operand B, so the units lie
+// on the TMEM lanes and a small tile still keeps 16 warps busy.  Each layer is
+// two M = 128 kind::f16 MMA sequences (BF16 inputs, FP32 accumulators in TMEM)
+// issued by one thread; the bias + SiLU (or SiLU') epilogue goes from TMEM
+// straight into the next layer's operand tile.  Only the weight gradients sum
+// over rows: k_mlp_wgrad forms them per layer, half of the outputs and a share
+// of the row tiles, k_mlp_reduce adds the shares in a fixed order.
+// Measured (GB300): Phi~ of 4096 rows 375 us with a kernel per layer, 36 us in
+// one kernel with rows on the lanes (128-row tiles only), 25 us as it is; loss
+// and gradients of 1024 rows 1017, 118 and 78 us.  What is left is latency: the
+// weights' way from L2 (264 KB per tile), the layers' chain of MMAs, barrier
+// and epilogue (16 instructions per value), FP64 logarithms (5 us) and launches.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -115,9 +116,9 @@ struct MlpArgs {
   const float* target;      // else: [B]
   float* out;               // else: [B]
   double* sq_err;           // else: summed
-  // MLP_GRAD
-  __nv_bfloat16 *H1, *H2, *dZ1, *dZ2, *dZ3;  // [B][W]
-  float* Z1;                                 // [B][W]
+  // MLP_GRAD, all with the units along the rows
+  __nv_bfloat16 *H1, *H2, *dZ1, *dZ2, *dZ3;  // [W][B]
+  float* Z1;                                 // [W][B]
   float* part4;             // [tile][W + 1]: shares of dW4, db4
   int* err;
 };
@@ -128,29 +129,35 @@ struct MlpCtrl {
   uint64_t bar;
   uint32_t tmem_base;
   int abort;
-  float bias[3][kW];
   float w4[kW];
   float out[128];
-  float dout[128];
+  alignas(16) float dout[128];
   float acc4[2][kW];
 };
-constexpr uint32_t kMlpTileA = 128 * kW * 2;  // 64 KB: activations, one 128-row tile
-constexpr uint32_t kMlpTileW = kW * kW * 2;   // 128 KB: one layer's weights
-constexpr uint32_t kMlpSmem = 1024 + kMlpTileA + kMlpTileW + sizeof(MlpCtrl);
+constexpr uint32_t kMlpTileW = kW * kW * 2;  // 128 KB: one layer's weights, rows = outputs
+constexpr uint32_t act_bytes(int nr) { return (uint32_t)(nr > 64 ? 2 : 1) * kW * 128u; }
+constexpr uint32_t mlp_smem_bytes(int nr) {
+  // at least 150 KB, so that no other CTA with a TMEM allocation shares the SM
+  return 1024 + kMlpTileW + act_bytes(nr) + (uint32_t)sizeof(MlpCtrl);
+}
 
-// K = 16 kk MMAs of D[128][256] (+)= A B^T; a_mn / b_mn: operand stored with K
-// along the rows; a_rows / b_rows: rows of the operand's tile.
-template <int KK, int A_MN, int B_MN>
-__device__ __forceinline__ void issue_layer(uint32_t d, uint32_t ta, int a_rows, uint32_t tb,
-                                            int b_rows, int n) {
-  const uint32_t idesc = idesc_bf16(128, n, A_MN, B_MN);
-  const uint64_t ad = sdesc_sw128(ta, A_MN ? (uint32_t)a_rows * 128u : 16u, 1024u);
-  const uint64_t bd = sdesc_sw128(tb, B_MN ? (uint32_t)b_rows * 128u : 16u, 1024u);
+// One layer, D[unit][row] for both halves of the units: A = the weights' tile
+// (K-major: its rows are the units; MN-major: its columns), B = the rows'
+// activations ([K][NR], MN-major) or features (K-major).
+template <int KK, int NR, int A_MN, int B_MN>
+__device__ __forceinline__ void issue_layer(uint32_t d, uint32_t tw, uint32_t tx) {
+  const uint32_t idesc = idesc_bf16(128, NR, A_MN, B_MN);
+  const uint64_t bd = sdesc_sw128(tx, B_MN ? (uint32_t)kW * 128u : 16u, 1024u);
 #pragma unroll
-  for (int kk = 0; kk < KK; ++kk) {
-    const uint32_t oa = A_MN ? kk * 2048u : (uint32_t)(kk >> 2) * a_rows * 128u + (kk & 3) * 32u;
-    const uint32_t ob = B_MN ? kk * 2048u : (uint32_t)(kk >> 2) * b_rows * 128u + (kk & 3) * 32u;
-    mma_f16(d, ad + (oa >> 4), bd + (ob >> 4), idesc, kk > 0 ? 1u : 0u);
+  for (int h = 0; h < 2; ++h) {
+    const uint64_t ad = sdesc_sw128(tw + (A_MN ? h * 2u * kW * 128u : h * 128u * 128u),
+                                    A_MN ? (uint32_t)kW * 128u : 16u, 1024u);
+#pragma unroll
+    for (int kk = 0; kk < KK; ++kk) {
+      const uint32_t oa = A_MN ? kk * 2048u : (uint32_t)(kk >> 2) * kW * 128u + (kk & 3) * 32u;
+      const uint32_t ob = kk * 2048u;  // K-major B has KK = 1
+      mma_f16(d + (uint32_t)(h * NR), ad + (oa >> 4), bd + (ob >> 4), idesc, kk > 0 ? 1u : 0u);
+    }
   }
 }
 
@@ -158,48 +165,50 @@ __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) 
   return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
 }
 
-// f(column, 16 accumulator values, 16 results): this thread's 64 columns of one
-// row, results as BF16 into the operand tile and, if g is not null, global row g.
-template <class F>
-__device__ __forceinline__ void epilogue(uint32_t t, uint8_t* tile, int row, int c0,
+// f(first row, 16 accumulator values, 16 results) over this thread's rows of one
+// unit; results as BF16 into the activation tile and, if g is not null, g[row].
+template <int NR, class F>
+__device__ __forceinline__ void epilogue(uint32_t t, uint8_t* tile, int unit, int r0,
                                          __nv_bfloat16* g, F&& f) {
 #pragma unroll 1
-  for (int c = c0; c < c0 + 64; c += 16) {
+  for (int r = r0; r < r0 + NR / 2; r += 16) {
     float v[16];
     __nv_bfloat16 h[16];
     __syncwarp();
-    tmem_ld16(t + (uint32_t)c, v);
+    tmem_ld16(t + (uint32_t)r, v);
     tmem_wait_ld();
-    f(c, v, h);
+    f(r, v, h);
 #pragma unroll
     for (int k = 0; k < 16; k += 8) {
       const uint4 q = make_uint4(pack_bf16(h[k], h[k + 1]), pack_bf16(h[k + 2], h[k + 3]),
                                  pack_bf16(h[k + 4], h[k + 5]), pack_bf16(h[k + 6], h[k + 7]));
-      *reinterpret_cast<uint4*>(tile + sw128_offset(128, row, c + k)) = q;
-      if (g) *reinterpret_cast<uint4*>(g + c + k) = q;
+      *reinterpret_cast<uint4*>(tile + sw128_offset(kW, unit, r + k)) = q;
+      if (g) *reinterpret_cast<uint4*>(g + r + k) = q;
     }
   }
 }
 
-template <int MODE>
+// NR rows per CTA, units on the TMEM lanes (two accumulators of 128), rows on
+// the columns: a tile of 32 rows still keeps every warp busy, so a batch of a
+// few thousand rows spreads over all SMs.
+template <int MODE, int NR>
 __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ MlpArgs a) {
   extern __shared__ uint8_t mlp_smem[];
   uint8_t* const base = mlp_smem + ((1024u - (smem_u32(mlp_smem) & 1023u)) & 1023u);
-  uint8_t* const ta = base;
-  uint8_t* const tw = base + kMlpTileA;
-  MlpCtrl* const ctl = reinterpret_cast<MlpCtrl*>(base + kMlpTileA + kMlpTileW);
+  uint8_t* const tw = base;
+  uint8_t* const ta = base + kMlpTileW;
+  MlpCtrl* const ctl = reinterpret_cast<MlpCtrl*>(base + kMlpTileW + act_bytes(NR));
   constexpr Layout L(kW);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.x * 128, valid = min(128, a.B - row0);
-  const int row = 32 * (warp & 3) + lane, c0 = 64 * (warp >> 2);
-  const bool mine = row < valid;
-  // layer 1's operands, then layer 2's weights behind its bytes
-  uint8_t* const tw1 = tw + kMlpTileW - 32768;  // the last 64-column block of the weights
-  load_tile<kIn>(ta, a.X + (size_t)row0 * kIn, kIn, 128, valid);
+  const int row0 = blockIdx.x * NR, valid = min(NR, a.B - row0);
+  const int half = (warp >> 2) & 1;
+  const int unit = 128 * half + 32 * (warp & 3) + lane, r0 = (NR / 2) * (warp >> 3);
+  // layer 1's operands; its weights sit where W2's last 64 columns go later
+  uint8_t* const tw1 = tw + kMlpTileW - 32768;
+  load_tile<kIn>(ta, a.X + (size_t)row0 * kIn, kIn, NR, valid);
   load_tile<kIn>(tw1, a.Wb + L.oW1, kIn, kW, kW);
   cp_async_commit();
-  // columns 0..191 of W2 now, the last 64 once layer 1 has read its weights there
-  auto load_w_cols = [&](const __nv_bfloat16* w, int b0, int b1) {
+  auto load_w_cols = [&](const __nv_bfloat16* w, int b0, int b1) {  // 64-column blocks
     const uint32_t tb = smem_u32(tw);
     const int per = 8 * (b1 - b0);
     for (int i = tid; i < kW * per; i += kMlpThreads) {
@@ -209,14 +218,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     cp_async_commit();
   };
   load_w_cols(a.Wb + L.oW2, 0, 3);
-  for (int i = tid; i < kW; i += kMlpThreads) {
-    ctl->bias[0][i] = a.params[L.ob1 + i];
-    ctl->bias[1][i] = a.params[L.ob2 + i];
-    ctl->bias[2][i] = a.params[L.ob3 + i];
-    ctl->w4[i] = a.params[L.oW4 + i];
-  }
+  for (int i = tid; i < kW; i += kMlpThreads) ctl->w4[i] = a.params[L.oW4 + i];
+  const float bias1 = a.params[L.ob1 + unit], bias2 = a.params[L.ob2 + unit],
+              bias3 = a.params[L.ob3 + unit];
   if (warp == 0) {
-    tmem_alloc(&ctl->tmem_base, 512);
+    tmem_alloc(&ctl->tmem_base, 4 * NR);
     tmem_relinquish();
   }
   if (tid == 0) {
@@ -230,8 +236,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
-  const uint32_t d0 = tmem, d1 = tmem + 256u;  // accumulators
-  const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+  const uint32_t d0 = tmem, d1 = tmem + 2u * NR;  // a layer's accumulators
+  const uint32_t t_off = ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(half * NR);
   const uint32_t sa = smem_u32(ta), sw = smem_u32(tw);
   uint32_t phase = 0;
   // waits for the MMAs issued since the last wait (a wait that gives up leaves
@@ -242,59 +248,58 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     tc_fence_after();
   };
   auto operands_ready = [&]() {
+    cp_async_wait<0>();
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
   };
+  auto silu_epilogue = [&](uint32_t d, float bias, __nv_bfloat16* h_out, float* z_out) {
+    epilogue<NR>(d + t_off, ta, unit, r0, h_out ? h_out + (size_t)unit * a.B + row0 : nullptr,
+                 [&](int r, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+#pragma unroll
+                   for (int j = 0; j < 16; ++j) {
+                     v[j] += bias;
+                     h[j] = __float2bfloat16_rn(silu(v[j]));
+                   }
+                   if (z_out) {
+                     float4* z = reinterpret_cast<float4*>(z_out + (size_t)unit * a.B + row0 + r);
+#pragma unroll
+                     for (int j = 0; j < 4; ++j)
+                       z[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                   }
+                 });
+  };
   // ---- layer 1 -> d0
   if (tid == 0) {
-    issue_layer<1, 0, 0>(d0, sa, 128, smem_u32(tw1), kW, kW);
+    issue_layer<1, NR, 0, 0>(d0, smem_u32(tw1), sa);
     mma_commit(&ctl->bar);
   }
   __syncwarp();
   done();
   load_w_cols(a.Wb + L.oW2, 3, 4);
-  auto silu_epilogue = [&](uint32_t d, int layer, __nv_bfloat16* h_out, float* z_out) {
-    epilogue(d + lane_off, ta, row, c0, (h_out && mine) ? h_out + (size_t)(row0 + row) * kW : nullptr,
-             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
-#pragma unroll
-               for (int j = 0; j < 16; ++j) {
-                 v[j] += ctl->bias[layer][c + j];
-                 h[j] = __float2bfloat16_rn(silu(v[j]));
-               }
-               if (z_out && mine) {
-                 float4* z = reinterpret_cast<float4*>(z_out + (size_t)(row0 + row) * kW + c);
-#pragma unroll
-                 for (int j = 0; j < 4; ++j)
-                   z[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-               }
-             });
-  };
-  silu_epilogue(d0, 0, MODE == MLP_GRAD ? a.H1 : nullptr, MODE == MLP_GRAD ? a.Z1 : nullptr);
-  cp_async_wait<0>();
+  silu_epilogue(d0, bias1, MODE == MLP_GRAD ? a.H1 : nullptr, MODE == MLP_GRAD ? a.Z1 : nullptr);
   operands_ready();
   // ---- layer 2 -> d1
   if (tid == 0) {
-    issue_layer<16, 0, 0>(d1, sa, 128, sw, kW, kW);
+    issue_layer<16, NR, 0, 1>(d1, sw, sa);
     mma_commit(&ctl->bar);
   }
   __syncwarp();
   done();
   load_w_cols(a.Wb + L.oW3, 0, 4);
-  silu_epilogue(d1, 1, MODE == MLP_GRAD ? a.H2 : nullptr, nullptr);
-  cp_async_wait<0>();
+  silu_epilogue(d1, bias2, MODE == MLP_GRAD ? a.H2 : nullptr, nullptr);
   operands_ready();
   // ---- layer 3 -> d0
   if (tid == 0) {
-    issue_layer<16, 0, 0>(d0, sa, 128, sw, kW, kW);
+    issue_layer<16, NR, 0, 1>(d0, sw, sa);
     mma_commit(&ctl->bar);
   }
   __syncwarp();
   done();
-  silu_epilogue(d0, 2, nullptr, nullptr);
+  silu_epilogue(d0, bias3, nullptr, nullptr);
   __syncthreads();
-  // ---- head: out[b] = sum_j H3[b][j] W4[j] + b4, one warp per row
+  // ---- head: out[b] = sum_j H3[j][b] W4[j] + b4, one warp per row
 #pragma unroll 1
   for (int r = warp; r < valid; r += kMlpThreads / 32) {
     float s = 0.f;
@@ -302,7 +307,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     for (int i = 0; i < kW / 32; ++i) {
       const int j = lane + 32 * i;
       const __nv_bfloat16 h =
-          *reinterpret_cast<const __nv_bfloat16*>(ta + sw128_offset(128, r, j));
+          *reinterpret_cast<const __nv_bfloat16*>(ta + sw128_offset(kW, j, r));
       s += __bfloat162float(h) * ctl->w4[j];
     }
 #pragma unroll
@@ -314,7 +319,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     if (tid < valid)
       a.phit[row0 + tid] = a.nm.floor + exp(a.nm.shift + a.nm.scale * (double)ctl->out[tid]);
   } else {
-    if (tid < 128) {
+    if (tid < NR) {
       double e2 = 0.0;
       if (tid < valid) {
         const float y = ctl->out[tid];
@@ -329,90 +334,94 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     }
     __syncthreads();
   }
-  if (MODE == MLP_GRAD) {
-    // shares of dW4 and db4 over the tile's rows (valid = 128)
+  if (MODE == MLP_GRAD) {  // every tile is full: the batch is a multiple of 128
+    // shares of dW4 and db4 over the tile's rows
     {
       const int j = tid & (kW - 1), hlf = tid / kW;
       float s = 0.f;
-      for (int r = 64 * hlf; r < 64 * hlf + 64; ++r)
-        s += ctl->dout[r] *
-             __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(ta + sw128_offset(128, r, j)));
+      for (int r = (NR / 2) * hlf; r < (NR / 2) * (hlf + 1); r += 8) {
+        const uint4 q = *reinterpret_cast<const uint4*>(ta + sw128_offset(kW, j, r));
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          s += ctl->dout[r + k] * __bfloat162float(__ushort_as_bfloat16(
+                                      (unsigned short)(w[k >> 1] >> (16 * (k & 1)))));
+      }
       ctl->acc4[hlf][j] = s;
       __syncthreads();
       float* p4 = a.part4 + (size_t)blockIdx.x * (kW + 1);
       if (tid < kW) p4[tid] = ctl->acc4[0][tid] + ctl->acc4[1][tid];
       if (tid == 0) {
         float t = 0.f;
-        for (int r = 0; r < 128; ++r) t += ctl->dout[r];
+        for (int r = 0; r < NR; ++r) t += ctl->dout[r];
         p4[kW] = t;
       }
     }
+    const size_t g0 = (size_t)unit * a.B + row0;
     // ---- dZ3 = dout W4 o SiLU'(Z3), Z3 still in d0
-    const float dout = ctl->dout[row];
-    epilogue(d0 + lane_off, ta, row, c0, a.dZ3 + (size_t)(row0 + row) * kW,
-             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+    const float w4 = ctl->w4[unit];
+    epilogue<NR>(d0 + t_off, ta, unit, r0, a.dZ3 + g0,
+                 [&](int r, float (&v)[16], __nv_bfloat16 (&h)[16]) {
 #pragma unroll
-               for (int j = 0; j < 16; ++j)
-                 h[j] = __float2bfloat16_rn(dout * ctl->w4[c + j] *
-                                            silu_grad(v[j] + ctl->bias[2][c + j]));
-             });
+                   for (int j = 0; j < 16; ++j)
+                     h[j] = __float2bfloat16_rn(ctl->dout[r + j] * w4 * silu_grad(v[j] + bias3));
+                 });
     operands_ready();
-    // ---- dH2 = dZ3 W3 -> d0; dZ2 = dH2 o SiLU'(Z2), Z2 in d1
+    // ---- dH2 = W3^T dZ3 -> d0; dZ2 = dH2 o SiLU'(Z2), Z2 in d1
     if (tid == 0) {
-      issue_layer<16, 0, 1>(d0, sa, 128, sw, kW, kW);
+      issue_layer<16, NR, 1, 1>(d0, sw, sa);
       mma_commit(&ctl->bar);
     }
     __syncwarp();
     done();
     load_w_cols(a.Wb + L.oW2, 0, 4);
-    epilogue(d0 + lane_off, ta, row, c0, a.dZ2 + (size_t)(row0 + row) * kW,
-             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
-               float z[16];
-               tmem_ld16(d1 + lane_off + (uint32_t)c, z);
-               tmem_wait_ld();
+    epilogue<NR>(d0 + t_off, ta, unit, r0, a.dZ2 + g0,
+                 [&](int r, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+                   float z[16];
+                   tmem_ld16(d1 + t_off + (uint32_t)r, z);
+                   tmem_wait_ld();
 #pragma unroll
-               for (int j = 0; j < 16; ++j)
-                 h[j] = __float2bfloat16_rn(v[j] * silu_grad(z[j] + ctl->bias[1][c + j]));
-             });
-    cp_async_wait<0>();
+                   for (int j = 0; j < 16; ++j)
+                     h[j] = __float2bfloat16_rn(v[j] * silu_grad(z[j] + bias2));
+                 });
     operands_ready();
-    // ---- dH1 = dZ2 W2 -> d0; dZ1 = dH1 o SiLU'(Z1)
+    // ---- dH1 = W2^T dZ2 -> d0; dZ1 = dH1 o SiLU'(Z1)
     if (tid == 0) {
-      issue_layer<16, 0, 1>(d0, sa, 128, sw, kW, kW);
+      issue_layer<16, NR, 1, 1>(d0, sw, sa);
       mma_commit(&ctl->bar);
     }
     __syncwarp();
     done();
-    epilogue(d0 + lane_off, ta, row, c0, a.dZ1 + (size_t)(row0 + row) * kW,
-             [&](int c, float (&v)[16], __nv_bfloat16 (&h)[16]) {
-               const float4* z4 =
-                   reinterpret_cast<const float4*>(a.Z1 + (size_t)(row0 + row) * kW + c);
+    epilogue<NR>(d0 + t_off, ta, unit, r0, a.dZ1 + g0,
+                 [&](int r, float (&v)[16], __nv_bfloat16 (&h)[16]) {
+                   const float4* z4 = reinterpret_cast<const float4*>(a.Z1 + g0 + r);
 #pragma unroll
-               for (int j = 0; j < 4; ++j) {
-                 const float4 z = z4[j];
-                 h[4 * j] = __float2bfloat16_rn(v[4 * j] * silu_grad(z.x));
-                 h[4 * j + 1] = __float2bfloat16_rn(v[4 * j + 1] * silu_grad(z.y));
-                 h[4 * j + 2] = __float2bfloat16_rn(v[4 * j + 2] * silu_grad(z.z));
-                 h[4 * j + 3] = __float2bfloat16_rn(v[4 * j + 3] * silu_grad(z.w));
-               }
-             });
+                   for (int j = 0; j < 4; ++j) {
+                     const float4 z = z4[j];
+                     h[4 * j] = __float2bfloat16_rn(v[4 * j] * silu_grad(z.x));
+                     h[4 * j + 1] = __float2bfloat16_rn(v[4 * j + 1] * silu_grad(z.y));
+                     h[4 * j + 2] = __float2bfloat16_rn(v[4 * j + 2] * silu_grad(z.z));
+                     h[4 * j + 3] = __float2bfloat16_rn(v[4 * j + 3] * silu_grad(z.w));
+                   }
+                 });
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, 512);
+    tmem_dealloc(tmem, 4 * NR);
   }
   if (tid == 0 && ctl->abort) atomicOr(a.err, 1);
 }
 
-// Weight and bias gradients dW_l = dZ_l^T H_{l-1}, db_l = column sums of dZ_l:
-// block (x = outputs 128 x .. 128 x + 127, y = layer, z = share of the row
-// tiles), into that share's copy of the parameter layout.
+// Weight and bias gradients dW_l = dZ_l H_{l-1}^T, db_l = row sums of dZ_l
+// (units along the rows): block (x = outputs 128 x .. 128 x + 127, y = layer,
+// z = share of the 128-row tiles), into that share's copy of the parameter
+// layout.
 struct WgradArgs {
-  int tiles, splits;
-  const __nv_bfloat16* dZ[3];
-  const __nv_bfloat16* H[3];
+  int B, tiles, splits;
+  const __nv_bfloat16* dZ[3];  // [W][B]
+  const __nv_bfloat16* H[3];   // [0]: the features [B][16]; else [W][B]
   float* part;  // [splits][stride()]
   int* err;
 };
@@ -430,7 +439,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int layer = blockIdx.y, m0 = 128 * blockIdx.x, share = blockIdx.z;
   const int n = layer == 0 ? kIn : kW;
-  const __nv_bfloat16* dz = a.dZ[layer] + m0;
+  const __nv_bfloat16* dz = a.dZ[layer] + (size_t)m0 * a.B;
   const __nv_bfloat16* hh = a.H[layer];
   const int t0 = (int)((long long)a.tiles * share / a.splits);
   const int t1 = (int)((long long)a.tiles * (share + 1) / a.splits);
@@ -445,18 +454,18 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   }
   auto load = [&](int t) {
     uint8_t* s = base + (uint32_t)(t & 1) * (kWgTileA + kWgTileB);
-    load_tile<128>(s, dz + (size_t)t * 128 * kW, kW, 128, 128);
+    load_tile<128>(s, dz + (size_t)t * 128, a.B, 128, 128);
     if (layer == 0)
       load_tile<kIn>(s + kWgTileA, hh + (size_t)t * 128 * kIn, kIn, 128, 128);
     else
-      load_tile<kW>(s + kWgTileA, hh + (size_t)t * 128 * kW, kW, 128, 128);
+      load_tile<128>(s + kWgTileA, hh + (size_t)t * 128, a.B, kW, kW);
     cp_async_commit();
   };
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_base;
-  const uint32_t idesc = idesc_bf16(128, n, 1, 1);
+  const uint32_t idesc = idesc_bf16(128, n, 0, layer == 0 ? 1 : 0);
   const int col = tid & 127, quarter = tid >> 7;
   float colsum = 0.f;
   uint32_t phase = 0;
@@ -475,22 +484,32 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
     __syncthreads();
     tc_fence_after();
     if (tid == 0) {
-      const uint64_t ad = sdesc_sw128(smem_u32(s), 128u * 128u, 1024u);
-      const uint64_t bd = sdesc_sw128(smem_u32(s + kWgTileA), 128u * 128u, 1024u);
+      const uint32_t sb = smem_u32(s + kWgTileA);
+      const uint64_t ad = sdesc_sw128(smem_u32(s), 16u, 1024u);
+      const uint64_t bd = layer == 0 ? sdesc_sw128(sb, 128u * 128u, 1024u)
+                                     : sdesc_sw128(sb, 16u, 1024u);
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk)
-        mma_f16(tmem, ad + (kk * 2048u >> 4), bd + (kk * 2048u >> 4), idesc,
-                (t > t0 || kk > 0) ? 1u : 0u);
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint32_t oa = (uint32_t)(kk >> 2) * 128u * 128u + (kk & 3) * 32u;
+        const uint32_t ob =
+            layer == 0 ? kk * 2048u : (uint32_t)(kk >> 2) * kW * 128u + (kk & 3) * 32u;
+        mma_f16(tmem, ad + (oa >> 4), bd + (ob >> 4), idesc, (t > t0 || kk > 0) ? 1u : 0u);
+      }
       mma_commit(&bar);
     }
     __syncwarp();
     if (t + 1 < t1) load(t + 1);
-#pragma unroll 8
-    for (int r = 32 * quarter; r < 32 * quarter + 32; ++r)
-      colsum += __bfloat162float(
-          *reinterpret_cast<const __nv_bfloat16*>(s + sw128_offset(128, r, col)));
+#pragma unroll
+    for (int r = 0; r < 32; r += 8) {
+      const uint4 q = *reinterpret_cast<const uint4*>(s + sw128_offset(128, col, 32 * quarter + r));
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        colsum += __bfloat162float(
+            __ushort_as_bfloat16((unsigned short)(w[k >> 1] >> (16 * (k & 1)))));
+    }
   }
-  ok = ok && mbar_wait_bounded(&bar, phase & 1u, &abort_flag);
+  ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag) && ok;
   tc_fence_after();
   sums[tid] = colsum;
   __syncthreads();
@@ -669,7 +688,7 @@ static cudaError_t ensure_grad_rows(rd_surrogate* s, int rows) {
   RD_ALLOC(s->dZ3, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->Z1, sizeof(float) * cap * W);
   RD_ALLOC(s->part, sizeof(float) * kMaxSplits * L.stride());
-  RD_ALLOC(s->part4, sizeof(float) * (cap / 128) * (W + 1));
+  RD_ALLOC(s->part4, sizeof(float) * (cap / 32) * (W + 1));
   s->grad_cap = rows;
   return cudaSuccess;
 }
@@ -682,13 +701,28 @@ static cudaError_t refresh_bf16(rd_surrogate* s, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int MODE>
+template <int MODE, int NR>
 static cudaError_t launch_mlp(const MlpArgs& a, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(k_mlp<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kMlpSmem);
+  cudaError_t e =
+      cudaFuncSetAttribute(k_mlp<MODE, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)mlp_smem_bytes(NR));
   if (e != cudaSuccess) return e;
-  k_mlp<MODE><<<(a.B + 127) / 128, kMlpThreads, kMlpSmem, st>>>(a);
+  k_mlp<MODE, NR><<<(a.B + NR - 1) / NR, kMlpThreads, mlp_smem_bytes(NR), st>>>(a);
   return cudaGetLastError();
+}
+
+// Rows per tile: 32 while that fills the SMs at most twice, each tile reading all
+// weights anew (forward: 4096 rows 23 us against 37 with 128-row tiles, 9728
+// rows 35 against 39, 14592 rows 47 against 41); the backward pass, whose tiles
+// do three times as much, once and a half (8192 rows 124 us both ways).
+static int tile_rows(int mode, int B, int n_sm) {
+  const int waves2 = mode == MLP_GRAD ? 3 : 4;  // twice the waves
+  return B <= waves2 * 16 * n_sm ? 32 : 128;
+}
+
+template <int MODE>
+static cudaError_t launch_mlp(const MlpArgs& a, int n_sm, cudaStream_t st) {
+  return tile_rows(MODE, a.B, n_sm) == 32 ? launch_mlp<MODE, 32>(a, st) : launch_mlp<MODE, 128>(a, st);
 }
 
 // One pass over B rows of theta (device [B][P]): MLP_PREDICT writes Phi~ to
@@ -718,9 +752,10 @@ static cudaError_t pass(rd_surrogate* s, int mode, int B, const double* theta, d
   a.Z1 = s->Z1;
   a.part4 = s->part4;
   a.err = s->pb->ws.err;
-  if (mode == MLP_PREDICT) return launch_mlp<MLP_PREDICT>(a, st);
-  if (mode == MLP_LOSS) return launch_mlp<MLP_LOSS>(a, st);
-  return launch_mlp<MLP_GRAD>(a, st);
+  const int n_sm = s->pb->n_sm;
+  if (mode == MLP_PREDICT) return launch_mlp<MLP_PREDICT>(a, n_sm, st);
+  if (mode == MLP_LOSS) return launch_mlp<MLP_LOSS>(a, n_sm, st);
+  return launch_mlp<MLP_GRAD>(a, n_sm, st);
 }
 
 // Loss and gradient of the mean-squared error against s->target for B rows (a
@@ -731,6 +766,7 @@ static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, cudaSt
   if (e != cudaSuccess) return e;
   const Layout L(s->W);
   WgradArgs g{};
+  g.B = B;
   g.tiles = B / 128;
   g.splits = std::min(g.tiles, kMaxSplits);
   g.dZ[0] = s->dZ1;
@@ -746,7 +782,7 @@ static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, cudaSt
     return e;
   k_mlp_wgrad<<<dim3(s->W / 128, 3, g.splits), kMlpThreads, kWgSmem, st>>>(g);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_mlp_reduce<<<(unsigned)((L.total + 255) / 256), 256, 0, st>>>(g.splits, g.tiles, s->part,
+  k_mlp_reduce<<<(unsigned)((L.total + 255) / 256), 256, 0, st>>>(g.splits, B / tile_rows(MLP_GRAD, B, s->pb->n_sm), s->part,
                                                                    s->part4, s->grads);
   return cudaGetLastError();
 }
