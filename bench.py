@@ -50,8 +50,8 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "68ffd2d87df72dd1ab55b2fbbb62bba1984fa39655bf48b589104d2a8c2c27e2",
-        "bytes": 1520384 + 1948416,
+        "sha256": "178b48f1a25d16c386255bdc94d6bc14c2b5a64e43c96271ce5ebcaf69284a8c",
+        "bytes": 1238784 + 2430976,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)

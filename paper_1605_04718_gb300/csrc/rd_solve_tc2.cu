@@ -11,9 +11,9 @@
 // against four transforms when both directions are diagonalised: half the
 // tensor-core work, two conversions of the data per step instead of four, and
 // no 1 / (alpha + beta (mu_k + mu_l)) per point.  The scan is FP32 throughout.
-// Measured against the four-transform kernels (GB300): 128^2 9.98 -> 6.33 us a
+// Measured against the four-transform kernels (GB300): 128^2 9.98 -> 5.8 us a
 // step of one proposal per SM; 64^2 18.7 -> 4.9 us for the four proposals an SM
-// holds; relative field error after 1000 steps at 128^2 2.2e-7 -> 1.9e-7.
+// holds; relative field error after 1000 steps at 128^2 2.2e-7 -> 1.8e-7.
 //
 // Layout.  A slab is one accumulator of 128 TMEM lanes x 128 columns; a CTA has
 // two.  The constant matrices are operand A, read from TMEM, the data operand B
@@ -29,16 +29,29 @@
 //
 // Warps 0-15 convert (TMEM -> registers -> reaction or scan -> split ->
 // shared memory), warp 16 issues every MMA from one thread, warp 17 forms the
-// growing domain's factors in FP64 one step ahead.  N > 64: the u and v halves
-// of the converters scan their slabs side by side (scanning u with all 16
-// warps and then v measured 7.05 us a step against 6.85: v's operand then
-// comes late for stage 2).  N <= 64: all 16 warps take slab 0 and then slab 1,
-// so each slab's MMAs run under the other's conversions (5.1 us a step against
-// 5.46 with eight warps per slab).  The converters bound the kernel: about 20
-// instructions per point for the reaction and 9 per value for the scan, on an
-// FP32 pipe that takes 1.5 cycles per FMA with three register operands, with
-// the tensor pipe 45 % busy.  The issuing loops are unrolled at compile time:
-// forming descriptors at run time cost 100 to 150 cycles an MMA against 64.
+// growing domain's factors in FP64 one step ahead.
+//   N > 64: one proposal's step is a chain -- reaction, stage 1, scan, stage 2 --
+//   so it is overlapped within itself.  u and v run one behind the other on the
+//   tensor cores; their scans run side by side, eight warps each (scanning u
+//   with all 16 warps and then v measured 7.05 us a step against 6.85: v's
+//   operand then comes late for stage 2).  Stage 2 of v is issued as two column
+//   halves, so the reaction of the first 64 columns runs under the second half
+//   (an N = 64 MMA takes 37 cycles against 64 for N = 128), and stage 1 starts
+//   with the correction products of those columns while the others are computed.
+//   Measured with both together: 6.65 -> 5.79 us, of which the reaction's
+//   arithmetic below is 0.3.
+//   N <= 64: all 16 warps take slab 0 and then slab 1, so each slab's MMAs run
+//   under the other's conversions (5.1 us a step against 5.46 with eight warps
+//   per slab).
+// The converters bound the kernel: 8 FP32 operations and two splits per point
+// for the reaction, 4 FMAs and a split per value for the scan, on an FP32 pipe
+// that takes 1.5 cycles per FMA with three register operands and 2 per FP16 pair
+// conversion; the tensor pipe is busy 50 to 60 % of a step, the rest of the chain
+// is hand-offs (a commit or an arrival reaches its waiter after 350 to 450
+// cycles; spinning waiters were no faster).  The issuing loops are unrolled at
+// compile time: forming descriptors at run time cost 100 to 150 cycles an MMA
+// against 64.  Branches around the stores, one per 8 values, cost 2 %: they end
+// the blocks that the compiler schedules the conversions in.
 //
 // Precision: every FP32 operand x is split into FP16 hi + lo and each product
 // formed as hi*hi + hi*lo + lo*hi, about 22 significant bits.  The tensor core
@@ -47,11 +60,16 @@
 // the N / 16 main products leave.  The data's lo part is stored negated (one
 // instruction less per pair) and the MMAs that read it set the negate bit.
 // Power-of-two scales keep operands inside the FP16 range:
-//   R' = 256 r, C' = 8 C -> D' = 2048 D; X' = 16 x; W' = 128 w.
+//   R' = 128 r, C' = 8 C -> D' = 1024 D; X' = 16 x; W' = 128 w.
+// The state and R' have the same scale, so the reaction's linear term is the
+// state as it is; the growing domain's constant (1 - alpha) w_ref only concerns
+// mode k = 0 and is added to the scan's result there, in the same operation as
+// the output scale.
 //
 // N <= 64: the block-diagonal A multiplies other proposals' data by zero, so a
 // reaction value outside the FP16 range (a diverging solve) must not reach the
-// MMA as infinity: it is stored as zero and every later observation or output
+// MMA as infinity (nor reach the scan as one: |r| >= 256): it is stored as zero, and
+// every later observation or output
 // of its proposal reads NaN, which is what an infinite operand leads to.
 //
 // Every wait is bounded; a timed-out wait makes the CTA leave, drain its MMAs,
@@ -93,11 +111,13 @@ struct Geo {
 };
 
 struct alignas(16) React {  // one proposal's step constants
-  float fa, fb, ftg, alpha, cu, cv;
+  float fa, fb, ftg, alpha;  // a, b, 128 tau gamma, 1 + tau m r
+  float off[2];              // growing domain: the term (1 - alpha) w_ref of k = 0, per field
 };
 
 struct Ctrl {
   uint64_t mma_done[2];    // per slab: a stage's MMAs completed (two phases per step)
+  uint64_t half_done;      // N > 64: slab 1's stage 2, first 64 columns
   uint64_t op_ready[2];    // per slab: scanned operand written
   uint64_t rx[2];          // N > 64: first / second half of both slabs' reaction written;
                            // N <= 64: slab 0 / 1's reaction written (16 warps)
@@ -140,8 +160,9 @@ __device__ __forceinline__ Ctrl* shared_ctl() {
   return reinterpret_cast<Ctrl*>(shared_base() + kOffCtrl);
 }
 
-__device__ __forceinline__ uint8_t* tile(uint8_t* base, int g, int hl) {
-  return base + (uint32_t)(2 * g + hl) * kTileBytes;
+// Shared address of slab g's hi tile (its lo tile follows).
+__device__ __forceinline__ uint32_t tile(int g) {
+  return smem_u32(shared_base()) + (uint32_t)(2 * g) * kTileBytes;
 }
 
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
@@ -162,7 +183,8 @@ __device__ __forceinline__ constexpr uint32_t kblock_off(int stage, int rows, in
 
 // K blocks [K0, K1) of one stage of slab g: the correction products (lo
 // operand parts), the main products, or both.  kb < K1 skips the blocks from kb.
-template <int STAGE, int ROWS, bool CORR, bool MAIN, int K0, int K1, bool FIRST>
+// COL0 (0 or 64, stage 2): the first of the ncols columns.
+template <int STAGE, int ROWS, bool CORR, bool MAIN, int K0, int K1, bool FIRST, int COL0 = 0>
 __device__ __forceinline__ void issue_blocks(uint32_t sbase, uint32_t tmem, int g, int ncols,
                                              int kb) {
   constexpr int b_mn = STAGE == 2;
@@ -170,9 +192,11 @@ __device__ __forceinline__ void issue_blocks(uint32_t sbase, uint32_t tmem, int 
   const uint32_t idesc_nb = idesc_f16_f32(128, ncols, 0, b_mn, 1);  // B = the negated lo
   const uint32_t a_hi = tmem + kColA + (STAGE == 1 ? 0u : 128u), a_lo = a_hi + 64u;
   constexpr uint32_t lbo = STAGE == 1 ? 16u : (uint32_t)ROWS * 128u;
-  const uint64_t bh = sdesc_sw128(sbase + (uint32_t)(2 * g) * kTileBytes, lbo, 1024u);
-  const uint64_t bl = sdesc_sw128(sbase + (uint32_t)(2 * g + 1) * kTileBytes, lbo, 1024u);
-  const uint32_t d = tmem + kColAcc + (uint32_t)(128 * g);
+  static_assert(COL0 == 0 || (COL0 == 64 && STAGE == 2), "columns start at a 64-column block");
+  const uint32_t tb = sbase + (uint32_t)(2 * g) * kTileBytes + (uint32_t)COL0 / 64u * ROWS * 128u;
+  const uint64_t bh = sdesc_sw128(tb, lbo, 1024u);
+  const uint64_t bl = sdesc_sw128(tb + kTileBytes, lbo, 1024u);
+  const uint32_t d = tmem + kColAcc + (uint32_t)(128 * g + COL0);
   if (CORR) {
 #pragma unroll
     for (int kk = K0; kk < K1; ++kk) {
@@ -191,56 +215,60 @@ __device__ __forceinline__ void issue_blocks(uint32_t sbase, uint32_t tmem, int 
   }
 }
 
-// Splits 8 values (times scale) of row r, columns c..c+7 into the hi and
-// negated lo tiles: one 16-byte store each.
-__device__ __forceinline__ void store8(uint8_t* hi, uint8_t* lo, int rows, int r, int c,
-                                       const float* x, float scale) {
-  uint32_t h[4], l[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) split_f16x2_neglo_scaled(x[2 * j], x[2 * j + 1], scale, h[j], l[j]);
-  const uint32_t off = sw128_offset(rows, r, c);
-  *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+// Predicated 16-byte shared store: a branch instead would end the basic block
+// that the compiler schedules the conversions in.
+__device__ __forceinline__ void st_shared16(uint32_t addr, const uint32_t (&v)[4], bool on) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t"
+      "@p st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n\t}" ::"r"(addr),
+      "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"((uint32_t)on)
+      : "memory");
 }
 
-// As store8 without a scale.  GUARD: a value outside the FP16 range (or NaN)
-// makes the 8 values zero and returns true, so that it cannot reach the
-// proposals that share the MMA's K extent through 0 * inf.
-template <bool GUARD>
-__device__ __forceinline__ bool store8n(uint8_t* hi, uint8_t* lo, int rows, int r, int c,
-                                        const float* x) {
+// Splits 8 values (x scale + off) of row r, columns c..c+7 into the hi tile and,
+// kTileBytes behind it, the negated lo tile: one 16-byte store each.
+__device__ __forceinline__ void store8(uint32_t hi, int rows, int r, int c, const float* x,
+                                       float scale, float off, bool on) {
   uint32_t h[4], l[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) split_f16x2_neglo(x[2 * j], x[2 * j + 1], h[j], l[j]);
-  bool out = false;
-  if (GUARD) {
-    uint32_t e = 0;  // bit 15 or 31 set where an exponent field is all ones
-#pragma unroll
-    for (int j = 0; j < 4; ++j) e |= (h[j] & 0x7C007C00u) + 0x04000400u;
-    out = (e & 0x80008000u) != 0u;
-    if (out)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) h[j] = l[j] = 0u;
+  for (int j = 0; j < 4; ++j) {
+    float y0 = x[2 * j], y1 = x[2 * j + 1];
+    fma_pair(y0, y1, scale, off);
+    split_f16x2_neglo(y0, y1, h[j], l[j]);
   }
-  const uint32_t off = sw128_offset(rows, r, c);
-  *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
-  *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
-  return out;
+  const uint32_t a = hi + sw128_offset(rows, r, c);
+  st_shared16(a, h, on);
+  st_shared16(a + kTileBytes, l, on);
 }
 
-// Explicit reaction in place on 8 points: state (x 128) ->
-// r_u = du + tau gamma (a - u + u^2 v) (+ cu), r_v = dv + tau gamma (b - u^2 v)
-// (+ cv), as deviations from the reference state, times 256 (the operand
-// scale, applied through the constants: exact).
-__device__ __forceinline__ void react8(float* u, float* v, float sw, float ref_u, float ref_v,
+// As store8 without a scale; returns a word with bit 15 or 31 set where a value
+// is 2^15 or larger (or NaN): |r| >= 256.
+__device__ __forceinline__ uint32_t store8n(uint32_t hi, int rows, int r, int c, const float* x,
+                                            bool on) {
+  uint32_t h[4], l[4], e = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    split_f16x2_neglo(x[2 * j], x[2 * j + 1], h[j], l[j]);
+    e |= (h[j] & 0x7C007C00u) + 0x08000800u;
+  }
+  const uint32_t a = hi + sw128_offset(rows, r, c);
+  st_shared16(a, h, on);
+  st_shared16(a + kTileBytes, l, on);
+  return e;
+}
+
+// Explicit reaction in place on 8 points, all times 128 (the operand scale is the
+// state's, so the linear term is the state itself):
+// r_u = du + tau gamma (a - u + u^2 v), r_v = dv + tau gamma (b - u^2 v), as
+// deviations from the reference state.
+__device__ __forceinline__ void react8(float* u, float* v, float ref_u, float ref_v,
                                        const React& k) {
-  const float sw8 = 256.f * sw, ftg8 = 256.f * k.ftg, cu8 = 256.f * k.cu, cv8 = 256.f * k.cv;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const float uu = fmaf(u[j], sw, ref_u), vv = fmaf(v[j], sw, ref_v);
-    const float u2v = uu * uu * vv;
-    u[j] = fmaf(ftg8, k.fa - uu + u2v, fmaf(u[j], sw8, cu8));
-    v[j] = fmaf(ftg8, k.fb - u2v, fmaf(v[j], sw8, cv8));
+    const float uu = fmaf(u[j], 0x1p-7f, ref_u), vv = fmaf(v[j], 0x1p-7f, ref_v);
+    const float uv = uu * vv;
+    u[j] = fmaf(k.ftg, fmaf(uu, uv, k.fa - uu), u[j]);
+    v[j] = fmaf(k.ftg, fmaf(-uu, uv, k.fb), v[j]);
   }
 }
 
@@ -248,7 +276,7 @@ __device__ __forceinline__ void react8(float* u, float* v, float sw, float ref_u
 // slab pair: column indices c0 + 8 step_c j, j < n8, of lane index idx, u at
 // TMEM columns t_u + c, v at t_v + c.  sl: the proposal's slot, -1 for idle rows.
 __device__ __noinline__ void observe(const DevProblem& pb, int size, int sl, int idx, int c0,
-                                     int step_c, int n8, uint32_t t_u, uint32_t t_v, float sw,
+                                     int step_c, int n8, uint32_t t_u, uint32_t t_v,
                                      int step, int obs, float* fields, size_t field_stride) {
   Ctrl* ctl = shared_ctl();
   const DevSize& S = pb.sz[size];
@@ -259,7 +287,8 @@ __device__ __noinline__ void observe(const DevProblem& pb, int size, int sl, int
   const float* yo = obs >= 0 ? S.yf + (size_t)obs * nfo * S.npts : nullptr;
   float* fo = out ? fields + (size_t)ctl->items[sl] * field_stride : nullptr;
   const bool blown = sl >= 0 && ctl->blown[sl];
-  if (blown) sw = __int_as_float(0x7fffffff);  // NaN, as the solve would have reached
+  // NaN where the solve would have reached it
+  const float sw = blown ? __int_as_float(0x7fffffff) : 0x1p-7f;
   double phi = 0.0;
   int bad = 0;
   for (int k = 0; k < n8; ++k) {
@@ -310,9 +339,8 @@ __device__ __noinline__ void observe(const DevProblem& pb, int size, int sl, int
 // accumulator columns at t to the operand row l, columns col0...
 template <int N>
 __device__ __noinline__ void slow_row(uint32_t t, int g, int rows, int l, int col0, bool store,
-                                      float alpha, float beta, float mu, float out_scale) {
-  uint8_t* const hi = tile(shared_base(), g, 0);
-  uint8_t* const lo = tile(shared_base(), g, 1);
+                                      float alpha, float beta, float mu, float out_scale,
+                                      float off) {
   float c[N], d[N];
   const float lam = fmaf(beta, mu, alpha);
   float cp = 0.f, dp = 0.f;
@@ -335,10 +363,10 @@ __device__ __noinline__ void slow_row(uint32_t t, int g, int rows, int l, int co
     x1 = d[i] - (i < N - 1 ? c[i] * x1 : 0.f);
     d[i] = x1;
   }
-  if (store)
-    for (int x = 0; x < N; x += 8) store8(hi, lo, rows, l, col0 + x, d + x, out_scale);
+  for (int x = 0; x < N; x += 8) store8(tile(g), rows, l, col0 + x, d + x, out_scale, off, store);
 }
 
+// Starts the load of H columns: tmem_wait_ld() before they are read.
 template <int H>
 __device__ __forceinline__ void load_cols(uint32_t t, float (&r)[H]) {
   __syncwarp();
@@ -351,22 +379,19 @@ __device__ __forceinline__ void load_cols(uint32_t t, float (&r)[H]) {
     for (int x = 0; x < H; x += 8)
       tmem_ld8(t + (uint32_t)x, *reinterpret_cast<float(*)[8]>(r + x));
   }
-  tmem_wait_ld();
 }
 
-// One scan segment (segment seg of a row) of slab g: accumulator columns t..
-// -> operand row l, columns col0...  slot: where the row's sums are exchanged.
+// One scan segment r (segment seg of a row) of slab g -> operand row l, columns
+// col0...  slot: where the row's sums are exchanged.
 template <int N>
-__device__ __forceinline__ bool scan_segment(uint64_t wait_ns, uint32_t t, int g, int seg,
+__device__ __forceinline__ bool scan_segment(uint64_t wait_ns, float (&r)[ScanSeg<N>::H], int g, int seg,
                                              int slot, int quad, uint32_t parity, int lane,
-                                             int col0, bool row_used, const ScanCoef& k) {
+                                             int col0, bool row_used, const ScanCoef& k,
+                                             float off) {
   using SG = ScanSeg<N>;
   constexpr int E = Geo<N>::S, H = SG::H;
-  uint8_t* const base = shared_base();
   Ctrl* const ctl = shared_ctl();
   const int l = 32 * quad + lane;
-  float r[H];
-  load_cols<H>(t, r);
   float left, right;
   {
     float2 lr[SG::NS];
@@ -399,8 +424,7 @@ __device__ __forceinline__ bool scan_segment(uint64_t wait_ns, uint32_t t, int g
   for (int m = H - 2; m >= 0; --m) {
     x = fmaf(k.a, x, r[m]);
     r[m] = x;
-    if (m % 8 == 0 && row_used)
-      store8(tile(base, g, 0), tile(base, g, 1), E, l, col0 + m, r + m, k.sc);
+    if (m % 8 == 0) store8(tile(g), E, l, col0 + m, r + m, k.sc, off, row_used);
   }
   return true;
 }
@@ -414,7 +438,6 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
   using G = Geo<N>;
   using SG = ScanSeg<N>;
   constexpr int E = G::S;  // slab edge
-  uint8_t* const base = shared_base();
   Ctrl* const ctl = shared_ctl();
   const int size = ctl->size;
   const DevSize& S = pb.sz[size];
@@ -429,12 +452,13 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
   const int p = G::kPair ? 0 : l / N;
   const int idx = l - p * N;  // index along the lanes within the block
   const int pmax = G::kPair ? 1 : (n_items + 2 * G::QB - 1) / (2 * G::QB);
-  const bool row_used = l < E && p < pmax;
+  const bool row_used = N == 128 || (l < E && p < pmax);
   const uint32_t t_acc = tmem + ((uint32_t)(32 * quad) << 16) + kColAcc;
   const float ref_u = S.ref_u, ref_v = S.ref_v;
   const float mu_l = l < E ? ctl->mu[idx] : 0.f;
+  // X' = 16 x from D' = 1024 D, with both stages' compensation
   const float kap = (float)N * 0x1p-29f;
-  const float out_scale = 0x1p-7f * (1.f + kap);
+  const float out_scale = 0x1p-6f * (1.f + 2.f * kap);
   const bool slow = ctl->slow != 0;
   // the slot of pair q in slab g: -1 for idle rows and blocks
   auto slot = [&](int g, int q) {
@@ -448,24 +472,26 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
   constexpr int NG = G::kPair ? 1 : 2;  // slabs scanned by one thread
   const int g0 = G::kPair ? (w4 >> 1) : 0;
   const int seg = N >= 48 ? (w4 & 1) : 0;
-  auto alpha_beta = [&](int g, int i, int step, float& alpha, float& beta) {
+  auto alpha_beta = [&](int g, int i, int step, float& alpha, float& beta, float& off) {
     const int s = slot(g, G::kPair ? 0 : block_of(i) >> 1);
     const int f = G::kPair ? g : (block_of(i) & 1);
     alpha = 1.f;
-    beta = 0.f;
+    beta = off = 0.f;
     if (s >= 0) {
       alpha = ctl->rk[s].alpha;
       beta = ctl->beta[growth ? step & 1 : 0][s][f];
+      if (idx == 0) off = ctl->rk[s].off[f];
     }
   };
   ScanCoef sc[NG][G::NB];  // recomputed each step on a growing domain
+  float off[NG][G::NB];
   auto set_coef = [&](int step) {
 #pragma unroll
     for (int g = 0; g < NG; ++g)
 #pragma unroll
       for (int i = 0; i < G::NB; ++i) {
         float alpha, beta;
-        alpha_beta(g0 + g, i, step, alpha, beta);
+        alpha_beta(g0 + g, i, step, alpha, beta, off[g][i]);
         sc[g][i] = scan_coef<N>(alpha, beta, mu_l, out_scale);
       }
   };
@@ -473,7 +499,6 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
   int next_obs = 0;
   for (int step = 0;; ++step) {
     const bool last = step == n_steps;
-    const float sw = step > 0 ? 0x1p-7f * (1.f + kap) : 0x1p-7f;
     const uint32_t ph = (uint32_t)step & 1u;
     const int obs = (next_obs < S.n_obs && step == S.obs_steps[next_obs]) ? next_obs++ : -1;
     if (growth && !last) {  // this step's beta is ready (see grower)
@@ -481,45 +506,67 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
     }
     // ---- observation / output, then the reaction -> stage-1 operands
     if constexpr (G::kPair) {
-      if (step > 0) {  // stage 2 of both slabs: the second commit of a step ends an odd phase
+      // stage 2 of slab 0 (the second commit of a step ends an odd phase) and of
+      // slab 1's first 64 columns; the rest of slab 1 runs under the first half's
+      // reaction
+      if (step > 0) {
         if (!mbar_wait_bounded(&ctl->mma_done[0], 1u, abort, wait_ns)) return;
-        if (!mbar_wait_bounded(&ctl->mma_done[1], 1u, abort, wait_ns)) return;
+        if (!mbar_wait_bounded(&ctl->half_done, ph ^ 1u ^ par.p0, abort, wait_ns)) return;
         tc_fence_after();
       }
-      if (obs >= 0 || last)
+      if (obs >= 0 || last) {
+        if (step > 0) {
+          if (!mbar_wait_bounded(&ctl->mma_done[1], 1u, abort, wait_ns)) return;
+          tc_fence_after();
+        }
         observe(pb, size, slot(0, 0), idx, 8 * w4, 4, (N - 8 * w4 + 31) / 32, t_acc, t_acc + 128u,
-                sw, step, obs, fields, field_stride);
+                step, obs, fields, field_stride);
+      }
       if (last) return;
       const int s = slot(0, 0);
-      React k = {0.f, 0.f, 0.f, 1.f, 0.f, 0.f};
+      React k = {0.f, 0.f, 0.f, 1.f, {0.f, 0.f}};
       if (s >= 0) k = ctl->rk[s];
-      // the whole share is loaded first: the first half's MMAs overwrite the state
-      float u[32], v[32];
-      __syncwarp();
+      // 8-column chunks 32 j + 8 w4, j = 0..3, of both fields, in two halves.  The
+      // first half's MMAs overwrite the state, so the second is loaded before the
+      // first is handed over
+      auto chunk_on = [&](int j) {  // compile-time for all but one j
+        return 32 * j + 32 <= N || (32 * j < N && 32 * j + 8 * w4 < N);
+      };
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = 32 * j + 8 * w4;
-        if (c < N) {
-          tmem_ld8(t_acc + (uint32_t)c, *reinterpret_cast<float(*)[8]>(u + 8 * j));
-          tmem_ld8(t_acc + 128u + (uint32_t)c, *reinterpret_cast<float(*)[8]>(v + 8 * j));
+      for (int hf = 0; hf < 2; ++hf) {
+        if (hf == 1 && step > 0) {  // the rest of slab 1
+          if (!mbar_wait_bounded(&ctl->mma_done[1], 1u, abort, wait_ns)) return;
+          tc_fence_after();
         }
-      }
-      tmem_wait_ld();
-      tc_fence_before();
+        float u[16], v[16];
+        __syncwarp();
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = 32 * j + 8 * w4;
-        if (c < N) {
-          react8(u + 8 * j, v + 8 * j, sw, ref_u, ref_v, k);
-          if (row_used) {
-            store8n<false>(tile(base, 0, 0), tile(base, 0, 1), E, idx, c, u + 8 * j);
-            store8n<false>(tile(base, 1, 0), tile(base, 1, 1), E, idx, c, v + 8 * j);
+        for (int j = 0; j < 2; ++j) {
+          const uint32_t c = (uint32_t)(64 * hf + 32 * j + 8 * w4);
+          if (chunk_on(2 * hf + j)) {
+            tmem_ld8(t_acc + c, *reinterpret_cast<float(*)[8]>(u + 8 * j));
+            tmem_ld8(t_acc + 128u + c, *reinterpret_cast<float(*)[8]>(v + 8 * j));
           }
         }
-        if (j & 1) {
-          fence_proxy_async_smem();
+        tmem_wait_ld();
+        if (hf == 1) {
+          tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&ctl->rx[j >> 1]);
+          if (lane == 0) mbar_arrive(&ctl->rx[0]);
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int c = 64 * hf + 32 * j + 8 * w4;
+          if (chunk_on(2 * hf + j)) {
+            react8(u + 8 * j, v + 8 * j, ref_u, ref_v, k);
+            store8n(tile(0), E, idx, c, u + 8 * j, row_used);
+            store8n(tile(1), E, idx, c, v + 8 * j, row_used);
+          }
+        }
+        fence_proxy_async_smem();
+        if (hf == 1) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&ctl->rx[1]);
         }
       }
     } else {
@@ -537,36 +584,45 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
         const uint32_t t_u = t_acc + (uint32_t)(128 * g + 2 * q * N), t_v = t_u + (uint32_t)N;
         const int s = slot(g, q);
         if (obs >= 0 || last)
-          observe(pb, size, s, idx, c0, CS / 8, c0 + CS < N ? 2 : 1, t_u, t_v, sw, step, obs,
+          observe(pb, size, s, idx, c0, CS / 8, c0 + CS < N ? 2 : 1, t_u, t_v, step, obs,
                   fields, field_stride);
         if (last) continue;
-        React k = {0.f, 0.f, 0.f, 1.f, 0.f, 0.f};
+        React k = {0.f, 0.f, 0.f, 1.f, {0.f, 0.f}};
         if (s >= 0) k = ctl->rk[s];
+        auto chunk_on = [&](int j) { return N != 48 || j == 0 || c0 + CS < N; };
         float u[16], v[16];
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int c = c0 + CS * j;
-          if (c < N) {
+          if (chunk_on(j)) {
             tmem_ld8(t_u + (uint32_t)c, *reinterpret_cast<float(*)[8]>(u + 8 * j));
             tmem_ld8(t_v + (uint32_t)c, *reinterpret_cast<float(*)[8]>(v + 8 * j));
           }
         }
         tmem_wait_ld();
+        const int row = 2 * q * N + idx;
+        uint32_t e = 0;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int c = c0 + CS * j;
-          if (c < N) {
-            react8(u + 8 * j, v + 8 * j, sw, ref_u, ref_v, k);
-            if (row_used) {
-              const int row = 2 * q * N + idx;
-              const bool b1 = store8n<true>(tile(base, g, 0), tile(base, g, 1), E, row, p * N + c,
-                                            u + 8 * j);
-              const bool b2 = store8n<true>(tile(base, g, 0), tile(base, g, 1), E, row + N,
-                                            p * N + c, v + 8 * j);
-              if ((b1 || b2) && s >= 0) ctl->blown[s] = 1;
-            }
+          if (chunk_on(j)) {
+            react8(u + 8 * j, v + 8 * j, ref_u, ref_v, k);
+            e |= store8n(tile(g), E, row, p * N + c, u + 8 * j, row_used);
+            e |= store8n(tile(g), E, row + N, p * N + c, v + 8 * j, row_used);
           }
+        }
+        if ((e & 0x80008000u) && row_used) {  // rare: see the top of the file
+          if (s >= 0) ctl->blown[s] = 1;
+          const uint32_t zero[4] = {0u, 0u, 0u, 0u};
+          for (int j = 0; j < 2; ++j)
+            if (chunk_on(j))
+              for (int f = 0; f < 2; ++f) {
+                const uint32_t a =
+                    tile(g) + sw128_offset(E, row + f * N, p * N + c0 + CS * j);
+                st_shared16(a, zero, true);
+                st_shared16(a + kTileBytes, zero, true);
+              }
         }
         fence_proxy_async_smem();
         tc_fence_before();
@@ -589,14 +645,18 @@ __device__ __forceinline__ void converter(const DevProblem& pb, uint32_t tmem, i
         const uint32_t t = t_acc + (uint32_t)(128 * g + col0);
         if (slow) {
           if (seg == 0) {
-            float alpha, beta;
-            alpha_beta(g, i, step, alpha, beta);
-            slow_row<N>(t, g, E, l, col0, row_used, alpha, beta, mu_l, out_scale);
+            float alpha, beta, o;
+            alpha_beta(g, i, step, alpha, beta, o);
+            slow_row<N>(t, g, E, l, col0, row_used, alpha, beta, mu_l, out_scale, o);
           }
-        } else if (!scan_segment<N>(wait_ns, t, g, seg, G::kPair ? 0 : block_of(i) & 1, quad,
-                                    ph ^ (NG == 2 && gi == 1 ? par.seg >> 1 : par.seg & 1u), lane,
-                                    col0, row_used, sc[gi][i])) {
-          return;
+        } else {
+          float r[SG::H];
+          load_cols<SG::H>(t, r);
+          tmem_wait_ld();
+          if (!scan_segment<N>(wait_ns, r, g, seg, G::kPair ? 0 : block_of(i) & 1, quad,
+                               ph ^ (NG == 2 && gi == 1 ? par.seg >> 1 : par.seg & 1u), lane, col0,
+                               row_used, sc[gi][i], off[gi][i]))
+            return;
         }
       }
       fence_proxy_async_smem();
@@ -634,18 +694,18 @@ __device__ __forceinline__ bool issuer(const DevProblem& pb, uint32_t tmem, int 
       tc_fence_after();
       if (elect_one()) {
         issue_blocks<1, E, true, false, 0, 4, true>(sbase, tmem, 0, N, KB);
-        issue_blocks<1, E, true, false, 0, 4, true>(sbase, tmem, 1, N, KB);
+        issue_blocks<1, E, true, false, 0, 2, true>(sbase, tmem, 1, N, KB);
       }
       __syncwarp();
       if (!mbar_wait_bounded(&ctl->rx[1], ph ^ par.p1, abort, wait_ns)) return false;
       tc_fence_after();
       if (elect_one()) {
-#pragma unroll
-        for (int g = 0; g < 2; ++g) {
-          issue_blocks<1, E, true, false, 4, KB, false>(sbase, tmem, g, N, KB);
-          issue_blocks<1, E, false, true, 0, KB, false>(sbase, tmem, g, N, KB);
-          mma_commit(&ctl->mma_done[g]);
-        }
+        issue_blocks<1, E, true, false, 4, KB, false>(sbase, tmem, 0, N, KB);
+        issue_blocks<1, E, false, true, 0, KB, false>(sbase, tmem, 0, N, KB);
+        mma_commit(&ctl->mma_done[0]);
+        issue_blocks<1, E, true, false, 2, KB, false>(sbase, tmem, 1, N, KB);
+        issue_blocks<1, E, false, true, 0, KB, false>(sbase, tmem, 1, N, KB);
+        mma_commit(&ctl->mma_done[1]);
       }
       __syncwarp();
     } else {
@@ -673,7 +733,13 @@ __device__ __forceinline__ bool issuer(const DevProblem& pb, uint32_t tmem, int 
         return false;
       tc_fence_after();
       if (elect_one()) {
-        issue_blocks<2, E, true, true, 0, KB, true>(sbase, tmem, g, ncols, kb);
+        if (G::kPair && g == 1) {  // in two column halves, see the converters
+          issue_blocks<2, E, true, true, 0, KB, true>(sbase, tmem, g, 64, kb);
+          mma_commit(&ctl->half_done);
+          issue_blocks<2, E, true, true, 0, KB, true, 64>(sbase, tmem, g, N - 64, kb);
+        } else {
+          issue_blocks<2, E, true, true, 0, KB, true>(sbase, tmem, g, ncols, kb);
+        }
         mma_commit(&ctl->mma_done[g]);
       }
       __syncwarp();
@@ -785,13 +851,18 @@ __device__ __forceinline__ void item_constants(const DevProblem& pb, const DevSi
   React k;
   k.fa = (float)th[0];
   k.fb = (float)th[1];
-  k.ftg = (float)(tau * th[3]);
-  k.cu = k.cv = 0.f;
+  k.ftg = (float)(128.0 * tau * th[3]);
+  k.off[0] = k.off[1] = 0.f;
   k.alpha = 1.f;
   if (pb.growth) {
-    k.alpha = (float)(1.0 + tau * 2.0 * th[4]);
-    k.cu = (float)(-tau * 2.0 * th[4] * (double)S.ref_u);
-    k.cv = (float)(-tau * 2.0 * th[4] * (double)S.ref_v);
+    // the constant (1 - alpha) w_ref has the k = 0 coefficient sqrt(N) of it,
+    // which the implicit solve divides by alpha; times 16 and stage 2's
+    // compensation
+    const double al = 1.0 + tau * 2.0 * th[4];
+    const double c = 16.0 * sqrt((double)S.n) * (1.0 - al) / al * (1.0 + S.n * 0x1p-29);
+    k.alpha = (float)al;
+    k.off[0] = (float)(c * (double)S.ref_u);
+    k.off[1] = (float)(c * (double)S.ref_v);
   } else {
     ctl->beta[0][j][0] = (float)(tau * (double)S.n * S.n);
     ctl->beta[0][j][1] = (float)(tau * th[2] * (double)S.n * S.n);
@@ -883,6 +954,7 @@ __device__ __forceinline__ void solve_loop(const DevProblem& pb, const WorkQueue
       mbar_init(&ctl->rx[g], kConvWarps);
       for (int i = 0; i < 8; ++i) mbar_init(&ctl->seg[g][i >> 1][i & 1], 2);
     }
+    mbar_init(&ctl->half_done, 1);
     mbar_init(&ctl->grow, 1);
     mbar_init(&ctl->fin, 1);
     mbar_init(&ctl->never, 1);

@@ -207,30 +207,21 @@ __device__ __forceinline__ float recip_nr(float x) {
   return fmaf(r, fmaf(-x, r, 1.f), r);
 }
 
-// hi = {fp16(a sa), fp16(b sb)} and nlo = the negated rounded remainders
-// {fp16(hi_a - a sa), fp16(hi_b - b sb)}, each as one 32-bit word with the
-// first value in the low half: split_f16 of the two scaled values.  The
-// remainder is one mixed-precision subtraction (FP16 minus FP32, rounded to
-// FP32; exact here) instead of a conversion back to FP32 and a subtraction;
-// an MMA that reads it sets its negate bit.
-__device__ __forceinline__ void split_f16x2_neglo_scaled2(float a, float b, float sa, float sb,
-                                                          uint32_t& hi, uint32_t& nlo) {
-  asm("{\n\t.reg .b64 x, s;\n\t.reg .f32 x0, x1, r0, r1;\n\t"
-      ".reg .b16 h0, h1;\n\t"
-      "mov.b64 x, {%2, %3};\n\t"
-      "mov.b64 s, {%4, %5};\n\t"
-      "mul.rn.f32x2 x, x, s;\n\t"
-      "mov.b64 {x0, x1}, x;\n\t"
-      "cvt.rn.f16x2.f32 %0, x1, x0;\n\t"
-      "mov.b32 {h0, h1}, %0;\n\t"
-      "sub.rn.f32.f16 r0, h0, x0;\n\t"
-      "sub.rn.f32.f16 r1, h1, x1;\n\t"
-      "cvt.rn.f16x2.f32 %1, r1, r0;\n\t}"
-      : "=r"(hi), "=r"(nlo)
-      : "f"(a), "f"(b), "f"(sa), "f"(sb));
+// {a0, a1} * s + o, one rounding per element, by the paired FP32 instruction.
+__device__ __forceinline__ void fma_pair(float& a0, float& a1, float s, float o) {
+  asm("{\n\t.reg .b64 x, y, z;\n\t"
+      "mov.b64 x, {%0, %1};\n\tmov.b64 y, {%2, %2};\n\tmov.b64 z, {%3, %3};\n\t"
+      "fma.rn.f32x2 x, x, y, z;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(s), "f"(o));
 }
-// split_f16x2_neglo_scaled2 of unscaled values: hi = {fp16(a), fp16(b)},
-// nlo = {fp16(hi_a - a), fp16(hi_b - b)}.
+
+// hi = {fp16(a), fp16(b)} and nlo = the negated rounded remainders
+// {fp16(hi_a - a), fp16(hi_b - b)}, each as one 32-bit word with the first value
+// in the low half: split_f16 of the two values.  The remainder is one
+// mixed-precision subtraction (FP16 minus FP32, rounded to FP32; exact here)
+// instead of a conversion back to FP32 and a subtraction; an MMA that reads it
+// sets its negate bit.
 __device__ __forceinline__ void split_f16x2_neglo(float a, float b, uint32_t& hi, uint32_t& nlo) {
   asm("{\n\t.reg .f32 r0, r1;\n\t.reg .b16 h0, h1;\n\t"
       "cvt.rn.f16x2.f32 %0, %3, %2;\n\t"
@@ -240,10 +231,6 @@ __device__ __forceinline__ void split_f16x2_neglo(float a, float b, uint32_t& hi
       "cvt.rn.f16x2.f32 %1, r1, r0;\n\t}"
       : "=r"(hi), "=r"(nlo)
       : "f"(a), "f"(b));
-}
-__device__ __forceinline__ void split_f16x2_neglo_scaled(float a, float b, float s, uint32_t& hi,
-                                                         uint32_t& nlo) {
-  split_f16x2_neglo_scaled2(a, b, s, s, hi, nlo);
 }
 
 }  // namespace tc
