@@ -50,7 +50,7 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "178b48f1a25d16c386255bdc94d6bc14c2b5a64e43c96271ce5ebcaf69284a8c",
+        "sha256": "f35060fe6468805daca0b9c74b0d34c46d5f16000fc5d53c6e07a508c65a96eb",
         "bytes": 1238784 + 2430976,
     },
 }

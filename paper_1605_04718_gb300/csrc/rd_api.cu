@@ -92,6 +92,7 @@ cudaError_t launch_solve_queue(rd_problem* p, const WorkQueue& q, const double* 
     return k == RD_KERNEL_TC_STACKED || k == RD_KERNEL_TC_RESIDENT ? 1000 + p->desc.nx[s] : k;
   };
   bool done[kMaxSizes] = {};
+  bool after_tc = false;
   for (int k0 = 0; k0 < q.n_sizes; ++k0) {
     if (done[k0]) continue;
     const int key = launch_key(q.order[k0]);
@@ -108,12 +109,14 @@ cudaError_t launch_solve_queue(rd_problem* p, const WorkQueue& q, const double* 
     const int grid = (want > 0 && want * p->n_sm < gmax) ? want * p->n_sm : gmax;
     cudaError_t e;
     if (key >= 1000)
-      e = launch_solve_tc(p->dev, sub, theta, phi, status, fields, grid, p->ws.err, st);
+      e = launch_solve_tc(p->dev, sub, theta, phi, status, fields, grid, p->ws.err, st,
+                          after_tc);
     else if (key == RD_KERNEL_CG)
       e = launch_solve_cg(p->dev, sub, theta, phi, status, fields, false, grid, st);
     else
       e = launch_solve_simt(p->dev, sub, theta, phi, status, fields, grid, st);
     if (e != cudaSuccess) return e;
+    after_tc = key >= 1000;
   }
   return cudaSuccess;
 }

@@ -112,12 +112,13 @@ cudaError_t launch_solve_1d(const DevProblem& pb, const WorkQueue& q, const doub
                             double* phi, uint32_t* status, void* fields, int grid,
                             cudaStream_t st, int* steps_out);
 // Tensor-core solve (rd_solve_tc2.cu): every size in its queue must be the same
-// N x N grid, N a multiple of 16 up to 128.
+// N x N grid, N a multiple of 16 up to 128.  after_tc: the launch before it in
+// the stream is another size's of the same batch.
 cudaError_t setup_solve_tc(int n);
 int grid_solve_tc(int n_sm);
 cudaError_t launch_solve_tc(const DevProblem& pb, const WorkQueue& q, const double* theta,
                             double* phi, uint32_t* status, void* fields, int grid, int* err,
-                            cudaStream_t st);
+                            cudaStream_t st, bool after_tc);
 // CUDA-core conjugate-gradient solves (rd_solve_simt.cu): the IMEX step by
 // plain CG (RD_KERNEL_CG, N <= 96) or the paper's semi-implicit step by
 // preconditioned CG (picard, N <= 80).

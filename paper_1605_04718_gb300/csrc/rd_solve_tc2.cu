@@ -69,8 +69,8 @@
 // N <= 64: the block-diagonal A multiplies other proposals' data by zero, so a
 // reaction value outside the FP16 range (a diverging solve) must not reach the
 // MMA as infinity (nor reach the scan as one: |r| >= 256): it is stored as zero, and
-// every later observation or output
-// of its proposal reads NaN, which is what an infinite operand leads to.
+// every later observation or output of its proposal reads NaN, which is what an
+// infinite operand leads to.
 //
 // Every wait is bounded; a timed-out wait makes the CTA leave, drain its MMAs,
 // free its TMEM and raise the error flag.
@@ -965,6 +965,9 @@ __device__ __forceinline__ void solve_loop(const DevProblem& pb, const WorkQueue
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  // a batch of several grid sizes is one launch per size: the next one's CTAs may
+  // take the SMs that this one does not fill or has left
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const uint32_t tmem = ctl->tmem_base;
   // every size of this launch is N x N: one DCT matrix serves all
   if (warp < kConvWarps) fill_constants<N>(pb.sz[q.order[0]], tmem, warp, lane);
@@ -1011,6 +1014,8 @@ __device__ __forceinline__ void solve_loop(const DevProblem& pb, const WorkQueue
     tmem_dealloc(tmem, 512);
   }
   if (tid == 0 && ctl->abort) atomicOr(err, 1);
+  // ... and this launch ends no sooner than the one before it
+  if (blockIdx.x == 0 && tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace tc2
@@ -1055,14 +1060,27 @@ int grid_solve_tc(int n_sm) { return n_sm; }
 
 cudaError_t launch_solve_tc(const DevProblem& pb, const WorkQueue& q, const double* theta,
                             double* phi, uint32_t* status, void* fields, int grid, int* err,
-                            cudaStream_t st) {
+                            cudaStream_t st, bool after_tc) {
   size_t stride = (size_t)2 * pb.max_n * pb.max_n;
   DevProblem pbv = pb;
   WorkQueue qv = q;
   float* fo = (float*)fields;
   void* args[] = {&pbv, &qv, (void*)&theta, &phi, &status, &fo, &stride, &err};
-  return cudaLaunchKernel(tc_kernel(pb.sz[q.order[0]].n), dim3(grid), dim3(tc2::kThreads), args,
-                          tc2::kSmemBytes, st);
+  // A launch that follows another size's only needs what both read (the queue and
+  // the parameters, written before the first of them) and may start early: 512
+  // proposals of each of 64^2, 96^2 and 128^2, 400 steps, 18.26 -> 16.04 ms; 12
+  // of each, 300 steps, take 1.82 ms, no longer than the 12 of 128^2 alone.
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(tc2::kThreads);
+  cfg.dynamicSmemBytes = tc2::kSmemBytes;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = after_tc ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, tc_kernel(pb.sz[q.order[0]].n), args);
 }
 
 }  // namespace rd

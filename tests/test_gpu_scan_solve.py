@@ -96,3 +96,23 @@ def test_parameters_outside_the_scan_match_the_cuda_core_kernel(n):
     for i in range(8):
         assert sa[i] == 0
         assert H.rel_l2(fa[i], fb[i]) < 2e-5, i
+
+
+def test_chains_over_several_sizes_hold_the_phi_of_their_state():
+    """One launch per size, started before the previous one ends, inside the
+    captured step: every chain's stored Phi is that of its own state and size."""
+    dss = [H.small_dataset(n, 30, seed=n, sigma=0.3) for n in (128, 32, 80)]
+    p = H.gpu_problem(dss, solver=rd.RD_SOLVER_AUTO)
+    C = 23
+    size_idx = np.arange(C) % 3
+    theta0 = rd_synth.lognormal_draws(TRUE4, [0.05] * 4, C, seed=5)
+    c = rd.rd_chains_create(p, theta0, 7, [0.02] * 4, size_idx=size_idx, capacity=8)
+    for _ in range(3):
+        rd.rd_chains_run(c, 2)
+    samples, counters = rd.rd_chains_read_samples(c, 6, 4, C)
+    th, phi = rd.rd_chains_get_state(c, 4, C)
+    assert counters[2] > 0 and np.array_equal(samples[-1].T, th)
+    got, st = rd.rd_evaluate_batch_host(p, th, size_idx=size_idx)
+    rd.rd_chains_destroy(c)
+    rd.rd_problem_destroy(p)
+    assert np.all(st == 0) and np.all(np.abs(got - phi) <= 1e-12 * phi)
