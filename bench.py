@@ -50,7 +50,7 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "f35060fe6468805daca0b9c74b0d34c46d5f16000fc5d53c6e07a508c65a96eb",
+        "sha256": "8ceb430559a377c3b06d2fc0df01d9b32aaaf95435c5b725a4d53ae8853bd916",
         "bytes": 1238784 + 2430976,
     },
 }

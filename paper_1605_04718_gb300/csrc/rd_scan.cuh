@@ -51,8 +51,8 @@ __device__ __forceinline__ float ipow(float x) {
   }
 }
 
-// Coefficients of one mode; N a multiple of 16.
-template <int N>
+// Coefficients of one mode; N a multiple of 16, H the segments' length.
+template <int N, int H = ScanSeg<N>::H>
 __device__ __forceinline__ ScanCoef scan_coef(float alpha, float beta, float mu, float out_scale) {
   ScanCoef c;
   const float lam = fmaf(beta, mu, alpha);
@@ -65,7 +65,7 @@ __device__ __forceinline__ ScanCoef scan_coef(float alpha, float beta, float mu,
   c.a = a;
   c.sc = __fdiv_rn(om * om, lam) * out_scale;
   c.g = __frcp_rn(om * (1.f + a));
-  c.ah = ipow<ScanSeg<N>::H>(a);
+  c.ah = ipow<H>(a);
   c.an = ipow<N>(a);
   // 1 - a^(2N) = (1 - a)(1 + a)(1 + a^2)...(1 + a^16)(1 + a^32 + ... ): no
   // cancellation for a near 1

@@ -31,7 +31,10 @@ namespace rd {
 //    N <= 80.
 // Fields are held as deviations from the initial-state mean as in the
 // eigenbasis kernel; for the Picard step that turns the rhs into
-// w^n - ref + tau gamma c + ref (1 - D).  Dot products are FP64.  A solve
+// w^n - ref + tau gamma c + ref (1 - D).  Dot products are
+// compensated pair sums (46 bits), the iteration's scalars FP64 in one thread: as
+// FP64 sums they took most of a step, 152 proposals of 64^2, 30 semi-implicit
+// steps 3.02 ms against 1.43 with them and the preconditioner's scan.  A solve
 // that reaches its iteration cap marks the proposal RD_P_NOT_CONVERGED.
 // ---------------------------------------------------------------------------
 constexpr int kCgMaxIter = 300;     // IMEX: plain CG
@@ -52,68 +55,87 @@ __device__ __forceinline__ void apply_op(const float* P, float* Q, float beta, D
   }
 }
 
+// Sum over all points of term(offset, sum) and f of it (in thread 0), to every
+// thread.
+template <int N, class T, class F>
+__device__ __forceinline__ double reduce_points(RedScratch* red, T&& term, F&& f) {
+  Pair part;
+  for (int i = threadIdx.x; i < N * N; i += kSimtThreads) term((i / N) * (N + 1) + i % N, part);
+  return cta_reduce(part, red, f);
+}
+
 // CG on [diag(dg) - beta Lap_h] X = b from the X given, R = b - A X on entry;
-// P, Q scratch; bb = |b|^2.  Returns false at the iteration cap.
+// P, Q scratch; bb = |b|^2 (thread 0's).  Returns false at the iteration cap.
+// The FP64 scalars of the iteration live in thread 0.
 template <int N, class Dg>
 __device__ bool cg_solve(float* X, float* R, float* P, float* Q, float beta, Dg dg, double bb,
-                         double* red) {
+                         RedScratch* red) {
   constexpr int NP = N + 1;
   const int tid = threadIdx.x;
-  double part = 0.0;
-  for (int i = tid; i < N * N; i += kSimtThreads) {
-    const int o = (i / N) * NP + i % N;
-    P[o] = R[o];
-    part += (double)R[o] * (double)R[o];
-  }
-  double rr = cta_sum_all(part, red);
   const double stop = kCgTol * kCgTol * bb;
+  double rr = 0.0;
+  bool done = reduce_points<N>(
+                  red,
+                  [&](int o, Pair& s) {
+                    P[o] = R[o];
+                    s.add_product(R[o], R[o]);
+                  },
+                  [&](double x) {
+                    rr = x;
+                    return x <= stop ? 1.0 : 0.0;
+                  }) != 0.0;
   for (int it = 0; it < kCgMaxIter; ++it) {
-    if (rr <= stop) return true;
+    if (done) return true;
     apply_op<N>(P, Q, beta, dg);
     __syncthreads();
-    part = 0.0;
+    const float al = (float)reduce_points<N>(
+        red, [&](int o, Pair& s) { s.add_product(P[o], Q[o]); },
+        [&](double pq) { return rr / pq; });
+    double be = reduce_points<N>(
+        red,
+        [&](int o, Pair& s) {
+          X[o] = fmaf(al, P[o], X[o]);
+          const float r = fmaf(-al, Q[o], R[o]);
+          R[o] = r;
+          s.add_product(r, r);
+        },
+        [&](double x) {
+          const double ratio = x / rr;
+          rr = x;
+          return x <= stop ? -1.0 : ratio;  // a ratio is not negative
+        });
+    done = be < 0.0;
+    if (done) return true;
+    const float bf = (float)be;
     for (int i = tid; i < N * N; i += kSimtThreads) {
       const int o = (i / N) * NP + i % N;
-      part += (double)P[o] * (double)Q[o];
-    }
-    const double pq = cta_sum_all(part, red);
-    const float al = (float)(rr / pq);
-    part = 0.0;
-    for (int i = tid; i < N * N; i += kSimtThreads) {
-      const int o = (i / N) * NP + i % N;
-      X[o] = fmaf(al, P[o], X[o]);
-      const float r = fmaf(-al, Q[o], R[o]);
-      R[o] = r;
-      part += (double)r * (double)r;
-    }
-    const double rr_new = cta_sum_all(part, red);
-    const float be = (float)(rr_new / rr);
-    rr = rr_new;
-    for (int i = tid; i < N * N; i += kSimtThreads) {
-      const int o = (i / N) * NP + i % N;
-      P[o] = fmaf(be, P[o], R[o]);
+      P[o] = fmaf(bf, P[o], R[o]);
     }
     __syncthreads();
   }
-  return rr <= stop;
+  return false;
 }
 
 // Preconditioned CG on [diag(dg) - beta Lap_h] X = b, M = [dm I - beta
 // Lap_h] solved in the eigenbasis; R = b on entry.  X = M^-1 b first.
 template <int N, class Dg>
 __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, const float* Cm,
-                          float beta, float dm, Dg dg, const float (&mur)[N / 16],
-                          const float (&muc)[N / 16], double* red) {
+                          float beta, float dm, Dg dg, const float* mu, float2* sums,
+                          RedScratch* red) {
   constexpr int NP = N + 1;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  double part = 0.0;
-  for (int i = tid; i < N * N; i += kSimtThreads) {
-    const int o = (i / N) * NP + i % N;
-    Z[o] = R[o];
-    part += (double)R[o] * (double)R[o];
-  }
-  const double bb = cta_sum_all(part, red);
-  implicit_solve_simt<N>(Z, Cm, dm, beta, mur, muc, ty, tx);  // x0 = M^-1 b
+  double stop = 0.0, rz = 0.0;  // thread 0's
+  reduce_points<N>(
+      red,
+      [&](int o, Pair& s) {
+        Z[o] = R[o];
+        s.add_product(R[o], R[o]);
+      },
+      [&](double bb) {
+        stop = kCgTol * kCgTol * bb;
+        return 0.0;
+      });
+  implicit_solve_simt<N>(Z, Cm, dm, beta, mu, sums, ty, tx);  // x0 = M^-1 b
   for (int i = tid; i < N * N; i += kSimtThreads) {
     const int o = (i / N) * NP + i % N;
     X[o] = Z[o];
@@ -121,55 +143,49 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
   __syncthreads();
   apply_op<N>(X, Q, beta, dg);
   __syncthreads();
-  part = 0.0;
-  for (int i = tid; i < N * N; i += kSimtThreads) {
-    const int o = (i / N) * NP + i % N;
-    const float r = R[o] - Q[o];
-    R[o] = r;
-    Z[o] = r;
-    part += (double)r * (double)r;
-  }
-  double rr = cta_sum_all(part, red);
-  const double stop = kCgTol * kCgTol * bb;
-  if (rr <= stop) return true;
-  implicit_solve_simt<N>(Z, Cm, dm, beta, mur, muc, ty, tx);
-  part = 0.0;
-  for (int i = tid; i < N * N; i += kSimtThreads) {
-    const int o = (i / N) * NP + i % N;
-    P[o] = Z[o];
-    part += (double)R[o] * (double)Z[o];
-  }
-  double rz = cta_sum_all(part, red);
+  // R <- the residual, Z its copy for the preconditioner; whether it is small
+  auto residual = [&](float al, const float* V) {
+    return reduce_points<N>(
+               red,
+               [&](int o, Pair& s) {
+                 const float r = fmaf(-al, V[o], R[o]);
+                 R[o] = r;
+                 Z[o] = r;
+                 s.add_product(r, r);
+               },
+               [&](double rr) { return rr <= stop ? 1.0 : 0.0; }) != 0.0;
+  };
+  if (residual(1.f, Q)) return true;
+  implicit_solve_simt<N>(Z, Cm, dm, beta, mu, sums, ty, tx);
+  reduce_points<N>(
+      red,
+      [&](int o, Pair& s) {
+        P[o] = Z[o];
+        s.add_product(R[o], Z[o]);
+      },
+      [&](double x) {
+        rz = x;
+        return 0.0;
+      });
   for (int it = 0; it < kPcgMaxIter; ++it) {
     apply_op<N>(P, Q, beta, dg);
     __syncthreads();
-    part = 0.0;
-    for (int i = tid; i < N * N; i += kSimtThreads) {
-      const int o = (i / N) * NP + i % N;
-      part += (double)P[o] * (double)Q[o];
-    }
-    const double pq = cta_sum_all(part, red);
-    const float al = (float)(rz / pq);
-    part = 0.0;
+    const float al = (float)reduce_points<N>(
+        red, [&](int o, Pair& s) { s.add_product(P[o], Q[o]); },
+        [&](double pq) { return rz / pq; });
     for (int i = tid; i < N * N; i += kSimtThreads) {
       const int o = (i / N) * NP + i % N;
       X[o] = fmaf(al, P[o], X[o]);
-      const float r = fmaf(-al, Q[o], R[o]);
-      R[o] = r;
-      Z[o] = r;
-      part += (double)r * (double)r;
     }
-    rr = cta_sum_all(part, red);
-    if (rr <= stop) return true;
-    implicit_solve_simt<N>(Z, Cm, dm, beta, mur, muc, ty, tx);
-    part = 0.0;
-    for (int i = tid; i < N * N; i += kSimtThreads) {
-      const int o = (i / N) * NP + i % N;
-      part += (double)R[o] * (double)Z[o];
-    }
-    const double rz_new = cta_sum_all(part, red);
-    const float be = (float)(rz_new / rz);
-    rz = rz_new;
+    if (residual(al, Q)) return true;
+    implicit_solve_simt<N>(Z, Cm, dm, beta, mu, sums, ty, tx);
+    const float be = (float)reduce_points<N>(
+        red, [&](int o, Pair& s) { s.add_product(R[o], Z[o]); },
+        [&](double x) {
+          const double ratio = x / rz;
+          rz = x;
+          return ratio;
+        });
     for (int i = tid; i < N * N; i += kSimtThreads) {
       const int o = (i / N) * NP + i % N;
       P[o] = fmaf(be, P[o], Z[o]);
@@ -181,9 +197,9 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
 
 template <int N, bool PICARD>
 __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const double th[kNPhys],
-                                float* sm, double* red, double* phi_out, uint32_t* st_out,
-                                float* fields_out) {
-  constexpr int TM = N / 16, NP = N + 1, NPTS = N * N, VS = N * NP;
+                                float* sm, RedScratch* red, double* red64, float2* sums, double* phi_out,
+                                uint32_t* st_out, float* fields_out) {
+  constexpr int NP = N + 1, NPTS = N * N, VS = N * NP;
   float* U = sm;
   float* V = sm + VS;
   float* R = sm + 2 * VS;
@@ -192,19 +208,13 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
   float* W = sm + 5 * VS;  // IMEX: rhs of v; Picard: the new u
   float* Z = sm + 6 * VS;  // Picard only
   float* Cm = sm + 7 * VS; // Picard only
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const int tid = threadIdx.x;
   const float ref_u = S.ref_u, ref_v = S.ref_v;
   for (int i = tid; i < NPTS; i += kSimtThreads) {
     const int y = i / N, x = i - y * N, o = y * NP + x;
     U[o] = S.u0f[i] - ref_u;
     V[o] = S.v0f[i] - ref_v;
     if (PICARD) Cm[o] = S.cmat[i];
-  }
-  float mur[TM], muc[TM];
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    mur[i] = S.mu[ty + 16 * i];
-    muc[i] = S.mu[tx + 16 * i];
   }
   const double d = th[2], r = th[4], tau = pb.tau;
   const float fa = (float)th[0], fb = (float)th[1], ftg = (float)(tau * th[3]);
@@ -229,29 +239,34 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
       auto dga = [alpha](int) { return alpha; };
       apply_op<N>(U, Q, bu, dga);
       __syncthreads();
-      double part = 0.0;
-      for (int i = tid; i < NPTS; i += kSimtThreads) {
-        const int o = (i / N) * NP + i % N;
-        const float du = U[o], dv = V[o];
-        const float uu = ref_u + du, vv = ref_v + dv;
-        const float u2v = uu * uu * vv;
-        const float rhs_u = fmaf(ftg, fa - uu + u2v, du) + cu;
-        W[o] = fmaf(ftg, fb - u2v, dv) + cv;
-        R[o] = rhs_u - Q[o];
-        part += (double)rhs_u * (double)rhs_u;
-      }
-      const double bbu = cta_sum_all(part, red);
-      conv &= cg_solve<N>(U, R, P, Q, bu, dga, bbu, red);
+      double bb = 0.0;  // |rhs|^2 (thread 0's)
+      auto keep = [&](double x) {
+        bb = x;
+        return 0.0;
+      };
+      reduce_points<N>(
+          red,
+          [&](int o, Pair& s) {
+            const float du = U[o], dv = V[o];
+            const float uu = ref_u + du, vv = ref_v + dv;
+            const float u2v = uu * uu * vv;
+            const float rhs_u = fmaf(ftg, fa - uu + u2v, du) + cu;
+            W[o] = fmaf(ftg, fb - u2v, dv) + cv;
+            R[o] = rhs_u - Q[o];
+            s.add_product(rhs_u, rhs_u);
+          },
+          keep);
+      conv &= cg_solve<N>(U, R, P, Q, bu, dga, bb, red);
       apply_op<N>(V, Q, bv, dga);
       __syncthreads();
-      part = 0.0;
-      for (int i = tid; i < NPTS; i += kSimtThreads) {
-        const int o = (i / N) * NP + i % N;
-        R[o] = W[o] - Q[o];
-        part += (double)W[o] * (double)W[o];
-      }
-      const double bbv = cta_sum_all(part, red);
-      conv &= cg_solve<N>(V, R, P, Q, bv, dga, bbv, red);
+      reduce_points<N>(
+          red,
+          [&](int o, Pair& s) {
+            R[o] = W[o] - Q[o];
+            s.add_product(W[o], W[o]);
+          },
+          keep);
+      conv &= cg_solve<N>(V, R, P, Q, bv, dga, bb, red);
     } else {
       // Picard: diagonals from u^n, v^n; mean diagonal for the preconditioner
       auto dg_u = [=](int o) {
@@ -261,24 +276,24 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
         const float uu = ref_u + U[o];
         return alpha + ftg * uu * uu;
       };
-      double su = 0.0, sv = 0.0;
-      for (int i = tid; i < NPTS; i += kSimtThreads) {
-        const int o = (i / N) * NP + i % N;
-        const float du = dg_u(o);
-        su += du;
-        sv += dg_v(o);
-        R[o] = U[o] + ftg * fa + ref_u * (1.f - du);
-      }
-      const float mu_u = (float)(cta_sum_all(su, red) / NPTS);
-      const float mu_v = (float)(cta_sum_all(sv, red) / NPTS);
-      conv &= pcg_solve<N>(W, R, Z, P, Q, Cm, bu, mu_u, dg_u, mur, muc, red);
+      const float mu_u = (float)reduce_points<N>(
+          red,
+          [&](int o, Pair& s) {
+            const float du = dg_u(o);
+            s.add(du);
+            R[o] = U[o] + ftg * fa + ref_u * (1.f - du);
+          },
+          [](double x) { return x / NPTS; });
+      const float mu_v = (float)reduce_points<N>(
+          red, [&](int o, Pair& s) { s.add(dg_v(o)); }, [](double x) { return x / NPTS; });
+      conv &= pcg_solve<N>(W, R, Z, P, Q, Cm, bu, mu_u, dg_u, S.mu, sums, red);
       for (int i = tid; i < NPTS; i += kSimtThreads) {
         const int o = (i / N) * NP + i % N;
         R[o] = V[o] + ftg * fb + ref_v * (1.f - dg_v(o));
       }
       __syncthreads();
       // v^{n+1} into V: its diagonal needs only u^n, which U still holds
-      conv &= pcg_solve<N>(V, R, Z, P, Q, Cm, bv, mu_v, dg_v, mur, muc, red);
+      conv &= pcg_solve<N>(V, R, Z, P, Q, Cm, bv, mu_v, dg_v, S.mu, sums, red);
       for (int i = tid; i < NPTS; i += kSimtThreads) {
         const int o = (i / N) * NP + i % N;
         U[o] = W[o];
@@ -305,7 +320,7 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
       ++next_obs;
     }
   }
-  const double tot = cta_sum(phi, red);
+  const double tot = cta_sum(phi, red64);
   const int any_bad = __syncthreads_or(bad);
   if (tid == 0) {
     const uint32_t st = (any_bad ? (uint32_t)RD_P_NONFINITE : 0u) |
@@ -326,7 +341,8 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
 #define RD_CG_CASE(NN)                                                              \
   case NN:                                                                          \
     if constexpr (NN <= NMAX)                                                       \
-      solve2d_cg_item<NN, PICARD>(pb, S, th, sm, red, &phi[b], &status[b], fo);     \
+      solve2d_cg_item<NN, PICARD>(pb, S, th, sm, &red, red64, sums, &phi[b], &status[b], \
+                                  fo);                                             \
     break;
 
 template <int NMAX, bool PICARD>
@@ -334,7 +350,9 @@ __global__ void __launch_bounds__(kSimtThreads, 1)
     k_solve2d_cg(DevProblem pb, WorkQueue q, const double* theta, double* phi,
                  uint32_t* status, float* fields, size_t field_stride) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ double red[kSimtThreads / 32];
+  __shared__ RedScratch red;
+  __shared__ double red64[kSimtThreads / 32];
+  __shared__ float2 sums[kSimtThreads];
   __shared__ int s_item, s_size;
   for (;;) {
     if (threadIdx.x == 0) {

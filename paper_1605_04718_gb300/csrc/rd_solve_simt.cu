@@ -34,10 +34,11 @@ namespace rd {
 // a Turing pattern grows from the initial noise) instead of on |w| ~ 1,
 // which keeps the small unstable modes accurate.
 //
-// Implicit solve by diagonalisation in the Neumann eigenbasis (orthonormal
-// DCT-II, C[k][i] = c_k cos(pi k (i + 1/2) / N)):
-//   P = W C^T, Q = C P, S = Q / (alpha + beta (mu_l + mu_k)), W1 = C^T S,
-//   W = W1 C,   mu_k = 4 sin^2(pi k / (2N)), beta = tau D / (rho^2 h^2).
+// Implicit solve: the Neumann eigenbasis (orthonormal DCT-II, C[k][i] =
+// c_k cos(pi k (i + 1/2) / N)) along x and a tridiagonal scan along y
+// (implicit_solve_simt):
+//   P = W C^T, S[.][k] = [(alpha + beta mu_k) I - beta Lap_1D]^-1 P[.][k], W = S C,
+//   mu_k = 4 sin^2(pi k / (2N)), beta = tau D / (rho^2 h^2).
 // Each product is an N x N x N GEMM from shared memory with 16 x 16 threads,
 // thread (ty, tx) owning rows ty + 16 i and columns tx + 16 j.  Rows are
 // padded to N + 1 floats so that every operand load is conflict-free.
@@ -46,10 +47,10 @@ namespace rd {
 // with the previous step (then w(T)) in two more shared-memory arrays.
 template <int N, bool STEADY>
 __device__ void solve2d_simt_item(const DevProblem& pb, const DevSize& S,
-                                  const double th[kNPhys], float* sm, double* red,
+                                  const double th[kNPhys], float* sm, double* red, float2* sums,
                                   double* phi_out, uint32_t* st_out,
                                   float* fields_out, int* steps_out) {
-  constexpr int TM = N / 16, NP = N + 1, NPTS = N * N;
+  constexpr int NP = N + 1, NPTS = N * N;
   float* U = sm;  // u - ref_u
   float* V = sm + N * NP;  // v - ref_v
   float* Cm = sm + 2 * N * NP;
@@ -62,12 +63,6 @@ __device__ void solve2d_simt_item(const DevProblem& pb, const DevSize& S,
     Cm[r * NP + c] = S.cmat[i];
     U[r * NP + c] = S.u0f[i] - ref_u;
     V[r * NP + c] = S.v0f[i] - ref_v;
-  }
-  float mur[TM], muc[TM];
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    mur[i] = S.mu[ty + 16 * i];
-    muc[i] = S.mu[tx + 16 * i];
   }
   const double d = th[2], r = th[4], tau = pb.tau;
   const float fa = (float)th[0], fb = (float)th[1], ftg = (float)(tau * th[3]);
@@ -105,8 +100,8 @@ __device__ void solve2d_simt_item(const DevProblem& pb, const DevSize& S,
       V[o] = fmaf(ftg, fb - u2v, dv) + cv;
     }
     __syncthreads();
-    implicit_solve_simt<N>(U, Cm, alpha, bu, mur, muc, ty, tx);
-    implicit_solve_simt<N>(V, Cm, alpha, bv, mur, muc, ty, tx);
+    implicit_solve_simt<N>(U, Cm, alpha, bu, S.mu, sums, ty, tx);
+    implicit_solve_simt<N>(V, Cm, alpha, bv, S.mu, sums, ty, tx);
     bool observe = !STEADY && next_obs < S.n_obs && step + 1 == S.obs_steps[next_obs];
     bool stop = false;
     if (STEADY) {
@@ -187,8 +182,8 @@ __device__ void solve2d_simt_item(const DevProblem& pb, const DevSize& S,
 #define RD_SIMT_CASE(NN)                                                      \
   case NN:                                                                    \
     if constexpr (NN <= NMAX)                                                 \
-      solve2d_simt_item<NN, STEADY>(pb, S, th, sm, red, &phi[b], &status[b], fo, \
-                                    steps_out ? &steps_out[b] : nullptr);     \
+      solve2d_simt_item<NN, STEADY>(pb, S, th, sm, red, sums, &phi[b], &status[b], \
+                                    fo, steps_out ? &steps_out[b] : nullptr);     \
     break;
 
 // NMAX: largest grid of the problem; sizes up to NMAX share one launch.
@@ -198,6 +193,7 @@ __global__ void __launch_bounds__(kSimtThreads, MINB)
                    uint32_t* status, float* fields, size_t field_stride, int* steps_out) {
   extern __shared__ __align__(16) float sm[];
   __shared__ double red[kSimtThreads / 32];
+  __shared__ float2 sums[kSimtThreads];
   __shared__ int s_item, s_size;
   for (;;) {
     if (threadIdx.x == 0) {
