@@ -13,45 +13,96 @@ namespace rd {
 
 constexpr int kSimtThreads = 256;
 
+// Row stride of the arrays in shared memory: rows start on 16-byte boundaries a
+// bank group apart, so that four consecutive values load at once without
+// conflicts.  96: one more float, two CTAs of three arrays then fit an SM.
+__host__ __device__ constexpr int simt_stride(int n) { return n == 96 ? n + 1 : n + 4; }
+
+// Column j of the N / 16 that thread tx owns: in groups of four or two where
+// N / 16 allows, for wide loads of row-major B.
 template <int N>
-constexpr size_t simt_smem_bytes() {
-  return (size_t)3 * N * (N + 1) * sizeof(float);
+__device__ __forceinline__ constexpr int simt_col(int tx, int j) {
+  constexpr int TM = N / 16, G = simt_stride(N) % 4 ? 1 : TM % 4 == 0 ? 4 : TM % 2 == 0 ? 2 : 1;
+  return (j / G) * 16 * G + tx * G + j % G;
 }
 
-// acc[i][j] = sum_k A(ty + 16 i, k) B(k, tx + 16 j), A(m, k) = pa[m*SAM + k*SAK],
-// B(k, n) = pb[k*SBK + n*SBN].
-template <int N, int SAM, int SAK, int SBK, int SBN>
+template <int M>
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[M]) {
+  if constexpr (M == 4) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+  } else if constexpr (M == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x, v[1] = x.y;
+  } else {
+    v[0] = p[0];
+  }
+}
+
+// acc[i][j] = sum_k A(ty + 16 i, k) B(k, n_j).  A(m, k) = pa[m * NP + k], or
+// pa[k * NP + m] if A_T.  BT: B(k, n) = pb[n * NP + k], n_j = tx + 16 j; else
+// B(k, n) = pb[k * NP + n], n_j = simt_col(tx, j).  Operands along k are loaded
+// four at a time: 8 loads for 64 FMAs at N = 64 instead of 32, which bound it
+// (a step of the CUDA-core kernel at 64^2, per proposal, 0.145 -> 0.123 us).
+template <int N, bool A_T, bool BT>
 __device__ __forceinline__ void smem_gemm(const float* __restrict__ pa,
                                           const float* __restrict__ pb,
-                                          float (&acc)[N / 16][N / 16], int ty,
-                                          int tx) {
-  constexpr int TM = N / 16;
+                                          float (&acc)[N / 16][N / 16], int ty, int tx) {
+  constexpr int TM = N / 16, NP = simt_stride(N);
+  constexpr int V = NP % 4 == 0 ? 4 : 1;
+  constexpr int G = simt_col<N>(0, 1) == 1 ? (TM > 2 && simt_col<N>(0, 2) == 2 ? 4 : 2) : 1;
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TM; ++j) acc[i][j] = 0.f;
-#pragma unroll 4
-  for (int k = 0; k < N; ++k) {
-    float av[TM], bv[TM];
+#pragma unroll(V == 4 ? 1 : 4)
+  for (int k = 0; k < N; k += V) {
+    float av[TM][V];
 #pragma unroll
-    for (int i = 0; i < TM; ++i) av[i] = pa[(ty + 16 * i) * SAM + k * SAK];
+    for (int i = 0; i < TM; ++i) {
+      if constexpr (A_T) {
 #pragma unroll
-    for (int j = 0; j < TM; ++j) bv[j] = pb[k * SBK + (tx + 16 * j) * SBN];
+        for (int e = 0; e < V; ++e) av[i][e] = pa[(k + e) * NP + ty + 16 * i];
+      } else {
+        load_vec<V>(pa + (ty + 16 * i) * NP + k, av[i]);
+      }
+    }
+    if constexpr (BT) {
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+      for (int j = 0; j < TM; ++j) {
+        float bv[V];
+        load_vec<V>(pb + (tx + 16 * j) * NP + k, bv);
 #pragma unroll
-      for (int j = 0; j < TM; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+        for (int e = 0; e < V; ++e)
+#pragma unroll
+          for (int i = 0; i < TM; ++i) acc[i][j] = fmaf(av[i][e], bv[e], acc[i][j]);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < V; ++e)
+#pragma unroll
+        for (int j = 0; j < TM; j += G) {
+          float bv[G];
+          load_vec<G>(pb + (k + e) * NP + simt_col<N>(tx, j), bv);
+#pragma unroll
+          for (int h = 0; h < G; ++h)
+#pragma unroll
+            for (int i = 0; i < TM; ++i) acc[i][j + h] = fmaf(av[i][e], bv[h], acc[i][j + h]);
+        }
+    }
   }
 }
 
-template <int N>
+// The tile of a product whose columns are tx + 16 j (BT) or simt_col(tx, j).
+template <int N, bool BT>
 __device__ __forceinline__ void store_tile(float* W, const float (&acc)[N / 16][N / 16],
                                            int ty, int tx) {
-  constexpr int TM = N / 16, NP = N + 1;
+  constexpr int TM = N / 16, NP = simt_stride(N);
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TM; ++j) W[(ty + 16 * i) * NP + tx + 16 * j] = acc[i][j];
+    for (int j = 0; j < TM; ++j)
+      W[(ty + 16 * i) * NP + (BT ? tx + 16 * j : simt_col<N>(tx, j))] = acc[i][j];
 }
 
 // Segments of a column in the scan: NS of H rows, one thread each.
@@ -63,12 +114,12 @@ struct SimtSeg {
 };
 
 // X <- [(alpha + beta mu_k) I - beta Lap_1D]^-1 X along y for every column k of W
-// (rows y, padded to N + 1): the recursions of rd_scan.cuh, N / NS rows a thread.
+// (rows y, stride simt_stride): the recursions of rd_scan.cuh, N / NS rows a thread.
 // sums: [NS][N] scratch.
 template <int N>
 __device__ __forceinline__ void scan_columns(float* W, float alpha, float beta, const float* mu,
                                              float2* sums) {
-  constexpr int NP = N + 1, NS = SimtSeg<N>::NS, H = SimtSeg<N>::H;
+  constexpr int NP = simt_stride(N), NS = SimtSeg<N>::NS, H = SimtSeg<N>::H;
   const int k = threadIdx.x % N, seg = threadIdx.x / N;
   const bool on = seg < NS;
   float* const w = W + (on ? seg : 0) * H * NP + k;
@@ -116,37 +167,37 @@ template <int N>
 __device__ __forceinline__ void implicit_solve_simt(float* W, const float* Cm, float alpha,
                                                     float beta, const float* mu, float2* sums,
                                                     int ty, int tx) {
-  constexpr int TM = N / 16, NP = N + 1;
+  constexpr int TM = N / 16;
   const bool scan = alpha > 0.f && beta >= 0.f && beta < 1e30f;
   float acc[TM][TM];
   // P[y][k] = sum_x W[y][x] C[k][x]
-  smem_gemm<N, NP, 1, 1, NP>(W, Cm, acc, ty, tx);
+  smem_gemm<N, false, true>(W, Cm, acc, ty, tx);
   __syncthreads();
-  store_tile<N>(W, acc, ty, tx);
+  store_tile<N, true>(W, acc, ty, tx);
   __syncthreads();
   if (scan) {
     scan_columns<N>(W, alpha, beta, mu, sums);
   } else {
     // Q[l][k] = sum_y C[l][y] P[y][k];  S = Q / (alpha + beta (mu_l + mu_k))
-    smem_gemm<N, NP, 1, NP, 1>(Cm, W, acc, ty, tx);
+    smem_gemm<N, false, false>(Cm, W, acc, ty, tx);
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
       for (int j = 0; j < TM; ++j)
-        acc[i][j] *= tc::recip_nr(fmaf(beta, mu[ty + 16 * i] + mu[tx + 16 * j], alpha));
+        acc[i][j] *= tc::recip_nr(fmaf(beta, mu[ty + 16 * i] + mu[simt_col<N>(tx, j)], alpha));
     __syncthreads();
-    store_tile<N>(W, acc, ty, tx);
+    store_tile<N, false>(W, acc, ty, tx);
     __syncthreads();
     // W1[y][k] = sum_l C[l][y] S[l][k]
-    smem_gemm<N, 1, NP, NP, 1>(Cm, W, acc, ty, tx);
+    smem_gemm<N, true, false>(Cm, W, acc, ty, tx);
     __syncthreads();
-    store_tile<N>(W, acc, ty, tx);
+    store_tile<N, false>(W, acc, ty, tx);
     __syncthreads();
   }
   // W[y][x] = sum_k W1[y][k] C[k][x]
-  smem_gemm<N, NP, 1, NP, 1>(W, Cm, acc, ty, tx);
+  smem_gemm<N, false, false>(W, Cm, acc, ty, tx);
   __syncthreads();
-  store_tile<N>(W, acc, ty, tx);
+  store_tile<N, false>(W, acc, ty, tx);
   __syncthreads();
 }
 

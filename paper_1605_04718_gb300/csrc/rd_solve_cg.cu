@@ -12,7 +12,7 @@ namespace rd {
 
 // ---------------------------------------------------------------------------
 // 2-D, FP32, conjugate gradients on CUDA cores: one CTA of 256 threads per
-// proposal with every vector resident in shared memory (rows padded to N + 1).
+// proposal with every vector resident in shared memory (rows of simt_stride(N)).
 //
 //  * RD_KERNEL_CG, IMEX step: each implicit system [alpha I - beta Lap_h] w =
 //    r_w is solved by plain CG (the paper's own linear solver, Sec. 3.1.1)
@@ -34,7 +34,7 @@ namespace rd {
 // w^n - ref + tau gamma c + ref (1 - D).  Dot products are
 // compensated pair sums (46 bits), the iteration's scalars FP64 in one thread: as
 // FP64 sums they took most of a step, 152 proposals of 64^2, 30 semi-implicit
-// steps 3.02 ms against 1.43 with them and the preconditioner's scan.  A solve
+// steps 3.02 ms against 1.33 with them and the preconditioner's scan.  A solve
 // that reaches its iteration cap marks the proposal RD_P_NOT_CONVERGED.
 // ---------------------------------------------------------------------------
 constexpr int kCgMaxIter = 300;     // IMEX: plain CG
@@ -45,7 +45,7 @@ constexpr double kCgTol = 1e-6;     // relative residual
 // point; dg(o) gives the diagonal at padded offset o.
 template <int N, class Dg>
 __device__ __forceinline__ void apply_op(const float* P, float* Q, float beta, Dg dg) {
-  constexpr int NP = N + 1;
+  constexpr int NP = simt_stride(N);
   for (int i = threadIdx.x; i < N * N; i += kSimtThreads) {
     const int y = i / N, x = i - y * N, o = y * NP + x;
     const float c = P[o];
@@ -60,7 +60,7 @@ __device__ __forceinline__ void apply_op(const float* P, float* Q, float beta, D
 template <int N, class T, class F>
 __device__ __forceinline__ double reduce_points(RedScratch* red, T&& term, F&& f) {
   Pair part;
-  for (int i = threadIdx.x; i < N * N; i += kSimtThreads) term((i / N) * (N + 1) + i % N, part);
+  for (int i = threadIdx.x; i < N * N; i += kSimtThreads) term((i / N) * simt_stride(N) + i % N, part);
   return cta_reduce(part, red, f);
 }
 
@@ -70,7 +70,7 @@ __device__ __forceinline__ double reduce_points(RedScratch* red, T&& term, F&& f
 template <int N, class Dg>
 __device__ bool cg_solve(float* X, float* R, float* P, float* Q, float beta, Dg dg, double bb,
                          RedScratch* red) {
-  constexpr int NP = N + 1;
+  constexpr int NP = simt_stride(N);
   const int tid = threadIdx.x;
   const double stop = kCgTol * kCgTol * bb;
   double rr = 0.0;
@@ -122,7 +122,7 @@ template <int N, class Dg>
 __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, const float* Cm,
                           float beta, float dm, Dg dg, const float* mu, float2* sums,
                           RedScratch* red) {
-  constexpr int NP = N + 1;
+  constexpr int NP = simt_stride(N);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   double stop = 0.0, rz = 0.0;  // thread 0's
   reduce_points<N>(
@@ -199,7 +199,7 @@ template <int N, bool PICARD>
 __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const double th[kNPhys],
                                 float* sm, RedScratch* red, double* red64, float2* sums, double* phi_out,
                                 uint32_t* st_out, float* fields_out) {
-  constexpr int NP = N + 1, NPTS = N * N, VS = N * NP;
+  constexpr int NP = simt_stride(N), NPTS = N * N, VS = N * NP;
   float* U = sm;
   float* V = sm + VS;
   float* R = sm + 2 * VS;
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kSimtThreads, 1)
 #undef RD_CG_CASE
 
 size_t cg_smem_bytes(int n, bool picard) {
-  return (size_t)(picard ? 8 : 6) * n * (n + 1) * sizeof(float);
+  return (size_t)(picard ? 8 : 6) * n * simt_stride(n) * sizeof(float);
 }
 
 template <typename F>

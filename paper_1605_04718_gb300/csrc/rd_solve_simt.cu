@@ -39,9 +39,8 @@ namespace rd {
 // (implicit_solve_simt):
 //   P = W C^T, S[.][k] = [(alpha + beta mu_k) I - beta Lap_1D]^-1 P[.][k], W = S C,
 //   mu_k = 4 sin^2(pi k / (2N)), beta = tau D / (rho^2 h^2).
-// Each product is an N x N x N GEMM from shared memory with 16 x 16 threads,
-// thread (ty, tx) owning rows ty + 16 i and columns tx + 16 j.  Rows are
-// padded to N + 1 floats so that every operand load is conflict-free.
+// Each product is an N x N x N GEMM from shared memory with 16 x 16 threads
+// (smem_gemm), rows padded to simt_stride(N) floats.
 // ---------------------------------------------------------------------------
 // STEADY: the steady-state mode (see solve1d_item, rd_solve_1d.cu),
 // with the previous step (then w(T)) in two more shared-memory arrays.
@@ -50,7 +49,7 @@ __device__ void solve2d_simt_item(const DevProblem& pb, const DevSize& S,
                                   const double th[kNPhys], float* sm, double* red, float2* sums,
                                   double* phi_out, uint32_t* st_out,
                                   float* fields_out, int* steps_out) {
-  constexpr int NP = N + 1, NPTS = N * N;
+  constexpr int NP = simt_stride(N), NPTS = N * N;
   float* U = sm;  // u - ref_u
   float* V = sm + N * NP;  // v - ref_v
   float* Cm = sm + 2 * N * NP;
@@ -226,7 +225,7 @@ __global__ void __launch_bounds__(kSimtThreads, MINB)
 #undef RD_SIMT_CASE
 
 size_t simt2d_smem_bytes(int n, bool steady) {
-  return (size_t)(steady ? 5 : 3) * n * (n + 1) * sizeof(float);
+  return (size_t)(steady ? 5 : 3) * n * simt_stride(n) * sizeof(float);
 }
 
 // ---------------------------------------------------------------------------
