@@ -16,10 +16,10 @@
 // over rows: k_mlp_wgrad forms them per layer, half of the outputs and a share
 // of the row tiles, k_mlp_reduce adds the shares in a fixed order.
 // Measured (GB300): Phi~ of 4096 rows 375 us with a kernel per layer, 36 us in
-// one kernel with rows on the lanes (128-row tiles only), 25 us as it is; loss
-// and gradients of 1024 rows 1017, 118 and 78 us.  What is left is latency: the
+// one kernel with rows on the lanes (128-row tiles only), 20 us as it is; loss
+// and gradients of 1024 rows 1017, 118 and 63 us.  What is left is latency: the
 // weights' way from L2 (264 KB per tile), the layers' chain of MMAs, barrier
-// and epilogue (16 instructions per value), FP64 logarithms (5 us) and launches.
+// and epilogue (16 instructions per value) and launches.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -107,8 +107,8 @@ __device__ __forceinline__ void load_tile(uint8_t* tile, const __nv_bfloat16* g,
 }
 
 struct MlpArgs {
-  int B;
-  const __nv_bfloat16* X;   // [B][16]
+  int B, P;
+  const double* theta;      // [B][P]
   const __nv_bfloat16* Wb;  // BF16 weights in the parameter layout
   const float* params;
   Norm nm;
@@ -116,7 +116,8 @@ struct MlpArgs {
   const float* target;      // else: [B]
   float* out;               // else: [B]
   double* sq_err;           // else: summed
-  // MLP_GRAD, all with the units along the rows
+  // MLP_GRAD: the features [B][16]; the rest with the units along the rows
+  __nv_bfloat16* X;
   __nv_bfloat16 *H1, *H2, *dZ1, *dZ2, *dZ3;  // [W][B]
   float* Z1;                                 // [W][B]
   float* part4;             // [tile][W + 1]: shares of dW4, db4
@@ -205,7 +206,6 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   const int unit = 128 * half + 32 * (warp & 3) + lane, r0 = (NR / 2) * (warp >> 3);
   // layer 1's operands; its weights sit where W2's last 64 columns go later
   uint8_t* const tw1 = tw + kMlpTileW - 32768;
-  load_tile<kIn>(ta, a.X + (size_t)row0 * kIn, kIn, NR, valid);
   load_tile<kIn>(tw1, a.Wb + L.oW1, kIn, kW, kW);
   cp_async_commit();
   auto load_w_cols = [&](const __nv_bfloat16* w, int b0, int b1) {  // 64-column blocks
@@ -218,6 +218,22 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
     cp_async_commit();
   };
   load_w_cols(a.Wb + L.oW2, 0, 3);
+  // features x_j = (log theta_j - mu_j) / s_j as BF16, zero-padded to 16, while
+  // the weights are on their way; a thread each, since FP64 logarithms are what
+  // they cost (a kernel of its own took 5 us for 4096 rows)
+  for (int i = tid; i < NR * a.P; i += kMlpThreads) {
+    const int r = i / a.P, j = i - r * a.P;
+    float v = 0.f;
+    if (r < valid) {
+      const double t = a.theta[(size_t)(row0 + r) * a.P + j];
+      v = (float)((log(t > 0.0 ? t : 1e-300) - a.nm.in_mu[j]) / a.nm.in_sd[j]);
+    }
+    for (int k = j; k < kIn; k += a.P) {
+      const __nv_bfloat16 x = __float2bfloat16_rn(k == j ? v : 0.f);
+      *reinterpret_cast<__nv_bfloat16*>(ta + sw128_offset(NR, r, k)) = x;
+      if (MODE == MLP_GRAD) a.X[(size_t)(row0 + r) * kIn + k] = x;
+    }
+  }
   for (int i = tid; i < kW; i += kMlpThreads) ctl->w4[i] = a.params[L.oW4 + i];
   const float bias1 = a.params[L.ob1 + unit], bias2 = a.params[L.ob2 + unit],
               bias3 = a.params[L.ob3 + unit];
@@ -561,22 +577,6 @@ __global__ void k_mlp_reduce(int splits, int tiles, const float* part, const flo
 // ---------------------------------------------------------------------------
 // Small CUDA-core kernels
 // ---------------------------------------------------------------------------
-// Features x_i = (log theta_i - mu_i) / s_i as BF16, zero-padded to 16, one
-// thread per inferred parameter: the FP64 logarithms are what this costs, so no
-// lane of a warp is spent on padding.  Also clears the squared error's sum.
-__global__ void k_features(int B, int P, const double* theta, Norm nm, __nv_bfloat16* X,
-                           double* sq_err) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && sq_err) *sq_err = 0.0;
-  if (i >= B * P) return;
-  const int b = i / P, j = i - b * P;
-  const double t = theta[i];
-  const float v = (float)((log(t > 0.0 ? t : 1e-300) - nm.in_mu[j]) / nm.in_sd[j]);
-  __nv_bfloat16* x = X + (size_t)b * kIn;
-  x[j] = __float2bfloat16_rn(v);
-  for (int k = P + j; k < kIn; k += P) x[k] = __float2bfloat16_rn(0.f);
-}
-
 // Adam with bias correction and decoupled weight decay on the weights (mask
 // = 1) but not the biases; refreshes the BF16 copies of W1..W3.
 struct AdamArgs {
@@ -625,12 +625,11 @@ struct rd_surrogate {
   int adam_t = 0;
   // activations for up to `cap` rows
   int cap = 0;
-  __nv_bfloat16* X = nullptr;
-  float *out = nullptr, *target = nullptr;
+  float* out = nullptr;
   double* sqerr = nullptr;
   // the backward pass's, for up to `grad_cap` rows
   int grad_cap = 0;
-  __nv_bfloat16 *H1 = nullptr, *H2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
+  __nv_bfloat16 *X = nullptr, *H1 = nullptr, *H2 = nullptr, *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
   float *Z1 = nullptr, *part = nullptr, *part4 = nullptr;
 };
 
@@ -638,18 +637,17 @@ namespace rd {
 namespace mlp {
 
 static void free_acts(rd_surrogate* s) {
-  void* ptrs[] = {s->X, s->out, s->target, s->sqerr};
-  for (void* p : ptrs) cudaFree(p);
-  s->X = nullptr;
-  s->out = s->target = nullptr;
+  cudaFree(s->out);
+  cudaFree(s->sqerr);
+  s->out = nullptr;
   s->sqerr = nullptr;
   s->cap = 0;
 }
 
 static void free_grad(rd_surrogate* s) {
-  void* ptrs[] = {s->H1, s->H2, s->dZ1, s->dZ2, s->dZ3, s->Z1, s->part, s->part4};
+  void* ptrs[] = {s->X, s->H1, s->H2, s->dZ1, s->dZ2, s->dZ3, s->Z1, s->part, s->part4};
   for (void* p : ptrs) cudaFree(p);
-  s->H1 = s->H2 = s->dZ1 = s->dZ2 = s->dZ3 = nullptr;
+  s->X = s->H1 = s->H2 = s->dZ1 = s->dZ2 = s->dZ3 = nullptr;
   s->Z1 = s->part = s->part4 = nullptr;
   s->grad_cap = 0;
 }
@@ -664,9 +662,7 @@ cudaError_t ensure_rows(rd_surrogate* s, int rows) {
   free_acts(s);
   const size_t cap = (size_t)((rows + 127) / 128) * 128;
   cudaError_t e;
-  RD_ALLOC(s->X, sizeof(__nv_bfloat16) * cap * kIn);
   RD_ALLOC(s->out, sizeof(float) * cap);
-  RD_ALLOC(s->target, sizeof(float) * cap);
   RD_ALLOC(s->sqerr, sizeof(double));
   s->cap = (int)cap;
   s->pb->generation++;  // captured graphs may hold the old buffers
@@ -681,6 +677,7 @@ static cudaError_t ensure_grad_rows(rd_surrogate* s, int rows) {
   free_grad(s);
   const size_t cap = (size_t)rows, W = (size_t)s->W;
   const Layout L(s->W);
+  RD_ALLOC(s->X, sizeof(__nv_bfloat16) * cap * kIn);
   RD_ALLOC(s->H1, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->H2, sizeof(__nv_bfloat16) * cap * W);
   RD_ALLOC(s->dZ1, sizeof(__nv_bfloat16) * cap * W);
@@ -726,22 +723,24 @@ static cudaError_t launch_mlp(const MlpArgs& a, int n_sm, cudaStream_t st) {
 }
 
 // One pass over B rows of theta (device [B][P]): MLP_PREDICT writes Phi~ to
-// phit; MLP_LOSS writes s->out and the summed squared error against s->target;
+// phit; MLP_LOSS writes s->out and the summed squared error against target;
 // MLP_GRAD also leaves what the weight gradients need.
 static cudaError_t pass(rd_surrogate* s, int mode, int B, const double* theta, double* phit,
-                        cudaStream_t st) {
-  k_features<<<(B * s->P + 127) / 128, 128, 0, st>>>(B, s->P, theta, s->norm, s->X,
-                                                     mode == MLP_PREDICT ? nullptr : s->sqerr);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+                        const float* target, cudaStream_t st) {
+  if (mode != MLP_PREDICT) {
+    const cudaError_t e = cudaMemsetAsync(s->sqerr, 0, sizeof(double), st);
+    if (e != cudaSuccess) return e;
+  }
   MlpArgs a{};
   a.B = B;
+  a.P = s->P;
+  a.theta = theta;
   a.X = s->X;
   a.Wb = s->Wb;
   a.params = s->params;
   a.nm = s->norm;
   a.phit = phit;
-  a.target = s->target;
+  a.target = target;
   a.out = s->out;
   a.sq_err = s->sqerr;
   a.H1 = s->H1;
@@ -758,11 +757,12 @@ static cudaError_t pass(rd_surrogate* s, int mode, int B, const double* theta, d
   return launch_mlp<MLP_GRAD>(a, n_sm, st);
 }
 
-// Loss and gradient of the mean-squared error against s->target for B rows (a
+// Loss and gradient of the mean-squared error against target for B rows (a
 // multiple of 128): the summed squared error into s->sqerr, all parameter
-// gradients into s->grads.
-static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, cudaStream_t st) {
-  cudaError_t e = pass(s, MLP_GRAD, B, theta, nullptr, st);
+// gradients into grads.
+static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, const float* target,
+                             float* grads, cudaStream_t st) {
+  cudaError_t e = pass(s, MLP_GRAD, B, theta, nullptr, target, st);
   if (e != cudaSuccess) return e;
   const Layout L(s->W);
   WgradArgs g{};
@@ -783,7 +783,7 @@ static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, cudaSt
   k_mlp_wgrad<<<dim3(s->W / 128, 3, g.splits), kMlpThreads, kWgSmem, st>>>(g);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_mlp_reduce<<<(unsigned)((L.total + 255) / 256), 256, 0, st>>>(g.splits, B / tile_rows(MLP_GRAD, B, s->pb->n_sm), s->part,
-                                                                   s->part4, s->grads);
+                                                                   s->part4, grads);
   return cudaGetLastError();
 }
 
@@ -812,7 +812,7 @@ cudaError_t adam_step(rd_surrogate* s, double lr, double b1, double b2, double e
 }
 
 cudaError_t predict(rd_surrogate* s, int B, const double* theta, double* phit, cudaStream_t st) {
-  return pass(s, MLP_PREDICT, B, theta, phit, st);
+  return pass(s, MLP_PREDICT, B, theta, phit, nullptr, st);
 }
 
 }  // namespace mlp
@@ -966,13 +966,9 @@ rd_status rd_surrogate_loss_grad(rd_surrogate* s, int B, const double* theta,
   RD_SCHECK(B >= 128 && B % 128 == 0, RD_EINVAL, "B must be a positive multiple of 128");
   cudaStream_t st = s->pb->stream;
   RD_SCUDA(mlp::ensure_grad_rows(s, B));
-  RD_SCUDA(cudaMemcpyAsync(s->target, target, sizeof(float) * B, cudaMemcpyDeviceToDevice, st));
-  RD_SCUDA(mlp::loss_grad(s, B, theta, st));
+  RD_SCUDA(mlp::loss_grad(s, B, theta, target, grads ? grads : s->grads, st));
   double se = 0.0;
   RD_SCUDA(cudaMemcpyAsync(&se, s->sqerr, sizeof(double), cudaMemcpyDeviceToHost, st));
-  const mlp::Layout L(s->W);
-  if (grads)
-    RD_SCUDA(cudaMemcpyAsync(grads, s->grads, sizeof(float) * L.total, cudaMemcpyDeviceToDevice, st));
   RD_SCUDA(cudaStreamSynchronize(st));
   *loss = se / B;
   return RD_OK;
@@ -1082,9 +1078,8 @@ rd_status rd_surrogate_train(rd_surrogate* s, int n, const double* theta, const 
     double se = 0.0;
     for (int k = 0; k < nb; ++k) {
       const int b = order[k];
-      RD_SCUDA(cudaMemcpyAsync(s->target, d_z + (size_t)b * td->batch, sizeof(float) * td->batch,
-                               cudaMemcpyDeviceToDevice, st));
-      RD_SCUDA(mlp::loss_grad(s, td->batch, d_th + (size_t)b * td->batch * P, st));
+      RD_SCUDA(mlp::loss_grad(s, td->batch, d_th + (size_t)b * td->batch * P,
+                              d_z + (size_t)b * td->batch, s->grads, st));
       RD_SCUDA(mlp::adam_step(s, td->lr, td->beta1, td->beta2, 1e-8, td->weight_decay, st));
       if (ep == td->epochs - 1) {
         double v = 0.0;
@@ -1099,9 +1094,7 @@ rd_status rd_surrogate_train(rd_surrogate* s, int n, const double* theta, const 
   double hold_se = 0.0, hold_abs = 0.0;
   std::vector<float> outv(td->batch);
   for (int off = n_train; off + td->batch <= n_train + n_hold; off += td->batch) {
-    RD_SCUDA(cudaMemcpyAsync(s->target, d_z + off, sizeof(float) * td->batch,
-                             cudaMemcpyDeviceToDevice, st));
-    RD_SCUDA(mlp::pass(s, mlp::MLP_LOSS, td->batch, d_th + (size_t)off * P, nullptr, st));
+    RD_SCUDA(mlp::pass(s, mlp::MLP_LOSS, td->batch, d_th + (size_t)off * P, nullptr, d_z + off, st));
     double v = 0.0;
     RD_SCUDA(cudaMemcpyAsync(&v, s->sqerr, sizeof(double), cudaMemcpyDeviceToHost, st));
     RD_SCUDA(cudaMemcpyAsync(outv.data(), s->out, sizeof(float) * td->batch, cudaMemcpyDeviceToHost, st));
