@@ -265,8 +265,9 @@ rd_status rd_evaluate_batch_steady(rd_problem* p, int B, const double* theta,
 rd_status rd_set_turing_prior(rd_problem* p, int enable);
 
 /* Kernel that solves the proposals of grid size `size_idx` (RD_KERNEL_*).
- * Sizes that share a kernel run in one persistent launch; a batch whose sizes
- * use different kernels runs one launch per kernel, in stream order.  EINVAL
+ * The tensor-core kernels run one persistent launch per grid size N, a size's
+ * blocks starting as the one before leaves room; sizes that share another kernel
+ * run in one launch, and different kernels in stream order.  EINVAL
  * for a 1-D problem (always the Thomas solve), an unknown kernel, or
  * TC_RESIDENT at N != 128.  Takes effect at the next launch (captured chain
  * steps are re-captured). */
@@ -289,9 +290,8 @@ rd_status rd_get_size_schedule(const rd_problem* p, int size_idx, int* ctas_per_
  * stream), probe_steps IMEX steps per solve (0 = the problem's n_steps), and
  * sets the kernel and schedule with the lowest median time
  * (rd_set_size_kernel, rd_set_size_schedule): every kernel is timed at 1, 2,
- * 4, ... persistent CTAs per SM up to what fits on an SM.  Sizes
- * of a problem run one persistent launch per kernel kind, so the choice per
- * size stays within one batched evaluation.  times_out (host, may be NULL):
+ * 4, ... persistent CTAs per SM up to what fits on an SM.  The
+ * choice per size stays within one batched evaluation.  times_out (host, may be NULL):
  * [n_sizes][4] seconds per proposal for RD_KERNEL_SIMT, TC_STACKED,
  * TC_RESIDENT and CG at each one's best schedule, NaN where a kernel does
  * not apply.  Allocates scratch for the

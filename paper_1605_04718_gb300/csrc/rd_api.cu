@@ -316,10 +316,8 @@ rd_status rd_problem_destroy(rd_problem* p) {
   cudaFree(p->ws.queue_items);
   cudaFree(p->ws.queue_counters);
   cudaFree(p->ws.err);
-  cudaFree(p->h2d_theta);
-  cudaFree(p->h2d_size);
-  cudaFree(p->d2h_phi);
-  cudaFree(p->d2h_status);
+  cudaFree(p->stage_dev);
+  cudaFreeHost(p->stage_host);
   delete p;
   return RD_OK;
 }
@@ -550,6 +548,13 @@ rd_status rd_get_size_kernel(const rd_problem* p, int size_idx, int* kernel) {
   return RD_OK;
 }
 
+// A bounded wait gave up since the last check: clears the flag and says so.
+static rd_status report_timeout(rd_problem* p) {
+  RD_CUDA(cudaMemset(p->ws.err, 0, sizeof(int)));
+  set_error("a solve kernel's bounded wait gave up; its results are invalid");
+  return RD_ETIMEOUT;
+}
+
 rd_status rd_evaluate_batch_host(rd_problem* p, int B, const double* theta,
                                  const int* size_idx, double* loglik,
                                  uint32_t* status) {
@@ -557,36 +562,45 @@ rd_status rd_evaluate_batch_host(rd_problem* p, int B, const double* theta,
   RD_CHECK(B >= 0, RD_EINVAL, "B must be >= 0");
   if (B == 0) return RD_OK;
   RD_CHECK(theta && loglik && status, RD_EINVAL, "NULL argument");
+  // device: theta | phi | status | size; pinned host: phi | status | error flag, so
+  // that the results come back in two copies that do not block one by one
+  const size_t n_th = (size_t)B * p->desc.n_params;
   if (B > p->staging_cap) {
     RD_CUDA(cudaStreamSynchronize(p->stream));
-    cudaFree(p->h2d_theta);
-    cudaFree(p->h2d_size);
-    cudaFree(p->d2h_phi);
-    cudaFree(p->d2h_status);
-    p->h2d_theta = nullptr;
-    p->h2d_size = nullptr;
-    p->d2h_phi = nullptr;
-    p->d2h_status = nullptr;
+    cudaFree(p->stage_dev);
+    cudaFreeHost(p->stage_host);
+    p->stage_dev = nullptr;
+    p->stage_host = nullptr;
     p->staging_cap = 0;
-    RD_CUDA(cudaMalloc(&p->h2d_theta, sizeof(double) * (size_t)B * p->desc.n_params));
-    RD_CUDA(cudaMalloc(&p->h2d_size, sizeof(int) * (size_t)B));
-    RD_CUDA(cudaMalloc(&p->d2h_phi, sizeof(double) * (size_t)B));
-    RD_CUDA(cudaMalloc(&p->d2h_status, sizeof(uint32_t) * (size_t)B));
+    RD_CUDA(cudaMalloc(&p->stage_dev, sizeof(double) * (n_th + (size_t)B) +
+                                          (sizeof(uint32_t) + sizeof(int)) * (size_t)B));
+    RD_CUDA(cudaMallocHost(&p->stage_host, (sizeof(double) + sizeof(uint32_t)) * (size_t)B +
+                                               sizeof(int)));
     p->staging_cap = B;
   }
-  RD_CUDA(cudaMemcpyAsync(p->h2d_theta, theta, sizeof(double) * (size_t)B * p->desc.n_params,
-                          cudaMemcpyHostToDevice, p->stream));
+  double* const d_theta = (double*)p->stage_dev;
+  double* const d_phi = d_theta + n_th;
+  uint32_t* const d_status = (uint32_t*)(d_phi + B);
+  int* const d_size = (int*)(d_status + B);
+  char* const host = (char*)p->stage_host;
+  const size_t n_res = (sizeof(double) + sizeof(uint32_t)) * (size_t)B;
+  RD_CUDA(cudaMemcpyAsync(d_theta, theta, sizeof(double) * n_th, cudaMemcpyHostToDevice,
+                          p->stream));
   if (size_idx)
-    RD_CUDA(cudaMemcpyAsync(p->h2d_size, size_idx, sizeof(int) * (size_t)B,
-                            cudaMemcpyHostToDevice, p->stream));
-  rd_status r = rd_evaluate_batch(p, B, p->h2d_theta, size_idx ? p->h2d_size : nullptr,
-                                  p->d2h_phi, p->d2h_status, nullptr);
+    RD_CUDA(cudaMemcpyAsync(d_size, size_idx, sizeof(int) * (size_t)B, cudaMemcpyHostToDevice,
+                            p->stream));
+  rd_status r = rd_evaluate_batch(p, B, d_theta, size_idx ? d_size : nullptr, d_phi, d_status,
+                                  nullptr);
   if (r != RD_OK) return r;
-  RD_CUDA(cudaMemcpyAsync(loglik, p->d2h_phi, sizeof(double) * (size_t)B,
-                          cudaMemcpyDeviceToHost, p->stream));
-  RD_CUDA(cudaMemcpyAsync(status, p->d2h_status, sizeof(uint32_t) * (size_t)B,
-                          cudaMemcpyDeviceToHost, p->stream));
-  return rd_sync(p);  // waits, then reports a bounded wait that gave up
+  RD_CUDA(cudaMemcpyAsync(host, d_phi, n_res, cudaMemcpyDeviceToHost, p->stream));
+  RD_CUDA(cudaMemcpyAsync(host + n_res, p->ws.err, sizeof(int), cudaMemcpyDeviceToHost,
+                          p->stream));
+  RD_CUDA(cudaStreamSynchronize(p->stream));
+  memcpy(loglik, host, sizeof(double) * (size_t)B);
+  memcpy(status, host + sizeof(double) * (size_t)B, sizeof(uint32_t) * (size_t)B);
+  int err = 0;
+  memcpy(&err, host + n_res, sizeof(int));
+  return err ? report_timeout(p) : RD_OK;
 }
 
 rd_status rd_sync(rd_problem* p) {
@@ -594,12 +608,7 @@ rd_status rd_sync(rd_problem* p) {
   RD_CUDA(cudaStreamSynchronize(p->stream));
   int err = 0;
   RD_CUDA(cudaMemcpy(&err, p->ws.err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) {
-    RD_CUDA(cudaMemset(p->ws.err, 0, sizeof(int)));
-    set_error("a solve kernel's bounded wait gave up; its results are invalid");
-    return RD_ETIMEOUT;
-  }
-  return RD_OK;
+  return err ? report_timeout(p) : RD_OK;
 }
 
 // ------------------------------------------------------------------ autotuning

@@ -51,10 +51,8 @@ struct rd_problem {
   // persistent CTAs per SM of each size's launch (0 = the kernel's maximum)
   int ctas_per_sm[RD_MAX_SIZES] = {0, 0, 0, 0};
   // staging for rd_evaluate_batch_host
-  double* h2d_theta = nullptr;
-  int* h2d_size = nullptr;
-  double* d2h_phi = nullptr;
-  uint32_t* d2h_status = nullptr;
+  void* stage_dev = nullptr;   // parameters in, results out
+  void* stage_host = nullptr;  // pinned: results and the error flag
   int staging_cap = 0;
 };
 
