@@ -51,7 +51,7 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
         "sha256": "8ceb430559a377c3b06d2fc0df01d9b32aaaf95435c5b725a4d53ae8853bd916",
-        "bytes": 1238784 + 2430976,
+        "bytes": 1352960 + 2184448,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)
@@ -648,8 +648,7 @@ def run_gpu(args):
                     "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x max SM clock"}
         else:
             tpk = _find(pk, "bf16_tflops_sustained") or FALLBACK_PEAKS["bf16_tflops_sustained"]
-            kname = ("k_solve2d_tc128<2>" if kind == rd.RD_KERNEL_TC_RESIDENT
-                     else "k_solve2d_tc<128>")
+            kname = "k_solve2d_tc128<2>"  # both tensor-core kinds at 128^2
             roof = {"bound": "tensor", "achieved": achieved, "peak": tpk, "unit": "TFLOP/s",
                     "frac": achieved / tpk, "traffic": traffic_of(kname), "kernel": kname,
                     "peak_source": f"{pk_src} bf16 sustained (= fp16 rate): the kernel runs "
