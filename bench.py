@@ -50,8 +50,8 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "8ceb430559a377c3b06d2fc0df01d9b32aaaf95435c5b725a4d53ae8853bd916",
-        "bytes": 1352960 + 2184448,
+        "sha256": "4fc00d1f8fa694370bfd60a0e0af400faeca23a550e399df9725ee33f3ef293f",
+        "bytes": 957184 + 1379072,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)

@@ -70,7 +70,9 @@
 // reaction value outside the FP16 range (a diverging solve) must not reach the
 // MMA as infinity (nor reach the scan as one: |r| >= 256): it is stored as zero, and
 // every later observation or output of its proposal reads NaN, which is what an
-// infinite operand leads to.
+// infinite operand leads to.  With that, |D| <= 256 sqrt(N), and the scan's output
+// (at most |D| / alpha and the constant's term) stays inside the range too wherever
+// `irregular` lets a proposal share a CTA.
 //
 // Every wait is bounded; a timed-out wait makes the CTA leave, drain its MMAs,
 // free its TMEM and raise the error flag.
@@ -336,14 +338,20 @@ __device__ __noinline__ void observe(const DevProblem& pb, int size, int sl, int
 }
 
 // A whole row of N nodes by Gaussian elimination (any lam and beta), from the
-// accumulator columns at t to the operand row l, columns col0...
+// accumulator columns at t to the operand row l, columns col0...  For alpha, beta > 0
+// the pivots are beta + e_i with e_0 = lam, e_i = lam + e_{i-1} / (1 + e_{i-1} / beta),
+// the last one e_{N-1}: sums of positive terms, so that lam is not lost beside a
+// large beta (lam + 2 beta + beta c'_{i-1} loses 1.5e-5 of the row at beta / alpha = 1e4
+// and the whole row from 1e8 on; this form at most 3e-6 up to 1e25, in float32).
 template <int N>
 __device__ __noinline__ void slow_row(uint32_t t, int g, int rows, int l, int col0, bool store,
                                       float alpha, float beta, float mu, float out_scale,
                                       float off) {
-  float c[N], d[N];
+  float c[N], d[N];  // x_i = d_i + c_i x_{i+1}
   const float lam = fmaf(beta, mu, alpha);
-  float cp = 0.f, dp = 0.f;
+  const bool positive = alpha > 0.f && beta > 0.f;
+  float cp = 0.f, dp = 0.f, e = 0.f, s = 0.f;
+#pragma unroll 1
   for (int x = 0; x < N; x += 8) {
     float v[8];
     __syncwarp();
@@ -351,18 +359,27 @@ __device__ __noinline__ void slow_row(uint32_t t, int g, int rows, int l, int co
     tmem_wait_ld();
     for (int j = 0; j < 8; ++j) {
       const int i = x + j;
-      const float den = lam + ((i == 0 || i == N - 1) ? beta : 2.f * beta) + beta * cp;
-      cp = -beta / den;
-      dp = (v[j] + beta * dp) / den;
+      if (positive) {
+        e = fmaf(e, cp, lam);
+        s = fmaf(s, cp, v[j]);
+        cp = 1.f / (1.f + e / beta);
+        dp = s / (i == N - 1 ? e : e + beta);
+      } else {
+        const float den = lam + ((i == 0 || i == N - 1) ? beta : 2.f * beta) - beta * cp;
+        cp = beta / den;
+        dp = (v[j] + beta * dp) / den;
+      }
       c[i] = cp;
       d[i] = dp;
     }
   }
   float x1 = 0.f;
+#pragma unroll 1
   for (int i = N - 1; i >= 0; --i) {
-    x1 = d[i] - (i < N - 1 ? c[i] * x1 : 0.f);
+    x1 = d[i] + (i < N - 1 ? c[i] * x1 : 0.f);
     d[i] = x1;
   }
+#pragma unroll 1
   for (int x = 0; x < N; x += 8) store8(tile(g), rows, l, col0 + x, d + x, out_scale, off, store);
 }
 
@@ -776,15 +793,30 @@ __device__ __noinline__ bool grower(const DevProblem& pb, int lane, Parity par) 
   return true;
 }
 
-// Proposals the scan does not cover (negative diffusion, a growth factor out
-// of range, non-finite parameters): solved alone, by elimination.
-__device__ __forceinline__ bool irregular(const DevProblem& pb, const double th[kNPhys]) {
+// Proposals the scan does not cover (negative diffusion, alpha <= 0, a beta / alpha
+// above kScanMaxRatio at any step, non-finite parameters): solved alone, by
+// elimination.  So are, at N <= 64, those whose scanned values could leave the FP16
+// range (|x| <= 256 sqrt(N) / alpha, see the top of the file): as infinities they
+// would reach the other proposals of the block-diagonal products.
+template <int N>
+__device__ __forceinline__ bool irregular(const DevProblem& pb, const DevSize& S,
+                                          const double th[kNPhys]) {
   bool fin = true;
   for (int j = 0; j < kNPhys; ++j) fin = fin && isfinite(th[j]);
   if (!fin || !(th[2] >= 0.0)) return true;
-  if (!pb.growth) return false;
-  return !(1.0 + 2.0 * pb.tau * th[4] > 0.0) ||
-         !(fabs(2.0 * th[4] * pb.tau * pb.n_steps) < 40.0);
+  // FP32: the line is far from where either side fails, and an overflow is beyond it
+  float alpha = 1.f, top = (float)pb.tau * (float)(N * N) * fmaxf(1.f, (float)th[2]);
+  if (pb.growth) {
+    const double r2 = 2.0 * pb.tau * th[4], al = 1.0 + r2;
+    if (!(al > 0.0)) return true;
+    alpha = (float)al;
+    if (th[4] < 0.0) top *= expf(-(float)r2 * (float)pb.n_steps);
+    const float ref = fmaxf(fabsf(S.ref_u), fabsf(S.ref_v));
+    if (N <= 64 &&
+        !(16.f * sqrtf((float)N) * (256.f + fabsf((float)r2) * ref) <= 65000.f * alpha))
+      return true;
+  }
+  return !(top <= kScanMaxRatio * alpha);
 }
 
 // Pops proposals of one size of the queue: as many as a CTA holds, fewer when
@@ -810,7 +842,7 @@ __device__ __forceinline__ void pop_chunk(const DevProblem& pb, const WorkQueue&
       const int item = q.items[(size_t)s * q.capacity + i + j];
       double th[kNPhys];
       full_theta(pb, theta + (size_t)item * pb.n_params, th);
-      if (irregular(pb, th))
+      if (irregular<N>(pb, pb.sz[s], th))
         ctl->chunk[--z] = item;
       else
         ctl->chunk[a++] = item;
