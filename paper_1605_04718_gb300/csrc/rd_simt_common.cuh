@@ -159,16 +159,17 @@ __device__ __forceinline__ void scan_columns(float* W, float alpha, float beta, 
 }
 
 // In place: W <- [alpha I - beta Lap_h]^-1 W.  Two transforms along x and a scan
-// along y; outside the scan's range (alpha <= 0, beta < 0 or not finite) four
-// transforms and the division by the eigenvalues.  mu: the eigenvalues, sums:
-// 256 float2 of scratch.  A step of the CUDA-core kernel, per proposal, four
-// transforms -> two and a scan: 64^2 0.251 -> 0.145 us, 128^2 0.899 -> 0.406 us.
+// along y; outside the scan's range (alpha <= 0, beta < 0, beta / alpha above
+// kScanMaxRatio or not finite) four transforms and the division by the
+// eigenvalues.  mu: the eigenvalues, sums: 256 float2 of scratch.  A step of the
+// CUDA-core kernel, per proposal, four transforms -> two and a scan: 64^2 0.251 ->
+// 0.145 us, 128^2 0.899 -> 0.406 us.
 template <int N>
 __device__ __forceinline__ void implicit_solve_simt(float* W, const float* Cm, float alpha,
                                                     float beta, const float* mu, float2* sums,
                                                     int ty, int tx) {
   constexpr int TM = N / 16;
-  const bool scan = alpha > 0.f && beta >= 0.f && beta < 1e30f;
+  const bool scan = alpha > 0.f && beta >= 0.f && beta <= kScanMaxRatio * alpha;
   float acc[TM][TM];
   // P[y][k] = sum_x W[y][x] C[k][x]
   smem_gemm<N, false, true>(W, Cm, acc, ty, tx);

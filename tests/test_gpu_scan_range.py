@@ -89,3 +89,12 @@ def test_long_shrinking_and_growing_runs():
     theta = np.column_stack([np.tile(TRUE4, (27, 1)), np.full(27, 0.01)])
     theta[1, 4], theta[7, 4], theta[13, 4], theta[19, 4], theta[24, 4] = -30.0, -45.0, -50.0, 60.0, 200.0
     _check(ds, theta, 1e-3, growth=1)
+
+
+# as the first test; four FP32 transforms instead of the elimination
+@pytest.mark.parametrize("n", [16, 32, 64, 96, 128])
+def test_fast_diffusion_on_the_cuda_cores(n):
+    ds = H.small_dataset(n, 7, seed=n)
+    theta = _draws(n)
+    theta[1, 2], theta[4, 2], theta[6, 2], theta[7, 2] = 1e16, 1e12, 1e7, 1e30
+    _check(ds, theta, 1e-5, kernel=rd.RD_KERNEL_SIMT, fill=False)
