@@ -208,6 +208,12 @@ __device__ __forceinline__ void implicit_solve_simt(float* W, const float* Cm, f
 // FMA) and collected in c, so the sum carries about 46 bits.  The FP64 pipe takes
 // 64 cycles per warp instruction and an FP64 dot product needs three of them per
 // element (two conversions and an FMA); this needs 11 FP32 instructions.
+//
+// The exponent range is FP32's: a product above 2^128 overflows, and what is lost of
+// products near the smallest value is at most 2^-149 each, 2^-135.8 for 96^2, so 46 bits
+// need a sum of kPairMin or more.  A sum out of that range is reported, and the
+// proposal solved with Sum64 instead.
+constexpr float kPairMin = 0x1p-89f;
 struct Pair {
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x, float low = 0.f) {
@@ -222,16 +228,25 @@ struct Pair {
   }
 };
 
+// The same in FP64, for any range.
+struct Sum64 {
+  double s = 0.0;
+  __device__ __forceinline__ void add(float x) { s += (double)x; }
+  __device__ __forceinline__ void add_product(float x, float y) { s += (double)x * (double)y; }
+};
+
 // Scratch of cta_reduce.
 struct RedScratch {
   float2 part[kSimtThreads / 32];
+  double part64[kSimtThreads / 32];
   double out;
 };
 
 // f(sum over the CTA), f evaluated in thread 0 (so that its FP64 operations are
-// done once); the result in every thread.
+// done once); the result in every thread.  ok: cleared in warp 0 by a sum out of the
+// pairs' range.
 template <class F>
-__device__ __forceinline__ double cta_reduce(Pair v, RedScratch* red, F&& f) {
+__device__ __forceinline__ double cta_reduce(Pair v, RedScratch* red, bool& ok, F&& f) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
     v.add(__shfl_xor_sync(0xffffffffu, v.s, o), __shfl_xor_sync(0xffffffffu, v.c, o));
@@ -246,12 +261,29 @@ __device__ __forceinline__ double cta_reduce(Pair v, RedScratch* red, F&& f) {
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1)
       t.add(__shfl_xor_sync(0xffffffffu, t.s, o), __shfl_xor_sync(0xffffffffu, t.c, o));
+    // t.c is a small part of t.s, and finite where t.s is
+    ok = ok && fabsf(t.s) >= kPairMin && fabsf(t.s) <= 3.4028234e38f;
     if (lane == 0) red->out = f((double)t.s + (double)t.c);
   }
   __syncthreads();
   return red->out;
 }
 static_assert(kSimtThreads == 256, "cta_reduce combines 8 warps");
+
+template <class F>
+__device__ __forceinline__ double cta_reduce(Sum64 v, RedScratch* red, bool&, F&& f) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v.s += __shfl_xor_sync(0xffffffffu, v.s, o);
+  if ((threadIdx.x & 31) == 0) red->part64[threadIdx.x >> 5] = v.s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int i = 0; i < kSimtThreads / 32; ++i) t += red->part64[i];
+    red->out = f(t);
+  }
+  __syncthreads();
+  return red->out;
+}
 
 // FP64 sum over the CTA; result valid in thread 0.
 __device__ __forceinline__ double cta_sum(double v, double* red) {

@@ -34,8 +34,11 @@ namespace rd {
 // w^n - ref + tau gamma c + ref (1 - D).  Dot products are
 // compensated pair sums (46 bits), the iteration's scalars FP64 in one thread: as
 // FP64 sums they took most of a step, 152 proposals of 64^2, 30 semi-implicit
-// steps 3.02 ms against 1.33 with them and the preconditioner's scan.  A solve
-// that reaches its iteration cap marks the proposal RD_P_NOT_CONVERGED.
+// steps 3.02 ms against 1.33 with them and the preconditioner's scan.  The 46 bits
+// change no result (over 20 batches of 32^2 to 80^2 the fields were those of FP64 sums
+// to the bit); a proposal one of whose sums leaves the pairs' exponent range is solved
+// again with FP64 sums, decided once a step (a branch at every sum cost 4 to 10 %).
+// A solve that reaches its iteration cap marks the proposal RD_P_NOT_CONVERGED.
 // ---------------------------------------------------------------------------
 constexpr int kCgMaxIter = 300;     // IMEX: plain CG
 constexpr int kPcgMaxIter = 40;     // Picard: preconditioned CG
@@ -57,26 +60,26 @@ __device__ __forceinline__ void apply_op(const float* P, float* Q, float beta, D
 
 // Sum over all points of term(offset, sum) and f of it (in thread 0), to every
 // thread.
-template <int N, class T, class F>
-__device__ __forceinline__ double reduce_points(RedScratch* red, T&& term, F&& f) {
-  Pair part;
+template <int N, class Sum, class T, class F>
+__device__ __forceinline__ double reduce_points(RedScratch* red, bool& ok, T&& term, F&& f) {
+  Sum part;
   for (int i = threadIdx.x; i < N * N; i += kSimtThreads) term((i / N) * simt_stride(N) + i % N, part);
-  return cta_reduce(part, red, f);
+  return cta_reduce(part, red, ok, f);
 }
 
 // CG on [diag(dg) - beta Lap_h] X = b from the X given, R = b - A X on entry;
 // P, Q scratch; bb = |b|^2 (thread 0's).  Returns false at the iteration cap.
 // The FP64 scalars of the iteration live in thread 0.
-template <int N, class Dg>
+template <int N, class Sum, class Dg>
 __device__ bool cg_solve(float* X, float* R, float* P, float* Q, float beta, Dg dg, double bb,
-                         RedScratch* red) {
+                         RedScratch* red, bool& ok) {
   constexpr int NP = simt_stride(N);
   const int tid = threadIdx.x;
   const double stop = kCgTol * kCgTol * bb;
   double rr = 0.0;
-  bool done = reduce_points<N>(
-                  red,
-                  [&](int o, Pair& s) {
+  bool done = reduce_points<N, Sum>(
+                  red, ok,
+                  [&](int o, Sum& s) {
                     P[o] = R[o];
                     s.add_product(R[o], R[o]);
                   },
@@ -88,12 +91,12 @@ __device__ bool cg_solve(float* X, float* R, float* P, float* Q, float beta, Dg 
     if (done) return true;
     apply_op<N>(P, Q, beta, dg);
     __syncthreads();
-    const float al = (float)reduce_points<N>(
-        red, [&](int o, Pair& s) { s.add_product(P[o], Q[o]); },
+    const float al = (float)reduce_points<N, Sum>(
+        red, ok, [&](int o, Sum& s) { s.add_product(P[o], Q[o]); },
         [&](double pq) { return rr / pq; });
-    double be = reduce_points<N>(
-        red,
-        [&](int o, Pair& s) {
+    double be = reduce_points<N, Sum>(
+        red, ok,
+        [&](int o, Sum& s) {
           X[o] = fmaf(al, P[o], X[o]);
           const float r = fmaf(-al, Q[o], R[o]);
           R[o] = r;
@@ -118,16 +121,16 @@ __device__ bool cg_solve(float* X, float* R, float* P, float* Q, float beta, Dg 
 
 // Preconditioned CG on [diag(dg) - beta Lap_h] X = b, M = [dm I - beta
 // Lap_h] solved in the eigenbasis; R = b on entry.  X = M^-1 b first.
-template <int N, class Dg>
+template <int N, class Sum, class Dg>
 __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, const float* Cm,
                           float beta, float dm, Dg dg, const float* mu, float2* sums,
-                          RedScratch* red) {
+                          RedScratch* red, bool& ok) {
   constexpr int NP = simt_stride(N);
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   double stop = 0.0, rz = 0.0;  // thread 0's
-  reduce_points<N>(
-      red,
-      [&](int o, Pair& s) {
+  reduce_points<N, Sum>(
+      red, ok,
+      [&](int o, Sum& s) {
         Z[o] = R[o];
         s.add_product(R[o], R[o]);
       },
@@ -145,9 +148,9 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
   __syncthreads();
   // R <- the residual, Z its copy for the preconditioner; whether it is small
   auto residual = [&](float al, const float* V) {
-    return reduce_points<N>(
-               red,
-               [&](int o, Pair& s) {
+    return reduce_points<N, Sum>(
+               red, ok,
+               [&](int o, Sum& s) {
                  const float r = fmaf(-al, V[o], R[o]);
                  R[o] = r;
                  Z[o] = r;
@@ -157,9 +160,9 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
   };
   if (residual(1.f, Q)) return true;
   implicit_solve_simt<N>(Z, Cm, dm, beta, mu, sums, ty, tx);
-  reduce_points<N>(
-      red,
-      [&](int o, Pair& s) {
+  reduce_points<N, Sum>(
+      red, ok,
+      [&](int o, Sum& s) {
         P[o] = Z[o];
         s.add_product(R[o], Z[o]);
       },
@@ -170,8 +173,8 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
   for (int it = 0; it < kPcgMaxIter; ++it) {
     apply_op<N>(P, Q, beta, dg);
     __syncthreads();
-    const float al = (float)reduce_points<N>(
-        red, [&](int o, Pair& s) { s.add_product(P[o], Q[o]); },
+    const float al = (float)reduce_points<N, Sum>(
+        red, ok, [&](int o, Sum& s) { s.add_product(P[o], Q[o]); },
         [&](double pq) { return rz / pq; });
     for (int i = tid; i < N * N; i += kSimtThreads) {
       const int o = (i / N) * NP + i % N;
@@ -179,8 +182,8 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
     }
     if (residual(al, Q)) return true;
     implicit_solve_simt<N>(Z, Cm, dm, beta, mu, sums, ty, tx);
-    const float be = (float)reduce_points<N>(
-        red, [&](int o, Pair& s) { s.add_product(R[o], Z[o]); },
+    const float be = (float)reduce_points<N, Sum>(
+        red, ok, [&](int o, Sum& s) { s.add_product(R[o], Z[o]); },
         [&](double x) {
           const double ratio = x / rz;
           rz = x;
@@ -195,10 +198,13 @@ __device__ bool pcg_solve(float* X, float* R, float* Z, float* P, float* Q, cons
   return false;
 }
 
-template <int N, bool PICARD>
-__device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const double th[kNPhys],
-                                float* sm, RedScratch* red, double* red64, float2* sums, double* phi_out,
-                                uint32_t* st_out, float* fields_out) {
+// Returns false, with nothing written, if a sum left the range of Sum.
+template <int N, bool PICARD, class Sum>
+__device__ __forceinline__ bool solve2d_cg_item(const DevProblem& pb, const DevSize& S,
+                                                const double th[kNPhys], float* sm,
+                                                RedScratch* red, double* red64, float2* sums,
+                                                double* phi_out, uint32_t* st_out,
+                                                float* fields_out) {
   constexpr int NP = simt_stride(N), NPTS = N * N, VS = N * NP;
   float* U = sm;
   float* V = sm + VS;
@@ -223,7 +229,7 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
   const int nfo = (S.field_mask & 1) + ((S.field_mask >> 1) & 1);
   double phi = 0.0;
   int bad = 0;
-  bool conv = true;
+  bool conv = true, ok = true;  // ok: warp 0's
   int next_obs = 0;
   __syncthreads();
   for (int step = 0; step < pb.n_steps; ++step) {
@@ -244,9 +250,9 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
         bb = x;
         return 0.0;
       };
-      reduce_points<N>(
-          red,
-          [&](int o, Pair& s) {
+      reduce_points<N, Sum>(
+          red, ok,
+          [&](int o, Sum& s) {
             const float du = U[o], dv = V[o];
             const float uu = ref_u + du, vv = ref_v + dv;
             const float u2v = uu * uu * vv;
@@ -256,17 +262,18 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
             s.add_product(rhs_u, rhs_u);
           },
           keep);
-      conv &= cg_solve<N>(U, R, P, Q, bu, dga, bb, red);
+      conv &= cg_solve<N, Sum>(U, R, P, Q, bu, dga, bb, red, ok);
       apply_op<N>(V, Q, bv, dga);
       __syncthreads();
-      reduce_points<N>(
-          red,
-          [&](int o, Pair& s) {
+      reduce_points<N, Sum>(
+          red, ok,
+          [&](int o, Sum& s) {
             R[o] = W[o] - Q[o];
             s.add_product(W[o], W[o]);
           },
           keep);
-      conv &= cg_solve<N>(V, R, P, Q, bv, dga, bb, red);
+      conv &= cg_solve<N, Sum>(V, R, P, Q, bv, dga, bb, red, ok);
+      if (__syncthreads_or(!ok)) return false;
     } else {
       // Picard: diagonals from u^n, v^n; mean diagonal for the preconditioner
       auto dg_u = [=](int o) {
@@ -276,29 +283,29 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
         const float uu = ref_u + U[o];
         return alpha + ftg * uu * uu;
       };
-      const float mu_u = (float)reduce_points<N>(
-          red,
-          [&](int o, Pair& s) {
+      const float mu_u = (float)reduce_points<N, Sum>(
+          red, ok,
+          [&](int o, Sum& s) {
             const float du = dg_u(o);
             s.add(du);
             R[o] = U[o] + ftg * fa + ref_u * (1.f - du);
           },
           [](double x) { return x / NPTS; });
-      const float mu_v = (float)reduce_points<N>(
-          red, [&](int o, Pair& s) { s.add(dg_v(o)); }, [](double x) { return x / NPTS; });
-      conv &= pcg_solve<N>(W, R, Z, P, Q, Cm, bu, mu_u, dg_u, S.mu, sums, red);
+      const float mu_v = (float)reduce_points<N, Sum>(
+          red, ok, [&](int o, Sum& s) { s.add(dg_v(o)); }, [](double x) { return x / NPTS; });
+      conv &= pcg_solve<N, Sum>(W, R, Z, P, Q, Cm, bu, mu_u, dg_u, S.mu, sums, red, ok);
       for (int i = tid; i < NPTS; i += kSimtThreads) {
         const int o = (i / N) * NP + i % N;
         R[o] = V[o] + ftg * fb + ref_v * (1.f - dg_v(o));
       }
       __syncthreads();
       // v^{n+1} into V: its diagonal needs only u^n, which U still holds
-      conv &= pcg_solve<N>(V, R, Z, P, Q, Cm, bv, mu_v, dg_v, S.mu, sums, red);
+      conv &= pcg_solve<N, Sum>(V, R, Z, P, Q, Cm, bv, mu_v, dg_v, S.mu, sums, red, ok);
       for (int i = tid; i < NPTS; i += kSimtThreads) {
         const int o = (i / N) * NP + i % N;
         U[o] = W[o];
       }
-      __syncthreads();
+      if (__syncthreads_or(!ok)) return false;
     }
     if (next_obs < S.n_obs && step + 1 == S.obs_steps[next_obs]) {
       const float* yo = S.yf + (size_t)next_obs * nfo * NPTS;
@@ -336,17 +343,30 @@ __device__ void solve2d_cg_item(const DevProblem& pb, const DevSize& S, const do
     }
   }
   __syncthreads();
+  return true;
 }
 
-#define RD_CG_CASE(NN)                                                              \
-  case NN:                                                                          \
-    if constexpr (NN <= NMAX)                                                       \
-      solve2d_cg_item<NN, PICARD>(pb, S, th, sm, &red, red64, sums, &phi[b], &status[b], \
-                                  fo);                                             \
+template <int N, bool PICARD>
+__device__ __noinline__ void solve2d_cg_wide(const DevProblem& pb, const DevSize& S,
+                                             const double th[kNPhys], float* sm, RedScratch* red,
+                                             double* red64, float2* sums, double* phi_out,
+                                             uint32_t* st_out, float* fields_out) {
+  solve2d_cg_item<N, PICARD, Sum64>(pb, S, th, sm, red, red64, sums, phi_out, st_out, fields_out);
+}
+
+#define RD_CG_CASE(NN)                                                                      \
+  case NN:                                                                                  \
+    if constexpr (NN <= NMAX)                                                               \
+      if (!solve2d_cg_item<NN, PICARD, Pair>(pb, S, th, sm, &red, red64, sums, &phi[b],     \
+                                             &status[b], fo))                               \
+        solve2d_cg_wide<NN, PICARD>(pb, S, th, sm, &red, red64, sums, &phi[b], &status[b], \
+                                    fo);                                                    \
     break;
 
+// Two CTAs an SM where shared memory holds them (the FP64 repetition would take more
+// registers than that leaves).
 template <int NMAX, bool PICARD>
-__global__ void __launch_bounds__(kSimtThreads, 1)
+__global__ void __launch_bounds__(kSimtThreads, NMAX <= (PICARD ? 32 : 64) ? 2 : 1)
     k_solve2d_cg(DevProblem pb, WorkQueue q, const double* theta, double* phi,
                  uint32_t* status, float* fields, size_t field_stride) {
   extern __shared__ __align__(16) float sm[];
