@@ -67,8 +67,13 @@ enum {
 
 /* Implicit-diffusion solver of the IMEX step. */
 enum {
-  RD_SOLVER_AUTO = 0,      /* autotuned per grid size (2-D), Thomas (1-D) */
-  RD_SOLVER_THOMAS = 1,    /* 1-D tridiagonal (FP64) */
+  RD_SOLVER_AUTO = 0,      /* autotuned per grid size (2-D); 1-D: the tridiagonal solve
+                              (FP64) whose arrangement suits the size of the batch.
+                              IMEX results of two arrangements agree to rounding, not
+                              to the bit, so they depend on the batch in the last bits */
+  RD_SOLVER_THOMAS = 1,    /* 1-D tridiagonal (FP64), one thread per proposal in the IMEX
+                              step: the same bits in every batch, slower for batches of
+                              a few thousand and fewer */
   RD_SOLVER_DCT_SIMT = 2,  /* 2-D eigenbasis solve, FP32 CUDA-core GEMMs */
   RD_SOLVER_DCT_TC = 3     /* 2-D eigenbasis solve of one direction by split-FP16
                               tcgen05 GEMMs, tridiagonal solves of the other */
@@ -184,7 +189,8 @@ rd_status rd_set_observations(rd_problem* p, int size_idx, int n_times,
  * status:   device, [B] RD_P_* bits
  * fields:   device or NULL, [B][2][maxN^dim] final u, v (float for F32
  *           problems, double for F64), each proposal at stride 2*maxN^dim
- *           with its own N^dim values first. */
+ *           with its own N^dim values first.
+ * 1-D results with RD_SOLVER_AUTO depend on the batch in the last bits (see there). */
 rd_status rd_evaluate_batch(rd_problem* p, int B, const double* theta,
                             const int* size_idx, double* loglik,
                             uint32_t* status, void* fields);
@@ -326,7 +332,10 @@ rd_status rd_chains_set_proposal(rd_chains* c, const double* L);
  * Chains split over several objects -- one per GPU, each taking a contiguous
  * range of a run's chains with first = the range's start and the same seed --
  * then draw exactly the numbers the chains of one object of the total size
- * would (Sec. 2.1: many independent chains, pooled afterwards).  Set it
+ * would (Sec. 2.1: many independent chains, pooled afterwards); in 1-D their samples
+ * are the same to the bit with RD_SOLVER_THOMAS or RD_SCHEME_PICARD, and with
+ * RD_SOLVER_AUTO while all objects are on the same side of the line between its
+ * arrangements (about 9000 chains of 64 nodes).  Set it
  * before the first rd_chains_run; it is not part of a checkpoint.  EINVAL if
  * first + n_chains exceeds 2^32. */
 rd_status rd_chains_set_first_chain(rd_chains* c, uint32_t first);

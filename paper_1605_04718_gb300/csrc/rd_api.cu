@@ -236,6 +236,7 @@ rd_status rd_problem_create(const rd_problem_desc* desc, void* cuda_stream,
   dv.precision = desc->precision;
   dv.growth = desc->growth;
   dv.n_params = desc->n_params;
+  dv.thomas = desc->solver == RD_SOLVER_THOMAS;
   dv.tau = desc->tau;
   dv.w_max = p->desc.w_max;
   dv.wait_ns = 4000000000ull;

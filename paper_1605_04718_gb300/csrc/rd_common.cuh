@@ -42,6 +42,7 @@ struct DevProblem {
   int growth;
   int n_params;
   int max_n;
+  int thomas;  // 1-D IMEX step: a thread per proposal whatever the batch (RD_SOLVER_THOMAS)
   double tau;
   double w_max;
   unsigned long long wait_ns;  // limit of the solve kernels' bounded waits

@@ -19,7 +19,9 @@
 //    divisions for c' and d' of a node, and the coefficients of all nodes.
 //    256 proposals of 100 nodes: 227 -> 60 us a step.
 // The kernel reads the number of queued proposals and takes the path whose
-// instructions per SM quarter are fewer (warps_worth).
+// instructions per SM quarter are fewer (lanes_for).  The IMEX paths agree to rounding
+// only, so RD_SOLVER_THOMAS, whose results do not depend on the batch, always gives a
+// proposal one thread.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -636,7 +638,7 @@ __global__ void __launch_bounds__(128)
   extern __shared__ __align__(16) double sm1d[];
   const bool picard = pb.scheme == RD_SCHEME_PICARD;
   int P = lanes_for(pb.max_n, picard, queued(q), 4 * n_sm);
-  if (picard && pb.ss_tol > 0.0) P = 1;
+  if (picard ? pb.ss_tol > 0.0 : pb.thomas != 0) P = 1;
   if (P > 1 && P < p_min) P = p_min;
   if (P > 1) {
     // one warp per SM quarter: more would share its FP64 pipe
