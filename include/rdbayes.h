@@ -449,10 +449,10 @@ rd_status rd_chains_set_surrogate(rd_chains* c, rd_surrogate* s);
  * RD_P_NOT_SOLVED and Phi = +inf. */
 rd_status rd_sync(rd_problem* p);
 
-/* Limit of every bounded wait inside the tensor-core solve kernels (default
- * 4 s; (0, 60] seconds).  A healthy wait lasts microseconds; a wait that runs
- * out makes the kernel's CTA stop popping work, drain the MMAs it issued,
- * free its tensor memory and raise the problem's error flag, which rd_sync and
+/* Limit of every bounded wait inside the tensor-core kernels, the solves' and the
+ * surrogate's (default 4 s; (0, 60] seconds).  A healthy wait lasts microseconds;
+ * a wait that runs out makes the kernel's CTA stop popping work, drain the MMAs it
+ * issued, free its tensor memory and raise the problem's error flag, which rd_sync and
  * rd_evaluate_batch_host report as RD_ETIMEOUT.  The context stays usable.
  * Takes effect at the next launch (captured chain steps are re-captured). */
 rd_status rd_set_wait_limit(rd_problem* p, double seconds);
@@ -464,7 +464,9 @@ rd_status rd_set_wait_limit(rd_problem* p, double seconds);
  * every other wait of the CTA, runs out after the wait limit, so the launch
  * ends in bounded time with RD_ETIMEOUT and every proposal of the batch left
  * RD_P_NOT_SOLVED.  step = -1 (the default) turns it off.  CUDA-core kernels
- * have no waits and ignore it. */
+ * have no waits and ignore it.  RD_STALL_SURROGATE instead lets the surrogate's
+ * kernels wait for products whose completion is never signalled. */
+#define RD_STALL_SURROGATE 0x7fffffff
 rd_status rd_debug_stall_at_step(rd_problem* p, int step);
 
 /* Message of the last failed call on this thread ("" if none). */

@@ -122,12 +122,14 @@ struct MlpArgs {
   float* Z1;                                 // [W][B]
   float* part4;             // [tile][W + 1]: shares of dW4, db4
   int* err;
+  unsigned long long wait_ns;  // limit of the bounded waits
+  int stall;                // failure-path test aid: layer 1's MMAs are never committed
 };
 
 enum { MLP_PREDICT = 0, MLP_LOSS = 1, MLP_GRAD = 2 };
 
 struct MlpCtrl {
-  uint64_t bar;
+  uint64_t bar, fin;
   uint32_t tmem_base;
   int abort;
   float w4[kW];
@@ -140,6 +142,15 @@ constexpr uint32_t act_bytes(int nr) { return (uint32_t)(nr > 64 ? 2 : 1) * kW *
 constexpr uint32_t mlp_smem_bytes(int nr) {
   // at least 150 KB, so that no other CTA with a TMEM allocation shares the SM
   return 1024 + kMlpTileW + act_bytes(nr) + (uint32_t)sizeof(MlpCtrl);
+}
+
+// After a wait that gave up: waits (again bounded) until every MMA that thread 0
+// issued has finished, so that no tensor memory is freed under one.  By warp 0.
+__device__ __forceinline__ void drain(uint64_t* fin) {
+  if (threadIdx.x == 0) mma_commit(fin);
+  __syncwarp();
+  volatile int never = 0;
+  mbar_wait_bounded(fin, 0, &never);
 }
 
 // One layer, D[unit][row] for both halves of the units: A = the weights' tile
@@ -243,6 +254,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   }
   if (tid == 0) {
     mbar_init(&ctl->bar, 1);
+    mbar_init(&ctl->fin, 1);
     ctl->abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -257,9 +269,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   const uint32_t sa = smem_u32(ta), sw = smem_u32(tw);
   uint32_t phase = 0;
   // waits for the MMAs issued since the last wait (a wait that gives up leaves
-  // wrong values and raises the error flag at the end)
+  // wrong values and raises the error flag at the end; later ones give up at once)
   auto done = [&]() {
-    mbar_wait_bounded(&ctl->bar, phase & 1u, &ctl->abort);
+    mbar_wait_bounded(&ctl->bar, phase & 1u, &ctl->abort, a.wait_ns);
     ++phase;
     tc_fence_after();
   };
@@ -289,7 +301,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   // ---- layer 1 -> d0
   if (tid == 0) {
     issue_layer<1, NR, 0, 0>(d0, smem_u32(tw1), sa);
-    mma_commit(&ctl->bar);
+    if (!a.stall) mma_commit(&ctl->bar);
   }
   __syncwarp();
   done();
@@ -424,6 +436,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const __grid_constant__ 
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
+    if (ctl->abort) drain(&ctl->fin);
     tc_fence_after();
     tmem_dealloc(tmem, 4 * NR);
   }
@@ -440,6 +453,8 @@ struct WgradArgs {
   const __nv_bfloat16* H[3];   // [0]: the features [B][16]; else [W][B]
   float* part;  // [splits][stride()]
   int* err;
+  unsigned long long wait_ns;
+  int stall;
 };
 constexpr uint32_t kWgTileA = 128 * 128 * 2, kWgTileB = 128 * kW * 2;
 constexpr uint32_t kWgSmem = 1024 + 2 * (kWgTileA + kWgTileB) + 4 * 128 * 4;
@@ -448,7 +463,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   extern __shared__ uint8_t wg_smem[];
   uint8_t* const base = wg_smem + ((1024u - (smem_u32(wg_smem) & 1023u)) & 1023u);
   float* const sums = reinterpret_cast<float*>(base + 2 * (kWgTileA + kWgTileB));  // [4][128]
-  __shared__ uint64_t bar;
+  __shared__ uint64_t bar, fin;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   constexpr Layout L(kW);
@@ -465,6 +480,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   }
   if (tid == 0) {
     mbar_init(&bar, 1);
+    mbar_init(&fin, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -490,7 +506,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   for (int t = t0; t < t1; ++t) {
     uint8_t* s = base + (uint32_t)(t & 1) * (kWgTileA + kWgTileB);
     if (t > t0) {  // the other buffer's MMAs are done: it may be refilled
-      ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag) && ok;
+      ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag, a.wait_ns) && ok;
       ++phase;
       tc_fence_after();
     }
@@ -511,7 +527,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
             layer == 0 ? kk * 2048u : (uint32_t)(kk >> 2) * kW * 128u + (kk & 3) * 32u;
         mma_f16(tmem, ad + (oa >> 4), bd + (ob >> 4), idesc, (t > t0 || kk > 0) ? 1u : 0u);
       }
-      mma_commit(&bar);
+      if (!a.stall) mma_commit(&bar);
     }
     __syncwarp();
     if (t + 1 < t1) load(t + 1);
@@ -525,7 +541,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
             __ushort_as_bfloat16((unsigned short)(w[k >> 1] >> (16 * (k & 1)))));
     }
   }
-  ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag) && ok;
+  ok = mbar_wait_bounded(&bar, phase & 1u, &abort_flag, a.wait_ns) && ok;
   tc_fence_after();
   sums[tid] = colsum;
   __syncthreads();
@@ -551,6 +567,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_wgrad(const __grid_const
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
+    if (abort_flag) drain(&fin);
     tc_fence_after();
     tmem_dealloc(tmem, 256);
   }
@@ -751,6 +768,8 @@ static cudaError_t pass(rd_surrogate* s, int mode, int B, const double* theta, d
   a.Z1 = s->Z1;
   a.part4 = s->part4;
   a.err = s->pb->ws.err;
+  a.wait_ns = s->pb->dev.wait_ns;
+  a.stall = s->pb->dev.stall_step == RD_STALL_SURROGATE;
   const int n_sm = s->pb->n_sm;
   if (mode == MLP_PREDICT) return launch_mlp<MLP_PREDICT>(a, n_sm, st);
   if (mode == MLP_LOSS) return launch_mlp<MLP_LOSS>(a, n_sm, st);
@@ -777,6 +796,8 @@ static cudaError_t loss_grad(rd_surrogate* s, int B, const double* theta, const 
   g.H[2] = s->H2;
   g.part = s->part;
   g.err = s->pb->ws.err;
+  g.wait_ns = s->pb->dev.wait_ns;
+  g.stall = s->pb->dev.stall_step == RD_STALL_SURROGATE;
   if ((e = cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kWgSmem)) != cudaSuccess)
     return e;
