@@ -50,8 +50,8 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "4fc00d1f8fa694370bfd60a0e0af400faeca23a550e399df9725ee33f3ef293f",
-        "bytes": 957184 + 1379072,
+        "sha256": "1ae72c51553cb11ad0c971364c653f590645641de6502e84001e0d43b351e3f5",
+        "bytes": 1463552 + 1346304,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)

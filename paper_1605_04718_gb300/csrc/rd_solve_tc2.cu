@@ -1038,7 +1038,8 @@ __device__ __forceinline__ void solve_loop(const DevProblem& pb, const WorkQueue
     __syncthreads();
   }
   if (warp == kIssueWarp) {
-    if (lane == 0) mma_commit(&ctl->fin);
+    // by the lane that issued the MMAs: a commit covers its own thread's alone
+    if (elect_one()) mma_commit(&ctl->fin);
     __syncwarp();
     volatile int never = 0;
     mbar_wait_bounded(&ctl->fin, 0, &never);
