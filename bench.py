@@ -75,6 +75,12 @@ def traffic_of(kernel):
     return None
 
 
+def transform_flops(n, steps):
+    """Flops of one N x N solve's transforms: of one direction and back, 2 N^3 each for
+    both fields (every kernel that transforms solves the other direction by a scan)."""
+    return 8.0 * n**3 * steps
+
+
 def peaks():
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(path):
@@ -630,10 +636,7 @@ def run_gpu(args):
         pk, pk_src = peaks()
         value = solves_all / t_all
         kind = rd.rd_get_size_kernel(p, 0)
-        # transforms x 2 N^3 x 2 fields per step: the tensor-core kernel transforms one
-        # direction and back, the CUDA-core kernel both
-        n_tr = 4 if kind == rd.RD_KERNEL_SIMT else 2
-        flop_per_solve = n_tr * 4.0 * n**3 * spec["n_steps"]
+        flop_per_solve = transform_flops(n, spec["n_steps"])
         bytes_per_solve = 16.0 * n * n * spec["n_steps"]  # u, v FP32 read + write per step
         # the solve kernel's launch duration, taken from the timed steps: one
         # launch per step, 99.997 % of the step's device time (the ncu launch
@@ -658,7 +661,7 @@ def run_gpu(args):
                                        "other kernels of a step take 0.003 % of it)",
                      "standalone_ms": 1e3 * k_standalone, "standalone_reps": len(kt),
                      "standalone_ms_each": [1e3 * x for x in kt],
-                     "work": f"{4 * n_tr} N^3 flop per proposal-step ({n_tr} transforms x 2 N^3 x 2 fields) "
+                     "work": f"8 N^3 flop per proposal-step (2 transforms x 2 N^3 x 2 fields) "
                              f"x {spec['n_steps']} steps x {C} proposals per launch"})
         hbm = _find(pk, "hbm_gbs", "hbm_GBps", "copy_gbs") or FALLBACK_PEAKS["hbm_gbs"]
         roof["hbm_equiv"] = {"gbs": bytes_per_solve * C / k_dur / 1e9, "peak_gbs": hbm,
