@@ -50,8 +50,8 @@ KERNELS = {"simt": 1, "stacked": 2, "resident": 3}
 # one the capture ran on, else null.
 TRAFFIC = {
     "k_solve2d_tc128<2>": {
-        "sha256": "1ae72c51553cb11ad0c971364c653f590645641de6502e84001e0d43b351e3f5",
-        "bytes": 1463552 + 1346304,
+        "sha256": "3fba1054617e921b7754b783eacec8bce6436a3cd362fa46d5fa22aa0f56c3b5",
+        "bytes": 1210112 + 1420288,
     },
 }
 TRAFFIC_SOURCES = {  # the kernel's own code (its loads and stores)

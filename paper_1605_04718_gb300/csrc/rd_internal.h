@@ -117,7 +117,7 @@ int grid_solve_tc(int n_sm);
 cudaError_t launch_solve_tc(const DevProblem& pb, const WorkQueue& q, const double* theta,
                             double* phi, uint32_t* status, void* fields, int grid, int* err,
                             cudaStream_t st, bool after_tc);
-// CUDA-core conjugate-gradient solves (rd_solve_simt.cu): the IMEX step by
+// CUDA-core conjugate-gradient solves (rd_solve_cg.cu): the IMEX step by
 // plain CG (RD_KERNEL_CG, N <= 96) or the paper's semi-implicit step by
 // preconditioned CG (picard, N <= 80).
 bool cg_applicable(int n, bool picard);

@@ -726,9 +726,10 @@ static cudaError_t launch_mlp(const MlpArgs& a, cudaStream_t st) {
 }
 
 // Rows per tile: 32 while that fills the SMs at most twice, each tile reading all
-// weights anew (forward: 4096 rows 23 us against 37 with 128-row tiles, 9728
-// rows 35 against 39, 14592 rows 47 against 41); the backward pass, whose tiles
-// do three times as much, once and a half (8192 rows 124 us both ways).
+// weights anew (forward, calls back to back: 4096 rows 16 us against 34 with 128-row
+// tiles, 9728 rows 28 against 34, 12160 rows 40 against 34); the backward pass, whose
+// tiles do three times as much, once and a half (loss and gradients: 4864 rows 77 us
+// against 112, 8192 rows 111 us both ways, 14592 rows 158 against 124).
 static int tile_rows(int mode, int B, int n_sm) {
   const int waves2 = mode == MLP_GRAD ? 3 : 4;  // twice the waves
   return B <= waves2 * 16 * n_sm ? 32 : 128;

@@ -17,7 +17,8 @@
 //  * semi-implicit: the elimination is serial and its result reproducible to
 //    the bit, so only what is independent moves to other lanes: u and v, the
 //    divisions for c' and d' of a node, and the coefficients of all nodes.
-//    256 proposals of 100 nodes: 227 -> 60 us a step.
+//    256 proposals of 100 nodes: 227 -> 60 us a step, up to 94 when blocks with work
+//    come to share an SM (nothing keeps two of the first n_sm blocks apart).
 // The kernel reads the number of queued proposals and takes the path whose
 // instructions per SM quarter are fewer (lanes_for).  The IMEX paths agree to rounding
 // only, so RD_SOLVER_THOMAS, whose results do not depend on the batch, always gives a
@@ -641,7 +642,7 @@ __global__ void __launch_bounds__(128)
   if (picard ? pb.ss_tol > 0.0 : pb.thomas != 0) P = 1;
   if (P > 1 && P < p_min) P = p_min;
   if (P > 1) {
-    // one warp per SM quarter: more would share its FP64 pipe
+    // at most one warp per SM quarter on average: more would share its FP64 pipe
     if ((int)blockIdx.x >= n_sm) return;
     double* sm = sm1d + (size_t)(threadIdx.x >> 5) * (32 / P) * 6 * pb.max_n;
     if (P == 8)

@@ -11,8 +11,8 @@
 // against four transforms when both directions are diagonalised: half the
 // tensor-core work, two conversions of the data per step instead of four, and
 // no 1 / (alpha + beta (mu_k + mu_l)) per point.  The scan is FP32 throughout.
-// Measured against the four-transform kernels (GB300): 128^2 9.98 -> 5.8 us a
-// step of one proposal per SM; 64^2 18.7 -> 4.9 us for the four proposals an SM
+// Measured against the four-transform kernels (GB300): 128^2 9.98 -> 5.5 us a
+// step of one proposal per SM; 64^2 18.7 -> 4.5 us for the four proposals an SM
 // holds; relative field error after 1000 steps at 128^2 2.2e-7 -> 1.8e-7.
 //
 // Layout.  A slab is one accumulator of 128 TMEM lanes x 128 columns; a CTA has
