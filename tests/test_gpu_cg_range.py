@@ -53,3 +53,20 @@ def test_scaled_fields_give_the_scaled_result(n, picard, scale):
     assert np.all(st0 == 0) and np.all(st1 == 0)
     for f in range(2):
         assert H.rel_l2(got[f], ref[f]) < 8e-6, f
+
+
+def test_a_diverging_proposal_is_not_taken_for_an_unconverged_solve():
+    """gamma 200 times too large: the fields pass 1e19 on their way out, where products of
+    their values overflow FP32 although every system is still solved; the status is
+    RD_P_NONFINITE alone, as the oracle's."""
+    ds = H.small_dataset(64, 100, seed=64)
+    p = H.gpu_problem([ds], solver=rd.RD_SOLVER_AUTO)
+    rd.rd_set_size_kernel(p, 0, rd.RD_KERNEL_CG)
+    theta = np.tile([0.1, 0.9, 10.0, 200.0], (9, 1))
+    theta[::3, 3] = 4e4
+    phi, st = rd.rd_evaluate_batch_host(p, theta)
+    rd.rd_problem_destroy(p)
+    P = H.oracle_problem(ds)
+    for i in range(9):
+        assert st[i] == P.forward(list(theta[i]) + [0.0])[1]
+    assert np.array_equal(np.isinf(phi), theta[:, 3] > 1e3)
