@@ -32,6 +32,7 @@ RD_MAX_SIZES, RD_MAX_OBS, RD_NPARAM, RD_NPHYS = 4, 8, 5, 8
 RD_GROWTH_NONE, RD_GROWTH_EXP, RD_GROWTH_POLY4 = 0, 1, 2
 RD_NOALLOC_MAX_BATCH = 65536
 RD_PMH_MAX_PROPOSALS = 16
+RD_STALL_SURROGATE = 0x7FFFFFFF  # rd_debug_stall_at_step: the surrogate's kernels
 RD_SURROGATE_WIDTH = 256
 SURROGATE_IN = 16  # padded network inputs
 

@@ -15,7 +15,6 @@ pytestmark = pytest.mark.gpu
 
 DEV = torch.device("cuda:0") if torch.cuda.is_available() else None
 TRUE4 = [0.1, 0.9, 10.0, 200.0]
-RD_STALL_SURROGATE = 0x7FFFFFFF
 
 
 @pytest.mark.parametrize("rows", [256, 20096])  # tiles of 32 and of 128 rows
@@ -45,7 +44,7 @@ def test_bounded_wait_gives_up_and_the_surrogate_recovers(rows):
     before = predict(), grads()
     rd.rd_sync(p)
     rd.rd_set_wait_limit(p, 0.05)
-    rd.rd_debug_stall_at_step(p, RD_STALL_SURROGATE)
+    rd.rd_debug_stall_at_step(p, rd.RD_STALL_SURROGATE)
     for call in (predict, grads):
         t0 = time.perf_counter()
         call()
